@@ -113,11 +113,24 @@ class Graph:
 
 def compute(n: int, src, dst, w):
     """Minimum spanning forest of one graph: (edge_mask, labels, total)."""
-    g = Graph(n, src, dst, w)
-    try:
-        return g.compute()
-    finally:
-        g.free()
+    return _one(int(n), src, dst, w)
+
+
+def _one(n: int, src, dst, w, labels: bool = True):
+    """One graph as a batch of one: the library keeps no handle, so it needs
+    no CSR (msf_compute_batched)."""
+    _check_i32(dst, "dst")
+    _check_i32(src, "src")
+    m = int(dst.shape[0])
+    wtype = _wtype(w)
+    mk = _out(dst, (m,), torch.uint8, np.uint8)
+    lb = _out(dst, (n,), torch.int32, np.int32) if labels else None
+    tt = _out(dst, (1,), torch.float64, np.float64)
+    off = np.array([0, n, 0, m], np.int64)  # voff, then eoff
+    dev = dst.device if isinstance(dst, torch.Tensor) else None
+    _abi.msf_compute_batched(1, off.ctypes.data, off.ctypes.data + 16, _ptr(src), _ptr(dst), _ptr(w), wtype,
+                             _ptr(mk), _ptr(lb), _ptr(tt), _stream_handle(dev))
+    return mk, lb, tt
 
 
 def compute_batched(voff, eoff, src, dst, w):
@@ -159,11 +172,7 @@ class MSFWeight(torch.autograd.Function):
             raise TypeError("MSFWeight needs float32 weights")
         G = len(batch.voff) - 1
         if G == 1:
-            g = Graph(int(batch.voff[-1]), batch.src, batch.dst, w)
-            try:
-                mask, _, totals = g.compute(labels=False)
-            finally:
-                g.free()
+            mask, _, totals = _one(int(batch.voff[-1]), batch.src, batch.dst, w, labels=False)
         else:
             mask, _, totals = compute_batched(batch.voff, batch.eoff, batch.src, batch.dst, w)
         ctx.save_for_backward(mask)

@@ -383,6 +383,33 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
   return MSF_OK;
 }
 
+// The one-shot solver gives the forest alone: a caller that asked for a
+// schedule, a builder, a kernel form or tighter limits than the defaults gets
+// the round loop over a CSR, whose steps those options are about.
+bool one_shot_allowed() {
+  const Options &o = options();
+  return o.exec_mode == 0 && o.shortcut_mode == MSF_SHORTCUT_CSP && !o.pairwise && o.build_mode == 0 &&
+         o.sweep == 0 && o.round_limit >= 64 && o.jump_limit >= 64;
+}
+
+int one_shot(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const void *w, int wtype,
+             uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
+  int rc;
+  Staged ss, sd, sw, om, ol, ot;
+  if ((rc = ss.input(src, (size_t)m * 4, s)) || (rc = sd.input(dst, (size_t)m * 4, s)) ||
+      (rc = sw.input(w, (size_t)m * 4, s)) || (rc = om.output(edge_mask, (size_t)m)) ||
+      (rc = ol.output(labels, (size_t)n * 4)) || (rc = ot.output(totals, 8))) {
+    cudaStreamSynchronize(s);  // copies already queued finish before their buffers return to the pool
+    return rc;
+  }
+  rc = solve_edges(n, m, (const int32_t *)ss.dev, (const int32_t *)sd.dev, (const uint32_t *)sw.dev, wtype,
+                   (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
+  if (rc) return rc;
+  if ((rc = om.copy_back(s)) || (rc = ol.copy_back(s)) || (rc = ot.copy_back(s))) return rc;
+  if (om.owned || ol.owned || ot.owned) MSF_CK(cudaStreamSynchronize(s));
+  return MSF_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -425,7 +452,12 @@ int msf_compute_batched(int32_t G, const int64_t *voff, const int64_t *eoff, con
   const int64_t n = voff[G], m = eoff[G];
   if (n > MAX_N || m > MAX_M) return fail(MSF_ERR_TOO_LARGE, "total n must be < 2^31 and total m < 2^32 - 1");
   if (m > 0 && (!src || !dst || !w)) return fail(MSF_ERR_INVALID_ARG, "NULL edge array");
+  if (m > 0 && n == 0) return fail(MSF_ERR_INVALID_ARG, "edges given for an empty vertex set");
   cudaStream_t s = (cudaStream_t)stream;
+  if (G == 1 && one_shot_allowed()) {
+    const int rc = one_shot(n, m, src, dst, w, wtype, edge_mask, labels, totals, s);
+    if (rc != SOLVE_NOT_RUN) return rc;
+  }
   msf_graph *g = nullptr;
   int rc = build_graph_common(n, m, src, dst, nullptr, w, wtype, G, voff, eoff, s, &g);
   if (rc) return rc;

@@ -278,6 +278,14 @@ void launch_backward(int64_t m, int32_t G, const int64_t *eoff_d, const uint8_t 
                      const double *gt, float *gw, cudaStream_t s);
 void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cudaStream_t s);
 
+// solve.cu
+// Forest of one graph from its edge list, without a CSR (pointers the device
+// can read; any output may be NULL).  Synchronizes `s`.  SOLVE_NOT_RUN: the
+// device cannot hold the kernel's blocks at once; the outputs are untouched.
+constexpr int SOLVE_NOT_RUN = -1;
+int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const uint32_t *w, int wtype,
+                uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s);
+
 // exec.cu
 int enqueue_msf_graph(const DevState &hs, cudaStream_t s, const DevState **host_state);
 int enqueue_cc_graph(const DevState &hs, cudaStream_t s, const DevState **host_state);

@@ -16,6 +16,7 @@
 #include <mutex>
 #include <string>
 
+#include "exact.cuh"
 #include "internal.cuh"
 
 namespace msf {
@@ -613,28 +614,6 @@ __global__ void __launch_bounds__(BT) k_label_write(DevState *st) {
 }
 
 // ---- exact forest weight ---------------------------------------------------
-// float32: bins[b] accumulates the signed 24-bit significands of the weights
-// whose (denormal-adjusted) biased exponent is b, so weight = sig * 2^(b-150);
-// bin 0 counts +inf and bin 255 counts -inf.  uint32: bin 0 is the sum.
-__device__ __forceinline__ void weight_bin(uint32_t ordw, int wtype, int *bin, long long *val) {
-  if (wtype == MSF_U32) {
-    *bin = 0;
-    *val = (long long)ordw;
-    return;
-  }
-  const uint32_t bits = (ordw & 0x80000000u) ? (ordw & 0x7fffffffu) : ~ordw;
-  const uint32_t E = (bits >> 23) & 0xffu, M = bits & 0x7fffffu;
-  const bool neg = bits >> 31;
-  if (E == 255u) {
-    *bin = neg ? 255 : 0;
-    *val = 1;
-    return;
-  }
-  const long long sig = E ? (long long)(M | 0x800000u) : (long long)M;
-  *bin = E ? (int)E : 1;
-  *val = neg ? -sig : sig;
-}
-
 // The edge mask from the forest's keys, once after the loop.  With the
 // bitmap (a full compute): one bit per forest edge (the bitmap, m / 8
 // bytes, stays mostly in L2), then k_mask_expand writes every mask byte in
@@ -663,21 +642,6 @@ __global__ void __launch_bounds__(BT) k_mask_from_keys(DevState *st) {
   }
 }
 
-// 16 mask bytes from 16 bits: byte j = bit j (each nibble spread to the low
-// bits of four bytes by one multiplication: its copies at shifts 0, 7, 14
-// and 21 do not overlap, and bit j of the nibble lands on bit 8j).
-__device__ __forceinline__ uint4 spread16(uint32_t v) {
-  constexpr uint32_t MUL = 0x00204081u, LOW = 0x01010101u;
-  return make_uint4(((v & 0xfu) * MUL) & LOW, (((v >> 4) & 0xfu) * MUL) & LOW, (((v >> 8) & 0xfu) * MUL) & LOW,
-                    (((v >> 12) & 0xfu) * MUL) & LOW);
-}
-// bits [e, e + 16) of the bitmap (the bitmap has a zero word past the end)
-__device__ __forceinline__ uint32_t bits16(const uint32_t *bits, int64_t e) {
-  const int64_t i = e >> 5;
-  const uint32_t o = (uint32_t)(e & 31);
-  const uint64_t w = (uint64_t)bits[i] | ((uint64_t)bits[i + 1] << 32);
-  return (uint32_t)(w >> o) & 0xffffu;
-}
 // The mask from the bitmap: 16-byte stores between the unaligned head and
 // tail of the caller's byte array, every byte written.
 __global__ void __launch_bounds__(BT) k_mask_expand(DevState *st) {
@@ -774,211 +738,6 @@ __global__ void __launch_bounds__(BT) k_sum(DevState *st) {
     const int32_t g = graph_of(st->eoff, G, (int64_t)(uint32_t)key);
     atomicAdd(reinterpret_cast<unsigned long long *>(st->bins) + (int64_t)g * 256 + bin, (unsigned long long)val);
   }
-}
-
-// Unsigned big integer of 6 64-bit limbs.
-struct Big {
-  unsigned long long w[6];
-};
-
-__device__ __forceinline__ void big_add_shifted(Big &a, unsigned long long v, int sh) {
-  // limbs below li get 0 with no carry; fixed trip counts keep the limbs in
-  // registers
-  const int li = sh >> 6, bo = sh & 63;
-  const unsigned long long lo = v << bo;
-  const unsigned long long hi = bo ? (v >> (64 - bo)) : 0ull;
-  unsigned long long c = 0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const unsigned long long add = (i == li) ? lo : (i == li + 1 ? hi : 0ull);
-    const unsigned long long s1 = a.w[i] + add;
-    const unsigned long long c1 = s1 < add;
-    const unsigned long long s2 = s1 + c;
-    const unsigned long long c2 = s2 < c;
-    a.w[i] = s2;
-    c = c1 | c2;
-  }
-}
-
-__device__ __forceinline__ int big_cmp(const Big &a, const Big &b) {
-  for (int i = 5; i >= 0; --i) {
-    if (a.w[i] != b.w[i]) return a.w[i] < b.w[i] ? -1 : 1;
-  }
-  return 0;
-}
-
-__device__ __forceinline__ void big_sub(Big &a, const Big &b) {  // a -= b, a >= b
-  unsigned long long br = 0;
-  for (int i = 0; i < 6; ++i) {
-    const unsigned long long d1 = a.w[i] - b.w[i];
-    const unsigned long long b1 = a.w[i] < b.w[i];
-    const unsigned long long d2 = d1 - br;
-    const unsigned long long b2 = d1 < br;
-    a.w[i] = d2;
-    br = b1 | b2;
-  }
-}
-
-
-// Shifts that give 0 for shift counts of 64 or more.
-__device__ __forceinline__ unsigned long long shl64(unsigned long long x, int s) { return s >= 64 ? 0ull : x << s; }
-__device__ __forceinline__ unsigned long long shr64(unsigned long long x, int s) { return s >= 64 ? 0ull : x >> s; }
-
-// Bits [lo, lo + 63] of a (lo >= 0).  Every limb is shifted into place (no
-// limb is selected by a computed index, which would move a to local memory).
-__device__ __forceinline__ unsigned long long big_window(const Big &a, int lo) {
-  unsigned long long w = 0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const int d = i * 64 - lo;
-    w |= d >= 0 ? shl64(a.w[i], d) : shr64(a.w[i], -d);
-  }
-  return w;
-}
-
-// Whether any bit below position `lo` is set.
-__device__ __forceinline__ bool big_any_below(const Big &a, int lo) {
-  bool any = false;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const int k = lo - i * 64;  // bits of limb i below lo
-    const unsigned long long mk = k >= 64 ? ~0ull : (k <= 0 ? 0ull : (1ull << k) - 1ull);
-    any = any || (a.w[i] & mk) != 0;
-  }
-  return any;
-}
-
-// Nearest double (ties to even) of (-1)^neg * a * 2^-149.
-__device__ __forceinline__ double big_to_double(const Big &a, bool neg) {
-  int h = -1;
-#pragma unroll
-  for (int i = 5; i >= 0; --i)
-    if (h < 0 && a.w[i]) h = i * 64 + 63 - __clzll((long long)a.w[i]);
-  if (h < 0) return 0.0;
-  unsigned long long mant;
-  int e2;  // value = mant * 2^e2
-  if (h <= 52) {
-    mant = a.w[0];
-    e2 = -149;
-  } else {
-    // the 64 bits ending at h: top 53 are the significand, then the round
-    // bit, then 10 bits that join the sticky bits below the window
-    unsigned long long w;
-    bool sticky;
-    if (h >= 63) {
-      w = big_window(a, h - 63);
-      sticky = big_any_below(a, h - 63);
-    } else {
-      w = a.w[0] << (63 - h);
-      sticky = false;
-    }
-    mant = w >> 11;
-    const unsigned long long rb = (w >> 10) & 1ull;
-    sticky = sticky || (w & 0x3ffull);
-    e2 = h - 52 - 149;
-    if (rb && (sticky || (mant & 1ull))) {
-      mant += 1;
-      if (mant == (1ull << 53)) {
-        mant >>= 1;
-        e2 += 1;
-      }
-    }
-  }
-  // normalize into [2^52, 2^53)
-  while (mant < (1ull << 52)) {
-    mant <<= 1;
-    e2 -= 1;
-  }
-  const unsigned long long biased = (unsigned long long)(e2 + 52 + 1023);
-  const unsigned long long bits = ((unsigned long long)neg << 63) | (biased << 52) | (mant & ((1ull << 52) - 1));
-  return __longlong_as_double((long long)bits);
-}
-
-// a += b (six limbs; the sums of the accumulators stay far below 2^384)
-__device__ __forceinline__ void big_add(Big &a, const Big &b) {
-  unsigned long long c = 0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const unsigned long long s1 = a.w[i] + b.w[i];
-    const unsigned long long c1 = s1 < b.w[i];
-    const unsigned long long s2 = s1 + c;
-    const unsigned long long c2 = s2 < c;
-    a.w[i] = s2;
-    c = c1 | c2;
-  }
-}
-
-// Nearest double of (P - N) * 2^-149: |P - N| and its sign, one rounding;
-// per-limb selects keep the limbs in registers.
-__device__ __forceinline__ double round_difference(const Big &P, const Big &N) {
-  const bool ge = big_cmp(P, N) >= 0;
-  Big D, E;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    D.w[i] = ge ? P.w[i] : N.w[i];
-    E.w[i] = ge ? N.w[i] : P.w[i];
-  }
-  big_sub(D, E);
-  return big_to_double(D, !ge);
-}
-
-// Exact total of one graph from its long accumulators (bin 0: +inf count
-// or, for u32 weights, the plain sum; bin 255: -inf count; bins 1..254:
-// signed multiples of 2^(e-1)), rounded once to nearest even.
-__device__ double combine_bins(const long long *b, int wtype) {
-  if (wtype == MSF_U32) return __ull2double_rn((unsigned long long)b[0]);
-  const bool pinf = b[0] > 0, ninf = b[255] > 0;
-  if (pinf || ninf) {
-    const unsigned long long bits = (pinf && ninf) ? 0x7ff8000000000000ull
-                                    : (pinf ? 0x7ff0000000000000ull : 0xfff0000000000000ull);
-    return __longlong_as_double((long long)bits);
-  }
-  Big P, N;
-  for (int i = 0; i < 6; ++i) P.w[i] = N.w[i] = 0;
-  for (int e = 1; e < 255; ++e) {
-    const long long v = b[e];
-    if (v > 0) big_add_shifted(P, (unsigned long long)v, e - 1);
-    else if (v < 0) big_add_shifted(N, (unsigned long long)(-v), e - 1);
-  }
-  return round_difference(P, N);
-}
-
-// The same by a whole warp (every lane calls it; lane 0 gets the result):
-// lane l adds bins 8l .. 8l+7 into its own pair of big integers, the pairs
-// are summed across the warp, lane 0 rounds the difference once.
-__device__ double combine_bins_warp(const long long *b, int wtype) {
-  if (wtype == MSF_U32) return __ull2double_rn((unsigned long long)b[0]);
-  const bool pinf = b[0] > 0, ninf = b[255] > 0;
-  if (pinf || ninf) {
-    const unsigned long long bits = (pinf && ninf) ? 0x7ff8000000000000ull
-                                    : (pinf ? 0x7ff0000000000000ull : 0xfff0000000000000ull);
-    return __longlong_as_double((long long)bits);
-  }
-  const int lane = threadIdx.x & 31;
-  Big P, N;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) P.w[i] = N.w[i] = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int e = 8 * lane + k;
-    const long long v = (e >= 1 && e <= 254) ? b[e] : 0;
-    if (v > 0) big_add_shifted(P, (unsigned long long)v, e - 1);
-    else if (v < 0) big_add_shifted(N, (unsigned long long)(-v), e - 1);
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    Big P2, N2;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      P2.w[i] = __shfl_down_sync(FULL, P.w[i], off);
-      N2.w[i] = __shfl_down_sync(FULL, N.w[i], off);
-    }
-    if (lane + off < 32) {
-      big_add(P, P2);
-      big_add(N, N2);
-    }
-  }
-  return round_difference(P, N);
 }
 
 // One warp per graph: the warp stages the graph's 256 long accumulators in

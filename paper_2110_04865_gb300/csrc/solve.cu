@@ -1,0 +1,1079 @@
+// One-shot forest of one edge list, without a CSR.
+//
+// A caller that hands over an edge list and keeps no handle needs no adjacency
+// structure: the strict order on (weight, edge index) makes the forest unique,
+// so any exact method returns the round loop's mask, labels and total.  The
+// CSR costs several passes over two records per edge and every round of the
+// loop sweeps all of them; here the edges are read once or twice:
+//
+//   select   one pass validates the edges and keeps the light ones, in two
+//            classes: about CLASS1 * n edges below a first threshold key, those
+//            up to CLASS2 * n below a second (keys of a sample; all edges when
+//            m is not much larger than n);
+//   rounds   Boruvka rounds on the first class until no edge is left between
+//            two components: every component's minimum edge by a minimum on
+//            its 64-bit key word, then every edge that is the minimum of one
+//            of its ends hooks that root onto the other (tie breaking as in
+//            Algorithm 2), then the ends are relabelled to their roots and the
+//            edges inside a component dropped; the same on what is left of the
+//            second class;
+//   filter   a second pass over the endpoints drops the edges inside a
+//            component of the light forest (nearly all of the heavy ones) and
+//            the rounds finish on the others.
+//
+// The lightest edge that leaves a component is in the forest (Sec. 2.3), and an
+// edge inside a component of the lighter edges' forest is not, so every step
+// is exact.
+//
+// Every warp owns a contiguous range of the edges and a region of the kept
+// list of the same capacity: it fills, reads, relabels and compacts its own
+// region in place, so the lists need no global counters and cannot overflow.
+// The rounds kernel is cooperative, one block of 1024 threads per SM; its
+// phases meet at a grid barrier (about 2 us, bounded wait), which costs less
+// than the kernel boundaries and conditional nodes of a graph loop (about 60
+// launches in the CSR path's small calls).  What bounds the steps: select and
+// filter the instruction issue and DRAM (R-MAT 20: 45 and 52 us for 201 and
+// 150 MB), the minimum passes L1 wavefronts (two parents and two minima
+// gathered per edge), late rounds the barriers.
+//
+// Measured on the whole call (build and round loop over the CSR before, this
+// after): R-MAT 26 112 -> 21.9 ms, the 256^3 grid 9.9 -> 2.4 ms, R-MAT 20 1.75
+// -> 0.52 ms, uniform n = 10^6, m = 16 n 2.7 -> 0.55 ms, R-MAT 16 0.49 -> 0.20
+// ms.  Fractions around these (CLASS1 0.25 to 1, CLASS2 1.2 to 3): R-MAT 26
+// 20.7 to 22.9 ms, the grid 2.3 to 4.4, uniform 0.52 to 0.70, R-MAT 20 0.48 to
+// 0.54; a single light class of 1.5 n: 28.4, 3.2, 0.68 and 0.57 ms.
+#include <cuda/atomic>
+
+#include <cstring>
+#include <mutex>
+#include <vector>
+
+#include "exact.cuh"
+#include "internal.cuh"
+
+namespace msf {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int ET = 1024;        // threads per block, one block per SM
+constexpr int EW = ET / 32;     // warps per block
+constexpr int SAMPLES = 1024;   // sampled weights for the thresholds
+constexpr int VOTES = 128;      // sampled edge ends for the giant component
+constexpr int TS_BITS = 11;     // slots of the block's table of minima
+constexpr int TS = 1 << TS_BITS;
+constexpr int HOPS = 16;        // hops of one settling pass
+constexpr int ROUND_CAP = 64;   // Boruvka rounds at most (components at least halve)
+constexpr uint32_t CAND = 0x80000000u;  // list entry may be a minimum of one of its ends
+constexpr uint32_t LONG = 0x80000000u;  // listed root whose chain goes on
+// Edges of the first class, and of both light classes, per vertex.
+constexpr double CLASS1 = 0.75, CLASS2 = 1.5;
+// Below this the light edges form one class: a second one saves less than its
+// rounds' barriers cost (R-MAT 16, m = 2^20: 197 us with one, 212 with two).
+constexpr int64_t TWO_CLASSES = 1 << 22;
+// Edges left from which a round's roots are settled in a step of their own:
+// below, all of them are in flight at once (155 648 threads) and the minimum
+// pass follows the chains itself, one barrier and about 5 us less per round
+// (R-MAT 16: 257 -> 199 us).
+constexpr unsigned long long SMALL = 1 << 17;
+constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
+
+struct Ctrl {
+  unsigned arrive[2];  // grid barriers of the two rounds kernels
+  unsigned abort;      // a barrier wait ran out
+  unsigned err;        // 1 = index out of range, 2 = NaN weight
+  unsigned long long live[2][4];  // edges left, by round modulo 4, of the two rounds kernels
+  unsigned long long thresh[2];  // keys of the first class lie below [0], of the second below [1]
+};
+
+struct Args {
+  int64_t n, m;
+  const int32_t *src, *dst;
+  const uint32_t *w;
+  int32_t wtype;
+  int32_t classes;      // 1 = every edge in the first class, 2 = none heavy, 3
+  int32_t second;       // there is a second class
+  int32_t smem_bits;    // the giant component's bitmap fits in shared memory
+  int64_t E;            // edges per warp region (a multiple of 128)
+  int64_t VE;           // vertices per warp region (a multiple of 128)
+  unsigned rank[2];     // the thresholds' ranks among SAMPLES
+  int32_t *p;
+  unsigned long long *r;
+  int32_t *roots;       // per warp region: roots that may have edges
+  uint32_t *gbits;      // vertices of the giant component, as a bitmap
+  unsigned *front, *back;  // per warp: entries of the first and second class
+  uint4 *list;          // (u, v, edge id, ordered weight), u | CAND
+  uint32_t *mbits;
+  unsigned long long *bins;  // [256] long accumulators (zeroed with the control block)
+  Ctrl *ctl;
+  uint8_t *mask;
+  int32_t *labels;
+  double *totals;
+  unsigned *host;       // pinned: [0] status bits
+};
+
+__device__ __forceinline__ int ld_rel(const int32_t *a) {
+  return cuda::atomic_ref<int, cuda::thread_scope_device>(*const_cast<int32_t *>(a)).load(cuda::memory_order_relaxed);
+}
+__device__ __forceinline__ void st_rel(int32_t *a, int v) {
+  cuda::atomic_ref<int, cuda::thread_scope_device>(*a).store(v, cuda::memory_order_relaxed);
+}
+__device__ __forceinline__ unsigned long long ld_rel64(const unsigned long long *a) {
+  return cuda::atomic_ref<unsigned long long, cuda::thread_scope_device>(*const_cast<unsigned long long *>(a))
+      .load(cuda::memory_order_relaxed);
+}
+
+// All blocks meet; false (everywhere, sooner or later) when a wait ran out.
+__device__ bool grid_barrier(Ctrl *c, int phase, unsigned &target) {
+  if (gridDim.x == 1) {
+    __syncthreads();
+    return true;
+  }
+  __shared__ unsigned ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    target += gridDim.x;
+    cuda::atomic_ref<unsigned, cuda::thread_scope_device> a(c->arrive[phase]), ab(c->abort);
+    __threadfence();
+    a.fetch_add(1u, cuda::memory_order_acq_rel);
+    unsigned good = 0;
+    for (unsigned it = 0; it < (1u << 25); ++it) {
+      if ((int)(a.load(cuda::memory_order_acquire) - target) >= 0) {
+        good = 1;
+        break;
+      }
+      if ((it & 1023u) == 1023u && ab.load(cuda::memory_order_relaxed)) break;
+    }
+    if (!good) ab.store(1u, cuda::memory_order_relaxed);
+    __threadfence();
+    ok = good;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Root of x, whose parent y was read, by its chain; x then points to it.  Hooks
+// happen in other phases, so the roots do not change meanwhile, and a parent
+// read from L1 is an ancestor even when it is out of date.  A long chain goes
+// on in L2 and is halved for the threads behind.
+__device__ __forceinline__ int32_t chase(int32_t *p, int32_t x, int32_t y) {
+  if (y == x) return x;
+  const int32_t x0 = x, y0 = y;
+  x = y;
+  y = __ldca(p + x);
+#pragma unroll 1
+  for (int k = 0; k < 4 && y != x; ++k) {
+    x = y;
+    y = __ldca(p + x);
+  }
+  while (y != x) {
+    const int32_t z = ld_rel(p + y);
+    if (z != y) st_rel(p + x, z);
+    x = z;
+    y = ld_rel(p + x);
+  }
+  if (x != y0) st_rel(p + x0, x);
+  return x;
+}
+
+// The block's shared-memory table of minima.  A slot belongs to the first root
+// that hashes to it; other roots go to r directly.  Late rounds have few
+// roots, most edges end in one of them, and both its atomics and its reads
+// would queue at one L2 line (R-MAT 20: 380 us for a pass over 1.2 M edges).
+struct Table {
+  int32_t key[TS];
+  unsigned long long val[TS];
+};
+__device__ __forceinline__ void table_clear(Table &t) {
+  for (int i = threadIdx.x; i < TS; i += ET) {
+    t.key[i] = -1;
+    t.val[i] = KEY_INF;
+  }
+}
+// The table's slot for a root, or -1 when another root holds it.
+__device__ __forceinline__ int table_slot(Table &t, int32_t root) {
+  const int slot = (int)(((uint32_t)root * 0x9E3779B1u) >> (32 - TS_BITS));
+  int k = *(volatile int32_t *)(t.key + slot);
+  if (k == -1) {
+    k = atomicCAS(t.key + slot, -1, root);
+    if (k == -1) k = root;
+  }
+  return k == root ? slot : -1;
+}
+// Lowers the slot's minimum to `key`; whether it did.
+__device__ __forceinline__ bool table_offer(Table &t, int slot, unsigned long long key) {
+  unsigned long long old = *(volatile unsigned long long *)(t.val + slot);
+  while (key < old) {
+    const unsigned long long seen = atomicCAS(t.val + slot, old, key);
+    if (seen == old) return true;
+    old = seen;
+  }
+  return false;
+}
+
+// The block's long accumulators of float32 weights (weight_bin): 64-bit sums as
+// two words, added with 32-bit shared atomics and a carry (a 64-bit shared
+// atomic is a compare-and-swap loop, and a warp's weights share few bins); the
+// low words four times over, by lane, to spread the equal bins of a warp.
+struct Sums {
+  unsigned lo[4][256], hi[256];
+  __device__ void clear() {
+    for (int i = threadIdx.x; i < 256; i += ET) lo[0][i] = lo[1][i] = lo[2][i] = lo[3][i] = hi[i] = 0;
+  }
+  __device__ __forceinline__ void add(uint32_t ordw) {
+    int bin;
+    long long val;
+    weight_bin(ordw, MSF_F32, &bin, &val);
+    const unsigned v = (unsigned)val;
+    const unsigned old = atomicAdd(&lo[threadIdx.x & 3][bin], v);
+    const unsigned h = (unsigned)((unsigned long long)val >> 32) + (old + v < old ? 1u : 0u);
+    if (h) atomicAdd(&hi[bin], h);
+  }
+  __device__ unsigned long long get(int b) const {
+    return ((unsigned long long)hi[b] << 32) + lo[0][b] + lo[1][b] + lo[2][b] + lo[3][b];
+  }
+};
+
+// Minimum pass over `cnt` entries of the warp from S, which end up at L (the
+// same place, or S lies further back in the region): with RELABEL the ends
+// become their roots first (their parents) and the entries inside a component
+// are dropped.  Every end's minimum is lowered to the entry's key; an entry that
+// lowered one is marked CAND (the final minimum did).  Returns the entries
+// left.
+template <bool RELABEL, bool CHASE = false>
+__device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const uint4 *S, uint4 *L, unsigned cnt) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  constexpr int U = 4;
+  unsigned out = 0;
+  for (unsigned b0 = 0; b0 < cnt; b0 += 32 * U) {
+    uint4 x[U];
+    bool on[U];
+    int32_t u[U], v[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned i = b0 + j * 32 + lane;
+      on[j] = i < cnt;
+      x[j] = on[j] ? S[i] : make_uint4(0u, 0u, 0u, 0u);
+      u[j] = (int32_t)(x[j].x & ~CAND);
+      v[j] = (int32_t)x[j].y;
+    }
+    if (RELABEL) {
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const int32_t a = u[j], b = v[j];
+        u[j] = on[j] ? __ldca(A.p + a) : 0;
+        v[j] = on[j] ? __ldca(A.p + b) : 0;
+      }
+      if (CHASE) {
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          if (!on[j]) continue;
+          u[j] = chase(A.p, (int32_t)(x[j].x & ~CAND), u[j]);
+          v[j] = chase(A.p, (int32_t)x[j].y, v[j]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) on[j] = on[j] && u[j] != v[j];
+    }
+    // ends in the table; the others read their global minimum
+    bool cand[U];
+    unsigned long long ru[U], rv[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
+      cand[j] = false;
+      ru[j] = rv[j] = 0ull;
+      if (on[j]) {
+        const int su = table_slot(tab, u[j]), sv = table_slot(tab, v[j]);
+        if (su < 0) ru[j] = ld_rel64(A.r + u[j]);
+        else cand[j] |= table_offer(tab, su, key);
+        if (sv < 0) rv[j] = ld_rel64(A.r + v[j]);
+        else cand[j] |= table_offer(tab, sv, key);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
+      if (key < ru[j]) {
+        atomicMin(A.r + u[j], key);
+        cand[j] = true;
+      }
+      if (key < rv[j]) {
+        atomicMin(A.r + v[j], key);
+        cand[j] = true;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned bal = __ballot_sync(FULL, on[j]);
+      const unsigned at = out + __popc(bal & below);
+      if (on[j]) L[at] = make_uint4((uint32_t)u[j] | (cand[j] ? CAND : 0u), (uint32_t)v[j], x[j].z, x[j].w);
+      out += __popc(bal);
+    }
+  }
+  __syncwarp();
+  return out;
+}
+
+// Hooks along every entry that is the minimum of one of its ends (tie
+// breaking: of two roots that chose the same edge the smaller stays a root).
+__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, Sums &sums,
+                                          unsigned long long &usum) {
+  const int lane = threadIdx.x & 31;
+  constexpr int U = 4;
+  for (unsigned b0 = 0; b0 < cnt; b0 += 32 * U) {
+    uint4 x[U];
+    unsigned long long ru[U], rv[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned i = b0 + j * 32 + lane;
+      x[j] = i < cnt ? L[i] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const bool c = (x[j].x & CAND) != 0;
+      ru[j] = c ? __ldca(A.r + (x[j].x & ~CAND)) : KEY_INF;
+      rv[j] = c ? __ldca(A.r + x[j].y) : KEY_INF;
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int32_t u = (int32_t)(x[j].x & ~CAND), v = (int32_t)x[j].y;
+      const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
+      const bool mu = ru[j] == key, mv = rv[j] == key;
+      if (!((x[j].x & CAND) && (mu || mv))) continue;
+      if (small) {  // the minima are cleared here (no other entry's key equals them, before or after)
+        if (mu) A.r[u] = KEY_INF;
+        if (mv) A.r[v] = KEY_INF;
+      }
+      if (mu && (!mv || v < u)) A.p[u] = v;
+      else A.p[v] = u;
+      if (A.mbits) atomicOr(A.mbits + (x[j].z >> 5), 1u << (x[j].z & 31u));
+      if (A.totals) {
+        if (A.wtype == MSF_U32) usum += x[j].w;
+        else sums.add(x[j].w);
+      }
+    }
+  }
+}
+
+// Four consecutive edges of a lane.
+struct Quad {
+  int4 s, d;
+  uint4 w;
+};
+template <bool VEC>
+__device__ __forceinline__ Quad load_quad(const Args &A, int64_t e, int64_t hi) {
+  Quad q;
+  q.s = q.d = make_int4(0, 0, 0, 0);
+  q.w = make_uint4(0u, 0u, 0u, 0u);
+  if (VEC && e + 4 <= hi) {
+    q.s = __ldcs(reinterpret_cast<const int4 *>(A.src + e));
+    q.d = __ldcs(reinterpret_cast<const int4 *>(A.dst + e));
+    q.w = __ldcs(reinterpret_cast<const uint4 *>(A.w + e));
+  } else if (e < hi) {
+    q.s.x = A.src[e];
+    q.d.x = A.dst[e];
+    q.w.x = A.w[e];
+    if (e + 1 < hi) {
+      q.s.y = A.src[e + 1];
+      q.d.y = A.dst[e + 1];
+      q.w.y = A.w[e + 1];
+    }
+    if (e + 2 < hi) {
+      q.s.z = A.src[e + 2];
+      q.d.z = A.dst[e + 2];
+      q.w.z = A.w[e + 2];
+    }
+    if (e + 3 < hi) {
+      q.s.w = A.src[e + 3];
+      q.d.w = A.dst[e + 3];
+      q.w.w = A.w[e + 3];
+    }
+  }
+  return q;
+}
+
+// Their ends only.
+struct Ends {
+  int4 s, d;
+};
+template <bool VEC>
+__device__ __forceinline__ Ends load_ends(const Args &A, int64_t e, int64_t hi) {
+  Ends q;
+  q.s = q.d = make_int4(0, 0, 0, 0);
+  if (VEC && e + 4 <= hi) {
+    q.s = __ldcs(reinterpret_cast<const int4 *>(A.src + e));
+    q.d = __ldcs(reinterpret_cast<const int4 *>(A.dst + e));
+  } else if (e < hi) {
+    int32_t *s = &q.s.x, *d = &q.d.x;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (e + j < hi) {
+        s[j] = A.src[e + j];
+        d[j] = A.dst[e + j];
+      }
+  }
+  return q;
+}
+
+// Whether a weight lies below a threshold key (weight tw, edge index te, te a
+// multiple of 128): one comparison per edge, with the edges of a batch of 128
+// all on one side of te.
+template <bool F32>
+struct Limit {
+  uint32_t at, under;  // largest weight below the threshold, for edges before and from te
+  int64_t te;
+  bool none;           // no weight lies below it from te on
+  uint32_t lim;
+  bool ok;
+  __device__ Limit(unsigned long long T) {
+    const uint32_t tw = (uint32_t)(T >> 32);
+    te = (int64_t)(uint32_t)T == 0xffffffffll ? (int64_t)1 << 40 : (int64_t)(uint32_t)T;
+    at = tw;
+    none = tw == 0;
+    under = tw - (none ? 0u : 1u);
+    if (F32) {  // the comparison is of floats (NaN: false)
+      at = from_ord(at);
+      under = none ? 0x7fffffffu : from_ord(under);
+    }
+  }
+  __device__ static uint32_t from_ord(uint32_t o) {
+    const uint32_t b = (o & 0x80000000u) ? o & 0x7fffffffu : ~o;
+    return (b << 1) > 0xff000000u ? ((b >> 31) ? 0x7fffffffu : 0x7f800000u) : b;
+  }
+  __device__ __forceinline__ void batch(int64_t e) {  // the batch of edges from e on
+    const bool before = e < te;
+    lim = before ? at : under;
+    ok = F32 || before || !none;
+  }
+  __device__ __forceinline__ bool below(uint32_t w) const {
+    return F32 ? __uint_as_float(w) <= __uint_as_float(lim) : (w <= lim && ok);
+  }
+};
+
+// First pass over the warp's edges [lo, hi): validation; the non-loop edges
+// below T0 go to the front of the warp's list, those from T0 to T1 to its back
+// (growing downwards from the region's end).  Two batches of edges per warp
+// are in flight.  The pass is bound by instruction issue, so an edge costs a
+// running maximum (the index check), a NaN test and one or two comparisons
+// until it is selected.
+template <bool VEC, bool F32>
+__device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t hi, unsigned long long T0,
+                                            unsigned long long T1, uint4 *L, unsigned &front, unsigned &back,
+                                            unsigned &err) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const uint32_t n = (uint32_t)A.n;
+  front = back = 0;
+  if (lo >= hi) return;
+  uint4 *LB = L + A.E - 1;
+  Limit<F32> l0(T0), l1(T1);
+  uint32_t top = 0;  // largest index seen
+  bool nan = false;
+  Quad q1 = load_quad<VEC>(A, lo + 4 * lane, hi), q2 = load_quad<VEC>(A, lo + 128 + 4 * lane, hi);
+  for (int64_t b = lo; b < hi; b += 128) {
+    const int64_t e0 = b + 4 * lane;
+    const Quad q = q1;
+    q1 = q2;
+    q2 = load_quad<VEC>(A, e0 + 256, hi);  // (zeros past the end: self-loops)
+    const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
+    const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
+    const uint32_t w[4] = {q.w.x, q.w.y, q.w.z, q.w.w};
+    l0.batch(b);
+    l1.batch(b);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      top = max(top, max(u[j], v[j]));
+      if (F32) nan |= __uint_as_float(w[j]) != __uint_as_float(w[j]);
+      const bool sel = l1.below(w[j]) && u[j] != v[j];
+      const unsigned m = __ballot_sync(FULL, sel);
+      if (!m) continue;
+      // (an edge with an invalid index is selected too; it is never used)
+      const unsigned mf = __ballot_sync(FULL, sel && l0.below(w[j]));
+      const bool fr = mf >> lane & 1u;
+      if (sel) {
+        uint4 *at = fr ? L + (front + __popc(mf & below)) : LB - (back + __popc(m & ~mf & below));
+        *at = make_uint4(u[j], v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
+      }
+      front += __popc(mf);
+      back += __popc(m & ~mf);
+    }
+  }
+  err = (top >= n ? 1u : 0u) | (nan ? 2u : 0u);
+  __syncwarp();
+}
+
+// Second pass over the warp's edges: those whose ends lie in different
+// components go to the list, as roots (parents are roots here).  A light edge
+// lies inside a component, so the weights are read for the edges left only.
+// Most edges lie inside the giant component: two bits of its bitmap tell,
+// from shared memory when it fits there (a gather of parents is one L1
+// wavefront per lane; R-MAT 20: 30 M of them).
+template <bool VEC, bool SMEM>
+__device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64_t hi, const uint32_t *bits,
+                                                uint4 *L) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned out = 0;
+  if (lo >= hi) return 0;
+  Ends q1 = load_ends<VEC>(A, lo + 4 * lane, hi), q2 = load_ends<VEC>(A, lo + 128 + 4 * lane, hi);
+  for (int64_t b = lo; b < hi; b += 128) {
+    const int64_t e0 = b + 4 * lane;
+    const Ends q = q1;
+    q1 = q2;
+    q2 = load_ends<VEC>(A, e0 + 256, hi);  // (zeros past the end: self-loops)
+    int32_t u[4] = {q.s.x, q.s.y, q.s.z, q.s.w}, v[4] = {q.d.x, q.d.y, q.d.z, q.d.w};
+    uint32_t bu[4], bv[4], w[4];
+    bool on[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      bu[j] = SMEM ? bits[(uint32_t)u[j] >> 5] : __ldca(bits + ((uint32_t)u[j] >> 5));
+      bv[j] = SMEM ? bits[(uint32_t)v[j] >> 5] : __ldca(bits + ((uint32_t)v[j] >> 5));
+    }
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      on[j] = !(__funnelshift_r(bu[j], bu[j], u[j]) & __funnelshift_r(bv[j], bv[j], v[j]) & 1u);
+      any |= on[j];
+    }
+    if (!__any_sync(FULL, any)) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      on[j] = on[j] && e0 + j < hi;
+      w[j] = on[j] ? __ldcs(A.w + e0 + j) : 0u;
+      u[j] = on[j] ? __ldca(A.p + u[j]) : 0;
+      v[j] = on[j] ? __ldca(A.p + v[j]) : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool o = u[j] != v[j];
+      const unsigned bal = __ballot_sync(FULL, o);
+      if (o)
+        L[out + __popc(bal & below)] =
+            make_uint4((uint32_t)u[j], (uint32_t)v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], A.wtype));
+      out += __popc(bal);
+    }
+  }
+  __syncwarp();
+  return out;
+}
+
+// The thresholds: the sample's keys (edge indices rounded down to a batch) of the two wanted ranks, found bit by bit
+// (one sample per thread, block 0).  The low half of a key, the edge index,
+// only matters where many samples share the threshold's weight.
+__device__ void pick_thresholds(const Args &A) {
+  static_assert(SAMPLES == ET, "one sample per thread");
+  const int64_t step = A.m / SAMPLES;  // m >= SAMPLES
+  const int64_t i = threadIdx.x;
+  const uint32_t h = (uint32_t)i * 0x9E3779B1u;
+  const int64_t e = i * A.m / SAMPLES + (int64_t)(((uint64_t)h * (uint64_t)step) >> 32);
+  const uint32_t w = ord_weight_dev(A.w[e], A.wtype);
+  const unsigned r0 = A.rank[0], r1 = A.rank[1];
+  uint32_t w0 = 0, w1 = 0;
+  for (int b = 31; b >= 0; --b) {
+    const uint32_t c0 = w0 | (1u << b), c1 = w1 | (1u << b);
+    if (__syncthreads_count(w < c0) <= (int)r0) w0 = c0;
+    if (__syncthreads_count(w < c1) <= (int)r1) w1 = c1;
+  }
+  // samples below w0: at most r0; with those equal to it: more
+  uint32_t e0 = 0xffffffffu, e1 = 0xffffffffu;
+  if (__syncthreads_count(w <= w0) > (int)(r0 + r0 / 4 + 1) || __syncthreads_count(w <= w1) > (int)(r1 + r1 / 4 + 1)) {
+    e0 = e1 = 0;
+    for (int b = 31; b >= 0; --b) {
+      const uint32_t c0 = e0 | (1u << b), c1 = e1 | (1u << b);
+      if (__syncthreads_count(w < w0 || (w == w0 && (uint32_t)e < c0)) <= (int)r0) e0 = c0;
+      if (__syncthreads_count(w < w1 || (w == w1 && (uint32_t)e < c1)) <= (int)r1) e1 = c1;
+    }
+  }
+  if (threadIdx.x == 0) {
+    A.ctl->thresh[0] = ((unsigned long long)w0 << 32) | (e0 == 0xffffffffu ? e0 : e0 & ~127u);
+    A.ctl->thresh[1] = ((unsigned long long)w1 << 32) | (e1 == 0xffffffffu ? e1 : e1 & ~127u);
+  }
+}
+
+// The root that most of VOTES sampled edge ends lie under (every block finds
+// the same one): the giant component, when there is one.
+__device__ int32_t vote_giant(const Args &A) {
+  __shared__ int32_t vote[VOTES];
+  __shared__ unsigned best;
+  if (threadIdx.x == 0) best = 0;
+  if (threadIdx.x < VOTES) {
+    const int64_t e = (int64_t)((unsigned long long)threadIdx.x * (unsigned long long)A.m / VOTES);
+    int32_t x = (threadIdx.x & 1) ? A.src[e] : A.dst[e];
+    if ((uint32_t)x >= (uint32_t)A.n) x = 0;  // (an invalid edge: the call fails later)
+    int32_t y = __ldca(A.p + x);
+    while (y != x) {
+      x = y;
+      y = __ldca(A.p + x);
+    }
+    vote[threadIdx.x] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < VOTES) {
+    unsigned c = 0;
+    for (int i = 0; i < VOTES; ++i) c += vote[i] == vote[threadIdx.x];
+    atomicMax(&best, (c << 16) | (unsigned)threadIdx.x);
+  }
+  __syncthreads();
+  return vote[best & 0xffffu];
+}
+
+// Parents, minima, root lists and the forest bitmap; the thresholds.
+__global__ void __launch_bounds__(ET, 1) k_prepare(Args A) {
+  const int64_t tid = (int64_t)blockIdx.x * ET + threadIdx.x, nthr = (int64_t)gridDim.x * ET;
+  for (int64_t v = tid; v < A.n; v += nthr) {
+    A.p[v] = (int32_t)v;
+    A.r[v] = KEY_INF;
+    A.roots[v] = (int32_t)v;
+  }
+  if (A.mbits) {
+    const int64_t words = (A.m + 31) / 32 + 2;
+    for (int64_t i = tid; i < words; i += nthr) A.mbits[i] = 0u;
+  }
+  if (A.classes > 1 && blockIdx.x == 0) pick_thresholds(A);
+}
+
+template <bool VEC, bool F32>
+__global__ void __launch_bounds__(ET, 1) k_select(Args A) {
+  const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
+  const int64_t lo = warp * A.E, hi = lo + A.E < A.m ? lo + A.E : A.m;
+  const unsigned long long T0 = A.classes > 1 ? A.ctl->thresh[0] : KEY_INF;
+  const unsigned long long T1 = A.classes > 2 ? A.ctl->thresh[1] : KEY_INF;
+  unsigned front, back, err = 0;
+  select_pass<VEC, F32>(A, lo, hi, T0, T1, A.list + lo, front, back, err);
+  if (err) atomicOr(&A.ctl->err, err);
+  if ((threadIdx.x & 31) == 0) {  // (an invalid edge ends the call: no list is used)
+    A.front[warp] = front;
+    A.back[warp] = back;
+  }
+}
+
+template <bool VEC, bool SMEM>
+__global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
+  extern __shared__ uint32_t dyn_bits[];
+  const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
+  const int64_t lo = warp * A.E, hi = lo + A.E < A.m ? lo + A.E : A.m;
+  unsigned front = 0;
+  if (!A.ctl->err && !A.ctl->abort) {  // (an invalid edge's index must not be used)
+    if (SMEM) {
+      const int64_t words = (A.n + 31) / 32;
+      for (int64_t i = threadIdx.x; i < words; i += ET) dyn_bits[i] = A.gbits[i];
+      __syncthreads();
+    }
+    front = filter_pass<VEC, SMEM>(A, lo, hi, SMEM ? dyn_bits : A.gbits, A.list + lo);
+  }
+  if ((threadIdx.x & 31) == 0) A.front[warp] = front;
+}
+
+// The rounds on the light classes (phase 0; the bitmap of the giant component
+// when a heavy class follows) or on the heavy edges left (phase 1); the
+// results at the end.
+__global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
+  __shared__ Sums sums;
+  __shared__ long long sbins[256];
+  __shared__ Table tab;
+  __shared__ unsigned s_live;
+  Ctrl *C = A.ctl;
+  if (C->abort) return;  // (phase 0 did not finish)
+  if (C->err) {          // an invalid edge: its indices must not be used
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.host[0] = C->err;
+    return;
+  }
+  unsigned target = 0;
+  const int64_t tid = (int64_t)blockIdx.x * ET + threadIdx.x, nthr = (int64_t)gridDim.x * ET;
+  const int64_t warp = tid >> 5;
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned long long usum = 0;  // uint32 weights of the thread's forest edges
+  sums.clear();
+  if (threadIdx.x == 0) s_live = 0;
+  table_clear(tab);
+  __syncthreads();
+  // the warp's vertices and its list of roots (all of them, or what the
+  // flattening before the filter left)
+  const int64_t vlo = warp * A.VE < A.n ? warp * A.VE : A.n, vhi = vlo + A.VE < A.n ? vlo + A.VE : A.n;
+  int32_t *V = A.roots + vlo;
+  unsigned vc = phase == 0 ? (unsigned)(vhi - vlo) : A.back[warp];
+  uint4 *L = A.list + warp * A.E;
+  unsigned it = 0;  // counter of the grid sums
+  auto aborted = [&]() { return *(volatile unsigned *)&C->abort != 0; };
+  // The block's table goes to r; then the grid meets and the warps' counts are
+  // summed (0 when the wait ran out).
+  auto total_live = [&](unsigned cnt) -> unsigned long long {
+    if (lane == 0 && cnt) atomicAdd(&s_live, cnt);
+    __syncthreads();
+    for (int i = threadIdx.x; i < TS; i += ET) {
+      const int32_t k = tab.key[i];
+      const unsigned long long v = tab.val[i];
+      if (k >= 0 && v < ld_rel64(A.r + k)) atomicMin(A.r + k, v);
+    }
+    table_clear(tab);  // (the thread's own slots)
+    if (threadIdx.x == 0) {
+      if (s_live) atomicAdd(&C->live[phase][it & 3u], (unsigned long long)s_live);
+      s_live = 0;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) C->live[phase][(it + 2) & 3u] = 0;
+    if (!grid_barrier(C, phase, target)) return 0;
+    const unsigned long long t = ld_rel64(&C->live[phase][it & 3u]);
+    ++it;
+    return t;
+  };
+  // The roots that hooked point to their new roots (Algorithm 3's chase of
+  // the changed roots): passes of up to HOPS hops, each parent written by its
+  // own thread only, until no chain is longer.  The list keeps the roots that
+  // did not hook; a root without a minimum has no edge left and leaves it.
+  // The minima are cleared on the way.
+  auto settle_roots = [&]() -> bool {
+    constexpr int U = 4;
+    for (int pass = 0; pass < ROUND_CAP; ++pass) {
+      unsigned out = 0;
+      bool more = false;
+      for (unsigned b0 = 0; b0 < vc; b0 += 32 * U) {
+        uint32_t k[U];
+        int32_t x[U];
+        unsigned long long rv[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const unsigned i = b0 + j * 32 + lane;
+          k[j] = i < vc ? (uint32_t)V[i] : 0xffffffffu;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const bool on = k[j] != 0xffffffffu;
+          const int32_t v = (int32_t)(k[j] & ~LONG);
+          rv[j] = on && pass == 0 ? ld_rel64(A.r + v) : 0ull;
+          x[j] = on && (pass == 0 || (k[j] & LONG)) ? ld_rel(A.p + v) : v;
+        }
+        int32_t y[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const int32_t v = (int32_t)(k[j] & ~LONG);
+          y[j] = k[j] != 0xffffffffu && rv[j] != KEY_INF && x[j] != v ? __ldca(A.p + x[j]) : x[j];
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          bool keep = k[j] != 0xffffffffu;
+          const int32_t v = (int32_t)(k[j] & ~LONG);
+          if (keep && rv[j] == KEY_INF) keep = false;
+          if (keep && pass == 0) A.r[v] = KEY_INF;
+          if (keep && x[j] != v) {
+            int32_t a = x[j], b = y[j];
+#pragma unroll 1
+            for (int h = 0; h < HOPS && b != a; ++h) {
+              a = b;
+              b = __ldca(A.p + a);
+            }
+            if (a != x[j]) st_rel(A.p + v, a);
+            keep = b != a;
+            more |= keep;
+            k[j] = (uint32_t)v | LONG;
+          }
+          const unsigned bal = __ballot_sync(FULL, keep);
+          if (keep) V[out + __popc(bal & below)] = (int32_t)k[j];
+          out += __popc(bal);
+        }
+      }
+      __syncwarp();
+      vc = out;
+      const unsigned long long left = total_live(__any_sync(FULL, more) ? 1u : 0u);
+      if (aborted()) return false;
+      if (!left) return true;
+    }
+    return true;  // (a pass shortens every chain HOPS-fold: never reached)
+  };
+  // Every vertex points to its root (a chain has one hop per round at most),
+  // the warp's list takes the roots among its vertices and, when asked for,
+  // the bitmap the members of the tree `giant`.
+  auto flatten = [&](bool bits, int32_t giant) -> bool {
+    constexpr int U = 4;
+    unsigned out = 0;
+    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+      int32_t x[U], y[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const int64_t v = v0 + j * 32 + lane;
+        x[j] = v < vhi ? ld_rel(A.p + v) : -1;
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) y[j] = x[j] >= 0 ? __ldca(A.p + x[j]) : -1;
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const int64_t v = v0 + j * 32 + lane;
+        int32_t a = x[j], b = y[j];
+        while (b != a) {
+          a = b;
+          b = __ldca(A.p + a);
+        }
+        if (a != x[j]) st_rel(A.p + v, a);
+        const bool root = v < vhi && a == (int32_t)v;
+        const unsigned mr = __ballot_sync(FULL, root);
+        if (root) V[out + __popc(mr & below)] = a;
+        out += __popc(mr);
+        if (bits) {
+          const unsigned mg = __ballot_sync(FULL, v < vhi && a == giant);
+          if (lane == 0 && v < vhi) A.gbits[v >> 5] = mg;
+        }
+      }
+    }
+    __syncwarp();
+    vc = out;
+    return grid_barrier(C, phase, target);
+  };
+  // Rounds on the warp's `cnt` entries until no edge is left; the minima of
+  // the first one have been offered.  With few edges left the roots are not
+  // settled in a step of their own (a barrier and a pass over the roots, about
+  // 5 us): the minimum pass follows the chains, all at the same time.
+  auto rounds = [&](unsigned cnt) -> bool {
+    unsigned long long live = total_live(cnt);
+    for (int k = 0; k < ROUND_CAP && live; ++k) {
+      const bool small = live <= SMALL;
+      hook_pass(A, L, cnt, small, sums, usum);
+      if (!grid_barrier(C, phase, target)) return false;
+      if (!small) {
+        if (!settle_roots()) return false;
+        cnt = min_pass<true>(A, tab, L, L, cnt);
+      } else {
+        cnt = min_pass<true, true>(A, tab, L, L, cnt);
+      }
+      live = total_live(cnt);
+    }
+    return !aborted();
+  };
+
+  unsigned cnt = A.front[warp];
+  cnt = min_pass<false>(A, tab, L, L, cnt);
+  if (!rounds(cnt)) return;
+  if (phase == 0 && A.second) {
+    if (!flatten(false, 0)) return;
+    const unsigned back = A.back[warp];
+    cnt = min_pass<true>(A, tab, L + A.E - back, L, back);
+    if (!rounds(cnt)) return;
+  }
+  const bool last = phase == 1 || A.classes < 3;
+  if (!last) {
+    flatten(true, vote_giant(A));
+    if (lane == 0) A.back[warp] = vc;
+  }
+  // the forest's weight so far
+  if (A.totals) {
+    if (A.wtype == MSF_U32) {
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) usum += __shfl_xor_sync(FULL, usum, d);
+      if (lane == 0 && usum) atomicAdd(A.bins, usum);
+    } else {
+      __syncthreads();
+      for (int i = threadIdx.x; i < 256; i += ET) {
+        const unsigned long long v = sums.get(i);
+        if (v) atomicAdd(A.bins + i, v);
+      }
+    }
+  }
+  if (!last) return;
+  // results.  The smallest vertex of every tree: r is all KEY_INF again, and
+  // the low half of a root's word takes the minimum of the tree's other
+  // vertices (through the block's table); a label is the smaller of it and the
+  // root.
+  constexpr int U = 4;
+  if (A.labels) {
+    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+      int32_t x[U], y[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) x[j] = v0 + j * 32 + lane < vhi ? ld_rel(A.p + v0 + j * 32 + lane) : 0;
+#pragma unroll
+      for (int j = 0; j < U; ++j) y[j] = __ldca(A.p + x[j]);
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const int64_t v = v0 + j * 32 + lane;
+        if (v >= vhi) continue;
+        int32_t a = x[j], b = y[j];
+        while (b != a) {
+          a = b;
+          b = __ldca(A.p + a);
+        }
+        if (a != x[j]) st_rel(A.p + v, a);
+        if (a <= (int32_t)v) continue;  // (the root itself is added when read)
+        const int slot = table_slot(tab, a);
+        unsigned *low = reinterpret_cast<unsigned *>(slot < 0 ? A.r + a : tab.val + slot);
+        if (slot < 0 || (unsigned)v < *(volatile unsigned *)low) atomicMin(low, (unsigned)v);
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < TS; i += ET) {
+      const unsigned b = *reinterpret_cast<unsigned *>(tab.val + i);
+      if (tab.key[i] >= 0 && b != 0xffffffffu) atomicMin(reinterpret_cast<unsigned *>(A.r + tab.key[i]), b);
+    }
+  }
+  if (!grid_barrier(C, phase, target)) return;
+  if (A.totals && blockIdx.x == 0) {
+    for (int i = threadIdx.x; i < 256; i += ET) sbins[i] = (long long)ld_rel64(A.bins + i);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const double t = combine_bins_warp(sbins, A.wtype);
+      if (threadIdx.x == 0) *A.totals = t;
+    }
+  }
+  if (A.labels) {
+    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+      int32_t x[U];
+      unsigned b[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) x[j] = v0 + j * 32 + lane < vhi ? __ldca(A.p + v0 + j * 32 + lane) : 0;
+#pragma unroll
+      for (int j = 0; j < U; ++j) b[j] = __ldca(reinterpret_cast<const unsigned *>(A.r + x[j]));
+#pragma unroll
+      for (int j = 0; j < U; ++j)
+        if (v0 + j * 32 + lane < vhi) A.labels[v0 + j * 32 + lane] = (int32_t)(b[j] < (unsigned)x[j] ? b[j] : (unsigned)x[j]);
+    }
+  }
+  if (A.mask) {
+    const int64_t m = A.m;
+    const int64_t head = (int64_t)((16 - (reinterpret_cast<uintptr_t>(A.mask) & 15)) & 15);
+    const int64_t h = head < m ? head : m;
+    const int64_t nq = (m - h) >> 4;
+    uint4 *q = reinterpret_cast<uint4 *>(A.mask + h);
+    for (int64_t e = tid; e < h; e += nthr) A.mask[e] = (uint8_t)((A.mbits[e >> 5] >> (e & 31)) & 1u);
+    for (int64_t i = tid; i < nq; i += nthr) q[i] = spread16(bits16(A.mbits, h + (i << 4)));
+    for (int64_t e = h + (nq << 4) + tid; e < m; e += nthr)
+      A.mask[e] = (uint8_t)((A.mbits[e >> 5] >> (e & 31)) & 1u);
+  }
+  if (tid == 0) A.host[0] = *(volatile unsigned *)&C->err;
+}
+
+// Pinned words that the kernel writes its status into; a call takes one and
+// gives it back.
+std::mutex g_pin_mu;
+std::vector<unsigned *> g_pin_free;
+struct Pinned {
+  unsigned *p = nullptr;
+  int take() {
+    {
+      std::lock_guard<std::mutex> lk(g_pin_mu);
+      if (!g_pin_free.empty()) {
+        p = g_pin_free.back();
+        g_pin_free.pop_back();
+      }
+    }
+    if (!p) MSF_CK(cudaHostAlloc((void **)&p, 64, cudaHostAllocPortable | cudaHostAllocMapped));
+    p[0] = 0;
+    return MSF_OK;
+  }
+  ~Pinned() {
+    if (!p) return;
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    g_pin_free.push_back(p);
+  }
+};
+
+size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+
+}  // namespace
+
+// Forest of one graph from its edge list (pointers the device can read).  Any
+// output may be NULL.  Synchronizes `s`.
+int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const uint32_t *w, int wtype,
+                uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s) {
+  Args A;
+  std::memset(&A, 0, sizeof(A));
+  A.n = n;
+  A.m = m;
+  A.src = src;
+  A.dst = dst;
+  A.w = w;
+  A.wtype = wtype;
+  const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
+                     reinterpret_cast<uintptr_t>(w)) & 15) == 0;
+  // blocks: one per 8192 edges or vertices, at most one per SM
+  int64_t want = ((m > n ? m : n) + 8191) / 8192;
+  if (want < 1) want = 1;
+  const int64_t cap = (int64_t)sm_count();
+  const int blocks = (int)(want < cap ? want : cap);
+  const int64_t warps = (int64_t)blocks * EW;
+  A.E = ((m + warps - 1) / warps + 127) / 128 * 128;
+  A.VE = ((n + warps - 1) / warps + 127) / 128 * 128;
+  A.classes = 1;
+  if (m >= 64 * SAMPLES) {
+    double la = CLASS1, lb = CLASS2;
+    if (m < TWO_CLASSES) la = lb;
+    if ((double)m > 1.25 * la * (double)n && la < lb) A.classes = 2;
+    if ((double)m > 1.25 * lb * (double)n) A.classes = 3;
+    A.second = A.classes > 1 && la < lb;
+    A.rank[0] = (unsigned)(la * (double)n / (double)m * SAMPLES);
+    A.rank[1] = (unsigned)(lb * (double)n / (double)m * SAMPLES);
+  }
+  const size_t bit_bytes = (size_t)((n + 31) / 32) * 4;
+  A.smem_bits = A.classes > 2 && bit_bytes <= SMEM_BITS;
+  const size_t dyn = A.smem_bits ? bit_bytes : 0;
+  size_t off = 0;
+  auto place = [&](size_t bytes) {
+    const size_t at = off;
+    off = align_up(off + bytes);
+    return at;
+  };
+  static_assert(sizeof(Ctrl) <= 256, "control block");
+  const size_t ctl_bytes = 256 + 256 * 8;  // control block, long accumulators
+  const size_t o_ctl = place(ctl_bytes), o_p = place((size_t)(n + 1) * 4), o_r = place((size_t)(n + 1) * 8);
+  const size_t o_roots = place((size_t)(n + 1) * 4), o_gbits = place(bit_bytes);
+  const size_t o_bits = place(((size_t)(m + 31) / 32 + 2) * 4);
+  const size_t o_front = place((size_t)warps * 4), o_back = place((size_t)warps * 4);
+  const size_t o_list = place((size_t)warps * (size_t)A.E * 16);
+  int err = MSF_OK;
+  char *base = (char *)pool_alloc(off, &err);
+  if (err) return err;
+  struct Back {
+    void *p;
+    ~Back() { pool_free(p); }
+  } back{base};
+  Pinned pin;
+  if (int rc = pin.take()) return rc;
+  pin.p[0] = 0x80000000u;  // not finished
+  A.ctl = (Ctrl *)(base + o_ctl);
+  A.p = (int32_t *)(base + o_p);
+  A.r = (unsigned long long *)(base + o_r);
+  A.roots = (int32_t *)(base + o_roots);
+  A.gbits = (uint32_t *)(base + o_gbits);
+  A.mbits = mask ? (uint32_t *)(base + o_bits) : nullptr;
+  A.bins = (unsigned long long *)(base + o_ctl + 256);
+  A.front = (unsigned *)(base + o_front);
+  A.back = (unsigned *)(base + o_back);
+  A.list = (uint4 *)(base + o_list);
+  A.mask = mask;
+  A.labels = labels;
+  A.totals = totals;
+  A.host = pin.p;
+  MSF_CK(cudaMemsetAsync(A.ctl, 0, ctl_bytes, s));
+  k_prepare<<<blocks, ET, 0, s>>>(A);
+  void (*select)(Args) = wtype == MSF_F32 ? (vec ? k_select<true, true> : k_select<false, true>)
+                                          : (vec ? k_select<true, false> : k_select<false, false>);
+  select<<<blocks, ET, 0, s>>>(A);
+  int phase = 0;
+  void *args[] = {&A, &phase};
+  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
+  if (e == cudaSuccess && A.classes > 2) {
+    void (*filter)(Args) = A.smem_bits ? (vec ? k_filter<true, true> : k_filter<false, true>)
+                                       : (vec ? k_filter<true, false> : k_filter<false, false>);
+    if (A.smem_bits)
+      e = cudaFuncSetAttribute(filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BITS);
+    if (e == cudaSuccess) {
+      filter<<<blocks, ET, dyn, s>>>(A);
+      phase = 1;
+      e = cudaLaunchCooperativeKernel((const void *)k_rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
+    }
+  }
+  if (e == cudaErrorCooperativeLaunchTooLarge) {  // (a share of the device that holds fewer blocks)
+    cudaGetLastError();
+    MSF_CK(cudaStreamSynchronize(s));
+    return SOLVE_NOT_RUN;
+  }
+  if (e == cudaSuccess) e = cudaGetLastError();
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) return cuda_fail(e, "forest of an edge list");
+  const unsigned st = *(volatile unsigned *)pin.p;
+  if (st & 0x80000000u) return fail(MSF_ERR_CHECK, "device consistency check failed");
+  if (st & 1u) return fail(MSF_ERR_INVALID_ARG, "vertex index out of range");
+  if (st & 2u) return fail(MSF_ERR_INVALID_ARG, "NaN weight");
+  return MSF_OK;
+}
+
+}  // namespace msf
