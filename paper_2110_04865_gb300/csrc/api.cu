@@ -392,18 +392,33 @@ bool one_shot_allowed() {
          o.sweep == 0 && o.round_limit >= 64 && o.jump_limit >= 64;
 }
 
-int one_shot(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const void *w, int wtype,
-             uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
+// Whether a call goes to the one-shot solvers: one graph, or graphs that all
+// fit one block each.
+bool one_shot_route(int32_t G, const int64_t *voff, const int64_t *eoff) {
+  if (!one_shot_allowed()) return false;
+  if (G == 1) return true;
+  for (int32_t g = 0; g < G; ++g)
+    if (!small_fits(voff[g + 1] - voff[g], eoff[g + 1] - eoff[g])) return false;
+  return true;
+}
+
+int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t *src, const int32_t *dst,
+             const void *w, int wtype, uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
+  const int64_t n = voff[G], m = eoff[G];
   int rc;
   Staged ss, sd, sw, om, ol, ot;
   if ((rc = ss.input(src, (size_t)m * 4, s)) || (rc = sd.input(dst, (size_t)m * 4, s)) ||
       (rc = sw.input(w, (size_t)m * 4, s)) || (rc = om.output(edge_mask, (size_t)m)) ||
-      (rc = ol.output(labels, (size_t)n * 4)) || (rc = ot.output(totals, 8))) {
+      (rc = ol.output(labels, (size_t)n * 4)) || (rc = ot.output(totals, (size_t)G * 8))) {
     cudaStreamSynchronize(s);  // copies already queued finish before their buffers return to the pool
     return rc;
   }
-  rc = solve_edges(n, m, (const int32_t *)ss.dev, (const int32_t *)sd.dev, (const uint32_t *)sw.dev, wtype,
-                   (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
+  const int32_t *u = (const int32_t *)ss.dev, *v = (const int32_t *)sd.dev;
+  const uint32_t *wd = (const uint32_t *)sw.dev;
+  if (G > 1 || small_single(n, m))
+    rc = solve_small(G, voff, eoff, n, m, u, v, wd, wtype, (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
+  else
+    rc = solve_edges(n, m, u, v, wd, wtype, (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
   if (rc) return rc;
   if ((rc = om.copy_back(s)) || (rc = ol.copy_back(s)) || (rc = ot.copy_back(s))) return rc;
   if (om.owned || ol.owned || ot.owned) MSF_CK(cudaStreamSynchronize(s));
@@ -454,8 +469,8 @@ int msf_compute_batched(int32_t G, const int64_t *voff, const int64_t *eoff, con
   if (m > 0 && (!src || !dst || !w)) return fail(MSF_ERR_INVALID_ARG, "NULL edge array");
   if (m > 0 && n == 0) return fail(MSF_ERR_INVALID_ARG, "edges given for an empty vertex set");
   cudaStream_t s = (cudaStream_t)stream;
-  if (G == 1 && one_shot_allowed()) {
-    const int rc = one_shot(n, m, src, dst, w, wtype, edge_mask, labels, totals, s);
+  if (one_shot_route(G, voff, eoff)) {
+    const int rc = one_shot(G, voff, eoff, src, dst, w, wtype, edge_mask, labels, totals, s);
     if (rc != SOLVE_NOT_RUN) return rc;
   }
   msf_graph *g = nullptr;

@@ -1,5 +1,6 @@
-// Device helpers shared by the end-of-run kernels: the long accumulators of
-// exact forest weights and the expansion of the forest bitmap into mask bytes.
+// Device helpers shared by the solvers and the end-of-run kernels: the long
+// accumulators of exact forest weights, thresholds of edge keys, and the
+// expansion of the forest bitmap into mask bytes.
 #pragma once
 
 #include "internal.cuh"
@@ -27,6 +28,40 @@ __device__ __forceinline__ void weight_bin(uint32_t ordw, int wtype, int *bin, l
   *bin = E ? (int)E : 1;
   *val = neg ? -sig : sig;
 }
+
+// A block's long accumulators of float32 weights (weight_bin) in shared memory:
+// 64-bit sums as two words, added with 32-bit shared atomics and a carry (a
+// 64-bit shared atomic is a compare-and-swap loop, and a block's weights share
+// few bins).  The low word is kept eight times, by lane, in eight banks: a
+// warp's equal bins then serialise four deep instead of thirty-two.
+struct BlockSums {
+  unsigned lo[256][8], hi[256];
+  __device__ void clear() {
+    for (int i = threadIdx.x; i < 256 * 8; i += blockDim.x) lo[i >> 3][i & 7] = 0;
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) hi[i] = 0;
+  }
+  __device__ __forceinline__ void add(uint32_t ordw) {
+    int bin;
+    long long val;
+    weight_bin(ordw, MSF_F32, &bin, &val);
+    const unsigned v = (unsigned)val;
+    const unsigned old = atomicAdd(&lo[bin][threadIdx.x & 7], v);
+    const unsigned h = (unsigned)((unsigned long long)val >> 32) + (old + v < old ? 1u : 0u);
+    if (h) atomicAdd(&hi[bin], h);
+  }
+  __device__ __forceinline__ void add_long(int bin, long long val) {
+    const unsigned v = (unsigned)val;
+    const unsigned old = atomicAdd(&lo[bin][0], v);
+    const unsigned h = (unsigned)((unsigned long long)val >> 32) + (old + v < old ? 1u : 0u);
+    if (h) atomicAdd(&hi[bin], h);
+  }
+  __device__ unsigned long long get(int b) const {
+    unsigned long long t = (unsigned long long)hi[b] << 32;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += lo[b][k];
+    return t;
+  }
+};
 
 // Unsigned big integer of 6 64-bit limbs.
 struct Big {
@@ -231,6 +266,55 @@ __device__ inline double combine_bins_warp(const long long *b, int wtype) {
     }
   }
   return round_difference(P, N);
+}
+
+// Whether a weight lies below a threshold key (weight tw, edge index te, te a
+// multiple of 128): one comparison per edge, with the edges of a batch of 128
+// all on one side of te.
+template <bool F32>
+struct Limit {
+  uint32_t at, under;  // largest weight below the threshold, for edges before and from te
+  int64_t te;
+  bool none;           // no weight lies below it from te on
+  uint32_t lim;
+  bool ok;
+  __device__ Limit(unsigned long long T) {
+    const uint32_t tw = (uint32_t)(T >> 32);
+    te = (int64_t)(uint32_t)T == 0xffffffffll ? (int64_t)1 << 40 : (int64_t)(uint32_t)T;
+    at = tw;
+    none = tw == 0;
+    under = tw - (none ? 0u : 1u);
+    if (F32) {  // the comparison is of floats (NaN: false)
+      at = from_ord(at);
+      under = none ? 0x7fffffffu : from_ord(under);
+    }
+  }
+  __device__ static uint32_t from_ord(uint32_t o) {
+    const uint32_t b = (o & 0x80000000u) ? o & 0x7fffffffu : ~o;
+    return (b << 1) > 0xff000000u ? ((b >> 31) ? 0x7fffffffu : 0x7f800000u) : b;
+  }
+  __device__ __forceinline__ void batch(int64_t e) {  // the batch of edges from e on
+    const bool before = e < te;
+    lim = before ? at : under;
+    ok = F32 || before || !none;
+  }
+  __device__ __forceinline__ bool below(uint32_t w) const {
+    return F32 ? __uint_as_float(w) <= __uint_as_float(lim) : (w <= lim && ok);
+  }
+};
+
+// Batches of 128 edges [lo, hi) through two register buffers in turn: a buffer
+// is loaded again once its batch is done, while the other's is worked on, and
+// none is copied to the other.
+template <class Q, class Load, class Body>
+__device__ __forceinline__ void stream2(int64_t lo, int64_t hi, Load load, Body body) {
+  Q a = load(lo), b = load(lo + 128);
+  for (int64_t k = lo; k < hi; k += 256) {
+    body(a, k);
+    a = load(k + 256);
+    if (k + 128 < hi) body(b, k + 128);
+    b = load(k + 384);
+  }
 }
 
 // 16 mask bytes from 16 bits: byte j = bit j (each nibble spread to the low

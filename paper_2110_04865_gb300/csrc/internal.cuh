@@ -186,6 +186,19 @@ void *pool_alloc(size_t bytes, int *err);  // err = MSF_OK / MSF_ERR_OOM
 void pool_free_after(void *p, cudaStream_t s);
 void pool_free(void *p);
 void pool_release_all();
+// A pool block given back at the end of a scope (after its work is done).
+struct PoolBlock {
+  void *p;
+  ~PoolBlock() { pool_free(p); }
+};
+// Pinned host memory of one call (its first 64 bytes zeroed), for a status that
+// a kernel writes and small tables that it reads in place.
+struct PinnedWords {
+  unsigned *p = nullptr;
+  size_t bytes = 0;
+  int take(size_t want);
+  ~PinnedWords();
+};
 
 // ---- device properties ---------------------------------------------------------
 int sm_count();
@@ -285,6 +298,16 @@ void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cuda
 constexpr int SOLVE_NOT_RUN = -1;
 int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const uint32_t *w, int wtype,
                 uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s);
+
+// small.cu
+// Forests of graphs that each fit in one SM's shared memory, one block per
+// graph: G graphs with host offsets, or one graph (G = 1, offsets unused).
+// Device pointers; any output may be NULL.  Synchronizes `s`.
+bool small_fits(int64_t n, int64_t m);
+bool small_single(int64_t n, int64_t m);  // one graph: faster so than by solve_edges
+int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, int64_t m, const int32_t *src,
+                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
+                cudaStream_t s);
 
 // exec.cu
 int enqueue_msf_graph(const DevState &hs, cudaStream_t s, const DevState **host_state);

@@ -155,6 +155,45 @@ void pool_free_after(void *p, cudaStream_t s) {
   g_pending.emplace_back(p, ev);
 }
 
+namespace {
+std::mutex g_pin_mu;
+std::vector<std::pair<unsigned *, size_t>> g_pin_free;
+constexpr size_t PIN_KEEP_BYTES = 1 << 20;  // larger blocks are not kept
+constexpr size_t PIN_KEEP = 32;             // blocks kept at most
+}  // namespace
+
+int PinnedWords::take(size_t want) {
+  {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    for (size_t i = g_pin_free.size(); i-- > 0 && !p;)
+      if (g_pin_free[i].second >= want) {
+        p = g_pin_free[i].first;
+        bytes = g_pin_free[i].second;
+        g_pin_free.erase(g_pin_free.begin() + (ptrdiff_t)i);
+      }
+  }
+  if (!p) {
+    size_t b = 4096;
+    while (b < want) b <<= 1;
+    MSF_CK(cudaHostAlloc((void **)&p, b, cudaHostAllocPortable | cudaHostAllocMapped));
+    bytes = b;
+  }
+  for (int i = 0; i < 16; ++i) p[i] = 0;
+  return MSF_OK;
+}
+
+PinnedWords::~PinnedWords() {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    if (bytes <= PIN_KEEP_BYTES && g_pin_free.size() < PIN_KEEP) {
+      g_pin_free.emplace_back(p, bytes);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
 void pool_release_all() {
   std::lock_guard<std::mutex> lk(g_pool_mu);
   for (auto &kv : g_free) {

@@ -45,8 +45,6 @@
 #include <cuda/atomic>
 
 #include <cstring>
-#include <mutex>
-#include <vector>
 
 #include "exact.cuh"
 #include "internal.cuh"
@@ -76,6 +74,8 @@ constexpr int64_t TWO_CLASSES = 1 << 22;
 // pass follows the chains itself, one barrier and about 5 us less per round
 // (R-MAT 16: 257 -> 199 us).
 constexpr unsigned long long SMALL = 1 << 17;
+// Edges or vertices per block: a call that does not fill the device.
+constexpr int64_t BLOCK_SHARE = 1024;
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
 struct Ctrl {
@@ -211,29 +211,6 @@ __device__ __forceinline__ bool table_offer(Table &t, int slot, unsigned long lo
   return false;
 }
 
-// The block's long accumulators of float32 weights (weight_bin): 64-bit sums as
-// two words, added with 32-bit shared atomics and a carry (a 64-bit shared
-// atomic is a compare-and-swap loop, and a warp's weights share few bins); the
-// low words four times over, by lane, to spread the equal bins of a warp.
-struct Sums {
-  unsigned lo[4][256], hi[256];
-  __device__ void clear() {
-    for (int i = threadIdx.x; i < 256; i += ET) lo[0][i] = lo[1][i] = lo[2][i] = lo[3][i] = hi[i] = 0;
-  }
-  __device__ __forceinline__ void add(uint32_t ordw) {
-    int bin;
-    long long val;
-    weight_bin(ordw, MSF_F32, &bin, &val);
-    const unsigned v = (unsigned)val;
-    const unsigned old = atomicAdd(&lo[threadIdx.x & 3][bin], v);
-    const unsigned h = (unsigned)((unsigned long long)val >> 32) + (old + v < old ? 1u : 0u);
-    if (h) atomicAdd(&hi[bin], h);
-  }
-  __device__ unsigned long long get(int b) const {
-    return ((unsigned long long)hi[b] << 32) + lo[0][b] + lo[1][b] + lo[2][b] + lo[3][b];
-  }
-};
-
 // Minimum pass over `cnt` entries of the warp from S, which end up at L (the
 // same place, or S lies further back in the region): with RELABEL the ends
 // become their roots first (their parents) and the entries inside a component
@@ -318,7 +295,7 @@ __device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const ui
 
 // Hooks along every entry that is the minimum of one of its ends (tie
 // breaking: of two roots that chose the same edge the smaller stays a root).
-__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, Sums &sums,
+__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, BlockSums &sums,
                                           unsigned long long &usum) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 4;
@@ -417,45 +394,9 @@ __device__ __forceinline__ Ends load_ends(const Args &A, int64_t e, int64_t hi) 
   return q;
 }
 
-// Whether a weight lies below a threshold key (weight tw, edge index te, te a
-// multiple of 128): one comparison per edge, with the edges of a batch of 128
-// all on one side of te.
-template <bool F32>
-struct Limit {
-  uint32_t at, under;  // largest weight below the threshold, for edges before and from te
-  int64_t te;
-  bool none;           // no weight lies below it from te on
-  uint32_t lim;
-  bool ok;
-  __device__ Limit(unsigned long long T) {
-    const uint32_t tw = (uint32_t)(T >> 32);
-    te = (int64_t)(uint32_t)T == 0xffffffffll ? (int64_t)1 << 40 : (int64_t)(uint32_t)T;
-    at = tw;
-    none = tw == 0;
-    under = tw - (none ? 0u : 1u);
-    if (F32) {  // the comparison is of floats (NaN: false)
-      at = from_ord(at);
-      under = none ? 0x7fffffffu : from_ord(under);
-    }
-  }
-  __device__ static uint32_t from_ord(uint32_t o) {
-    const uint32_t b = (o & 0x80000000u) ? o & 0x7fffffffu : ~o;
-    return (b << 1) > 0xff000000u ? ((b >> 31) ? 0x7fffffffu : 0x7f800000u) : b;
-  }
-  __device__ __forceinline__ void batch(int64_t e) {  // the batch of edges from e on
-    const bool before = e < te;
-    lim = before ? at : under;
-    ok = F32 || before || !none;
-  }
-  __device__ __forceinline__ bool below(uint32_t w) const {
-    return F32 ? __uint_as_float(w) <= __uint_as_float(lim) : (w <= lim && ok);
-  }
-};
-
 // First pass over the warp's edges [lo, hi): validation; the non-loop edges
 // below T0 go to the front of the warp's list, those from T0 to T1 to its back
-// (growing downwards from the region's end).  Two batches of edges per warp
-// are in flight.  The pass is bound by instruction issue, so an edge costs a
+// (growing downwards from the region's end).  The pass is bound by instruction issue, so an edge costs a
 // running maximum (the index check), a NaN test and one or two comparisons
 // until it is selected.
 template <bool VEC, bool F32>
@@ -471,12 +412,9 @@ __device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t h
   Limit<F32> l0(T0), l1(T1);
   uint32_t top = 0;  // largest index seen
   bool nan = false;
-  Quad q1 = load_quad<VEC>(A, lo + 4 * lane, hi), q2 = load_quad<VEC>(A, lo + 128 + 4 * lane, hi);
-  for (int64_t b = lo; b < hi; b += 128) {
+  auto load = [&](int64_t b) { return load_quad<VEC>(A, b + 4 * lane, hi); };  // (zeros past the end: self-loops)
+  auto body = [&](const Quad &q, int64_t b) {
     const int64_t e0 = b + 4 * lane;
-    const Quad q = q1;
-    q1 = q2;
-    q2 = load_quad<VEC>(A, e0 + 256, hi);  // (zeros past the end: self-loops)
     const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
     const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
     const uint32_t w[4] = {q.w.x, q.w.y, q.w.z, q.w.w};
@@ -499,7 +437,8 @@ __device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t h
       front += __popc(mf);
       back += __popc(m & ~mf);
     }
-  }
+  };
+  stream2<Quad>(lo, hi, load, body);
   err = (top >= n ? 1u : 0u) | (nan ? 2u : 0u);
   __syncwarp();
 }
@@ -517,12 +456,9 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
   const unsigned below = (1u << lane) - 1u;
   unsigned out = 0;
   if (lo >= hi) return 0;
-  Ends q1 = load_ends<VEC>(A, lo + 4 * lane, hi), q2 = load_ends<VEC>(A, lo + 128 + 4 * lane, hi);
-  for (int64_t b = lo; b < hi; b += 128) {
+  auto load = [&](int64_t b) { return load_ends<VEC>(A, b + 4 * lane, hi); };  // (zeros past the end: self-loops)
+  auto body = [&](const Ends &q, int64_t b) {
     const int64_t e0 = b + 4 * lane;
-    const Ends q = q1;
-    q1 = q2;
-    q2 = load_ends<VEC>(A, e0 + 256, hi);  // (zeros past the end: self-loops)
     int32_t u[4] = {q.s.x, q.s.y, q.s.z, q.s.w}, v[4] = {q.d.x, q.d.y, q.d.z, q.d.w};
     uint32_t bu[4], bv[4], w[4];
     bool on[4];
@@ -537,7 +473,7 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
       on[j] = !(__funnelshift_r(bu[j], bu[j], u[j]) & __funnelshift_r(bv[j], bv[j], v[j]) & 1u);
       any |= on[j];
     }
-    if (!__any_sync(FULL, any)) continue;
+    if (!__any_sync(FULL, any)) return;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       on[j] = on[j] && e0 + j < hi;
@@ -554,7 +490,8 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
             make_uint4((uint32_t)u[j], (uint32_t)v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], A.wtype));
       out += __popc(bal);
     }
-  }
+  };
+  stream2<Ends>(lo, hi, load, body);
   __syncwarp();
   return out;
 }
@@ -670,7 +607,7 @@ __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
 // when a heavy class follows) or on the heavy edges left (phase 1); the
 // results at the end.
 __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
-  __shared__ Sums sums;
+  __shared__ BlockSums sums;
   __shared__ long long sbins[256];
   __shared__ Table tab;
   __shared__ unsigned s_live;
@@ -940,31 +877,6 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   if (tid == 0) A.host[0] = *(volatile unsigned *)&C->err;
 }
 
-// Pinned words that the kernel writes its status into; a call takes one and
-// gives it back.
-std::mutex g_pin_mu;
-std::vector<unsigned *> g_pin_free;
-struct Pinned {
-  unsigned *p = nullptr;
-  int take() {
-    {
-      std::lock_guard<std::mutex> lk(g_pin_mu);
-      if (!g_pin_free.empty()) {
-        p = g_pin_free.back();
-        g_pin_free.pop_back();
-      }
-    }
-    if (!p) MSF_CK(cudaHostAlloc((void **)&p, 64, cudaHostAllocPortable | cudaHostAllocMapped));
-    p[0] = 0;
-    return MSF_OK;
-  }
-  ~Pinned() {
-    if (!p) return;
-    std::lock_guard<std::mutex> lk(g_pin_mu);
-    g_pin_free.push_back(p);
-  }
-};
-
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -983,8 +895,8 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   A.wtype = wtype;
   const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
                      reinterpret_cast<uintptr_t>(w)) & 15) == 0;
-  // blocks: one per 8192 edges or vertices, at most one per SM
-  int64_t want = ((m > n ? m : n) + 8191) / 8192;
+  // blocks: one per BLOCK_SHARE edges or vertices, at most one per SM
+  int64_t want = ((m > n ? m : n) + BLOCK_SHARE - 1) / BLOCK_SHARE;
   if (want < 1) want = 1;
   const int64_t cap = (int64_t)sm_count();
   const int blocks = (int)(want < cap ? want : cap);
@@ -1020,12 +932,9 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   int err = MSF_OK;
   char *base = (char *)pool_alloc(off, &err);
   if (err) return err;
-  struct Back {
-    void *p;
-    ~Back() { pool_free(p); }
-  } back{base};
-  Pinned pin;
-  if (int rc = pin.take()) return rc;
+  PoolBlock back{base};
+  PinnedWords pin;
+  if (int rc = pin.take(64)) return rc;
   pin.p[0] = 0x80000000u;  // not finished
   A.ctl = (Ctrl *)(base + o_ctl);
   A.p = (int32_t *)(base + o_p);
