@@ -61,6 +61,7 @@ constexpr int VOTES = 128;      // sampled edge ends for the giant component
 constexpr int TS_BITS = 11;     // slots of the block's table of minima
 constexpr int TS = 1 << TS_BITS;
 constexpr int HOPS = 16;        // hops of one settling pass
+constexpr int SHORT_CHAIN = 8;  // hops through L1 before a chain counts as long
 constexpr int ROUND_CAP = 64;   // Boruvka rounds at most (components at least halve)
 constexpr uint32_t CAND = 0x80000000u;  // list entry may be a minimum of one of its ends
 constexpr uint32_t LONG = 0x80000000u;  // listed root whose chain goes on
@@ -152,27 +153,30 @@ __device__ bool grid_barrier(Ctrl *c, int phase, unsigned &target) {
   return ok != 0;
 }
 
-// Root of x, whose parent y was read, by its chain; x then points to it.  Hooks
-// happen in other phases, so the roots do not change meanwhile, and a parent
-// read from L1 is an ancestor even when it is out of date.  A long chain goes
-// on in L2 and is halved for the threads behind.
+// Root of x, whose parent y was read, by its chain.  Hooks happen in other
+// phases, so the roots do not change meanwhile, and a parent read from L1 is an
+// ancestor even when it is out of date.  Short chains are left as they are (a
+// hub's many edges would all write its parent: 300 us of one pass over 88 000
+// edges); a long one goes on in L2, is halved for the threads behind, and x
+// then points to the root.
 __device__ __forceinline__ int32_t chase(int32_t *p, int32_t x, int32_t y) {
   if (y == x) return x;
-  const int32_t x0 = x, y0 = y;
+  const int32_t x0 = x;
   x = y;
   y = __ldca(p + x);
 #pragma unroll 1
-  for (int k = 0; k < 4 && y != x; ++k) {
+  for (int k = 0; k < SHORT_CHAIN && y != x; ++k) {
     x = y;
     y = __ldca(p + x);
   }
+  if (y == x) return x;
   while (y != x) {
     const int32_t z = ld_rel(p + y);
     if (z != y) st_rel(p + x, z);
     x = z;
     y = ld_rel(p + x);
   }
-  if (x != y0) st_rel(p + x0, x);
+  st_rel(p + x0, x);
   return x;
 }
 
