@@ -392,16 +392,6 @@ bool one_shot_allowed() {
          o.sweep == 0 && o.round_limit >= 64 && o.jump_limit >= 64;
 }
 
-// Whether a call goes to the one-shot solvers: one graph, or graphs that all
-// fit one block each.
-bool one_shot_route(int32_t G, const int64_t *voff, const int64_t *eoff) {
-  if (!one_shot_allowed()) return false;
-  if (G == 1) return true;
-  for (int32_t g = 0; g < G; ++g)
-    if (!small_fits(voff[g + 1] - voff[g], eoff[g + 1] - eoff[g])) return false;
-  return true;
-}
-
 int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t *src, const int32_t *dst,
              const void *w, int wtype, uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
   const int64_t n = voff[G], m = eoff[G];
@@ -415,11 +405,27 @@ int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t 
   }
   const int32_t *u = (const int32_t *)ss.dev, *v = (const int32_t *)sd.dev;
   const uint32_t *wd = (const uint32_t *)sw.dev;
-  if (G > 1 || small_single(n, m))
-    rc = solve_small(G, voff, eoff, n, m, u, v, wd, wtype, (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
-  else
-    rc = solve_edges(n, m, u, v, wd, wtype, (uint8_t *)om.dev, (int32_t *)ol.dev, (double *)ot.dev, s);
+  uint8_t *mk = (uint8_t *)om.dev;
+  int32_t *lb = (int32_t *)ol.dev;
+  double *tt = (double *)ot.dev;
+  unsigned status = 0;
+  if (G == 1) {
+    rc = small_single(n, m) ? solve_small(1, nullptr, voff, eoff, u, v, wd, wtype, mk, lb, tt, &status, s)
+                            : solve_edges(1, nullptr, voff, eoff, u, v, wd, wtype, mk, lb, tt, &status, s);
+  } else {
+    // a block each for the graphs that fit one, the others together
+    std::vector<int32_t> small, large;
+    for (int32_t g = 0; g < G; ++g)
+      (small_fits(voff[g + 1] - voff[g], eoff[g + 1] - eoff[g]) ? small : large).push_back(g);
+    rc = large.empty() ? MSF_OK
+                       : solve_edges((int32_t)large.size(), large.data(), voff, eoff, u, v, wd, wtype, mk, lb, tt,
+                                     &status, s);
+    if (rc == MSF_OK && !small.empty())
+      rc = solve_small((int32_t)small.size(), small.data(), voff, eoff, u, v, wd, wtype, mk, lb, tt, &status, s);
+  }
   if (rc) return rc;
+  if (status & 1u) return fail(MSF_ERR_INVALID_ARG, "vertex index out of range");
+  if (status & 2u) return fail(MSF_ERR_INVALID_ARG, "NaN weight");
   if ((rc = om.copy_back(s)) || (rc = ol.copy_back(s)) || (rc = ot.copy_back(s))) return rc;
   if (om.owned || ol.owned || ot.owned) MSF_CK(cudaStreamSynchronize(s));
   return MSF_OK;
@@ -469,7 +475,7 @@ int msf_compute_batched(int32_t G, const int64_t *voff, const int64_t *eoff, con
   if (m > 0 && (!src || !dst || !w)) return fail(MSF_ERR_INVALID_ARG, "NULL edge array");
   if (m > 0 && n == 0) return fail(MSF_ERR_INVALID_ARG, "edges given for an empty vertex set");
   cudaStream_t s = (cudaStream_t)stream;
-  if (one_shot_route(G, voff, eoff)) {
+  if (one_shot_allowed()) {
     const int rc = one_shot(G, voff, eoff, src, dst, w, wtype, edge_mask, labels, totals, s);
     if (rc != SOLVE_NOT_RUN) return rc;
   }

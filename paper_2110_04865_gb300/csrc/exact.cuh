@@ -298,10 +298,45 @@ struct Limit {
     lim = before ? at : under;
     ok = F32 || before || !none;
   }
+  __device__ __forceinline__ bool below(uint32_t w, int64_t e) const {  // of an edge on its own
+    if (F32) return __uint_as_float(w) <= __uint_as_float(e < te ? at : under);
+    return e < te ? w <= at : (w <= under && !none);
+  }
   __device__ __forceinline__ bool below(uint32_t w) const {
     return F32 ? __uint_as_float(w) <= __uint_as_float(lim) : (w <= lim && ok);
   }
 };
+
+// Four consecutive edges from index i on, of the edges [lo, hi) of the arrays
+// at src, dst, w; the others become self-loops of vertex 0.  vec: the arrays
+// are 16-byte aligned and i is a multiple of four.
+struct EdgeQuad {
+  int4 s, d;
+  uint4 w;
+};
+template <bool W>
+__device__ __forceinline__ EdgeQuad edge_quad(const int32_t *src, const int32_t *dst, const uint32_t *w, bool vec, int i,
+                                            int lo, int hi) {
+  EdgeQuad q;
+  q.s = q.d = make_int4(0, 0, 0, 0);
+  q.w = make_uint4(0u, 0u, 0u, 0u);
+  if (vec && i >= lo && i + 4 <= hi) {
+    q.s = *reinterpret_cast<const int4 *>(src + i);
+    q.d = *reinterpret_cast<const int4 *>(dst + i);
+    if (W) q.w = *reinterpret_cast<const uint4 *>(w + i);
+    return q;
+  }
+  int32_t *s = &q.s.x, *d = &q.d.x;
+  uint32_t *v = &q.w.x;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (i + j >= lo && i + j < hi) {
+      s[j] = src[i + j];
+      d[j] = dst[i + j];
+      if (W) v[j] = w[i + j];
+    }
+  return q;
+}
 
 // Batches of 128 edges [lo, hi) through two register buffers in turn: a buffer
 // is loaded again once its batch is done, while the other's is worked on, and

@@ -292,22 +292,25 @@ void launch_backward(int64_t m, int32_t G, const int64_t *eoff_d, const uint8_t 
 void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cudaStream_t s);
 
 // solve.cu
-// Forest of one graph from its edge list, without a CSR (pointers the device
-// can read; any output may be NULL).  Synchronizes `s`.  SOLVE_NOT_RUN: the
-// device cannot hold the kernel's blocks at once; the outputs are untouched.
+// Forest of one graph (which = NULL, K = 1) from its edge list without a CSR,
+// or of K graphs of a batch, `which` of those with the host offsets voff, eoff
+// (pointers the device can read; any output may be NULL).  Synchronizes `s`;
+// *status |= 1 for an index out of range, 2 for a NaN weight.  SOLVE_NOT_RUN:
+// the device cannot hold the kernel's blocks at once; the outputs are
+// untouched.
 constexpr int SOLVE_NOT_RUN = -1;
-int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const uint32_t *w, int wtype,
-                uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s);
+int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
+                unsigned *status, cudaStream_t s);
 
 // small.cu
-// Forests of graphs that each fit in one SM's shared memory, one block per
-// graph: G graphs with host offsets, or one graph (G = 1, offsets unused).
-// Device pointers; any output may be NULL.  Synchronizes `s`.
+// The same for graphs that each fit in one SM's shared memory (small_fits),
+// one block per graph.
 bool small_fits(int64_t n, int64_t m);
 bool small_single(int64_t n, int64_t m);  // one graph: faster so than by solve_edges
-int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, int64_t m, const int32_t *src,
+int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                cudaStream_t s);
+                unsigned *status, cudaStream_t s);
 
 // exec.cu
 int enqueue_msf_graph(const DevState &hs, cudaStream_t s, const DevState **host_state);

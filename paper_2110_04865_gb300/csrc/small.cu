@@ -40,10 +40,11 @@ struct SmallArgs {
   const uint32_t *w;
   int32_t wtype;
   int32_t vec;             // the three arrays are 16-byte aligned
-  const int64_t *voff, *eoff;  // offsets (pinned host memory, read in place), or NULL: one graph
+  const int64_t *voff, *eoff;  // [2 * block]: its graph's offsets (pinned host memory, read in place)
   const int32_t *order;    // graph of each block, or NULL
+  const int64_t *loff;     // first list entry of each block's graph, or NULL
   int64_t n, m;            // one graph
-  uint4 *list;             // kept edges, a graph's from its first batch on, 128 * graph further back
+  uint4 *list;             // kept edges
   uint8_t *mask;
   int32_t *labels;
   double *totals;
@@ -54,37 +55,6 @@ struct SmallArgs {
 __host__ __device__ inline size_t small_smem(int64_t n, int64_t m) {
   const int64_t nn = (n + 3) / 4 * 4;
   return (size_t)nn * 10 + (size_t)((m + 31) / 32 + 2) * 4;
-}
-
-// Four consecutive edges from index i on, of the edges [lo, hi) of the arrays
-// at src, dst, w; the others become self-loops of vertex 0.  vec: the arrays
-// are 16-byte aligned and i is a multiple of four.
-struct SQuad {
-  int4 s, d;
-  uint4 w;
-};
-template <bool W>
-__device__ __forceinline__ SQuad small_quad(const int32_t *src, const int32_t *dst, const uint32_t *w, bool vec, int i,
-                                            int lo, int hi) {
-  SQuad q;
-  q.s = q.d = make_int4(0, 0, 0, 0);
-  q.w = make_uint4(0u, 0u, 0u, 0u);
-  if (vec && i >= lo && i + 4 <= hi) {
-    q.s = *reinterpret_cast<const int4 *>(src + i);
-    q.d = *reinterpret_cast<const int4 *>(dst + i);
-    if (W) q.w = *reinterpret_cast<const uint4 *>(w + i);
-    return q;
-  }
-  int32_t *s = &q.s.x, *d = &q.d.x;
-  uint32_t *v = &q.w.x;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (i + j >= lo && i + j < hi) {
-      s[j] = src[i + j];
-      d[j] = dst[i + j];
-      if (W) v[j] = w[i + j];
-    }
-  return q;
 }
 
 // Light edges kept per vertex, for graphs of several times as many edges.
@@ -103,10 +73,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
   __shared__ unsigned long long s_usum, s_thresh;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned below = (1u << lane) - 1u;
-  const int g = A.order ? A.order[blockIdx.x] : (int)blockIdx.x;
-  const int64_t v0 = A.voff ? A.voff[g] : 0, e0 = A.eoff ? A.eoff[g] : 0;
-  const int n = (int)(A.voff ? A.voff[g + 1] - v0 : A.n);
-  const int64_t e1 = A.eoff ? A.eoff[g + 1] : A.m;
+  const int at = 2 * (int)blockIdx.x;
+  const int g = A.order ? A.order[blockIdx.x] : 0;
+  const int64_t v0 = A.order ? A.voff[at] : 0, e0 = A.order ? A.eoff[at] : 0;
+  const int n = (int)(A.order ? A.voff[at + 1] - v0 : A.n);
+  const int64_t e1 = A.order ? A.eoff[at + 1] : A.m;
   const int m = (int)(e1 - e0);
   const int nn = (n + 3) / 4 * 4;
   // a component's minimum: its smallest weight, then the smallest edge of that
@@ -358,11 +329,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     const int32_t *S = A.src + a0, *D = A.dst + a0;
     const uint32_t *W = A.w + a0;
     const bool vec = A.vec != 0;
-    L = A.list + a0 + lo + (int64_t)128 * g;
+    L = A.list + (A.loff ? A.loff[blockIdx.x] : 0) + lo;
     int cnt = 0;
     {
-      auto load = [&](int b) { return small_quad<true>(S, D, W, vec, b + 4 * lane, first, hi); };
-      auto body = [&](const SQuad &q, int b) {
+      auto load = [&](int b) { return edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi); };
+      auto body = [&](const EdgeQuad &q, int b) {
         const int i = b + 4 * lane;
         limit.batch(a0 + b);
         const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
@@ -380,7 +351,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
           cnt += __popc(bal);
         }
       };
-      stream2<SQuad>(lo, hi, load, body);
+      stream2<EdgeQuad>(lo, hi, load, body);
       __syncwarp();
     }
     if (invalid()) return;
@@ -388,8 +359,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     if (filter) {
       // the edges between components (the heavy ones: a light edge lies inside)
       cnt = 0;
-      auto load = [&](int b) { return small_quad<false>(S, D, W, vec, b + 4 * lane, first, hi); };
-      auto body = [&](const SQuad &q, int b) {
+      auto load = [&](int b) { return edge_quad<false>(S, D, W, vec, b + 4 * lane, first, hi); };
+      auto body = [&](const EdgeQuad &q, int b) {
         const int i = b + 4 * lane;
         const uint32_t u[4] = {p[q.s.x], p[q.s.y], p[q.s.z], p[q.s.w]};
         const uint32_t v[4] = {p[q.d.x], p[q.d.y], p[q.d.z], p[q.d.w]};
@@ -406,7 +377,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
           cnt += __popc(bal);
         }
       };
-      stream2<SQuad>(lo, hi, load, body);
+      stream2<EdgeQuad>(lo, hi, load, body);
       __syncwarp();
       rounds(cnt);
     }
@@ -531,11 +502,14 @@ bool small_fits(int64_t n, int64_t m) {
 // 235, (8000, 200000) 265 / 225, (4000, 200000) 176 / 230, (4000, 65536) 147 / 300.
 bool small_single(int64_t n, int64_t m) { return small_fits(n, m) && m + 8 * n <= ((int64_t)1 << 18); }
 
-// Forests of G graphs that all fit (small_fits); host offsets (NULL for one
-// graph of n vertices and m edges).  Synchronizes `s`.
-int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, int64_t m, const int32_t *src,
+// Forests of one graph (which = NULL), or of K graphs that fit (small_fits),
+// `which` of the graphs with the host offsets voff, eoff.  Synchronizes `s`;
+// *status: 1 = index out of range, 2 = NaN weight.
+int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                cudaStream_t s) {
+                unsigned *status, cudaStream_t s) {
+  const int64_t n = which ? 0 : voff[1], m = which ? 0 : eoff[1];
+  const int32_t G = which ? K : 1;
   SmallArgs A;
   std::memset(&A, 0, sizeof(A));
   A.src = src;
@@ -552,19 +526,22 @@ int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, 
   // pinned: status words, then the offsets and the blocks' graphs, which the
   // blocks read in place (a copy would cost a call more than their one read)
   PinnedWords pin;
-  if (int rc = pin.take(64 + (G > 1 ? (size_t)(G + 1) * 16 + (size_t)G * 4 : 0))) return rc;
+  if (int rc = pin.take(64 + (which ? (size_t)K * 44 : 0))) return rc;
   A.host = pin.p;
-  char *base = (char *)pool_alloc(((size_t)m + 128 * (size_t)G + 4096) * 16, &err);
+  int64_t entries = m + 256;
+  for (int32_t k = 0; which && k < K; ++k) entries += eoff[which[k] + 1] - eoff[which[k]] + 128;
+  char *base = (char *)pool_alloc((size_t)entries * 16, &err);
   if (err) return err;
   PoolBlock back{base};
   A.list = (uint4 *)base;
   int rc = MSF_OK;
-  if (G == 1) {
+  if (!which) {
     const size_t dyn = small_smem(n, m);
     rc = m <= 512 ? launch_small<256>(A, 1, dyn, s) : launch_small<1024>(A, 1, dyn, s);
   } else {
-    int64_t *hv = (int64_t *)(pin.p + 16), *he = hv + G + 1;
-    int32_t *order = (int32_t *)(he + G + 1);
+    // by block: vertex and edge offsets of its graph, its list, its number
+    int64_t *hv = (int64_t *)(pin.p + 16), *he = hv + 2 * K, *hl = he + 2 * K;
+    int32_t *order = (int32_t *)(hl + K);
     // graphs by falling size class
     int64_t count[42] = {0}, at[42], run = 0;
     size_t need[42] = {0};
@@ -574,23 +551,28 @@ int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, 
       while (((int64_t)1 << b) <= k) ++b;
       return b;
     };
-    for (int32_t g = 0; g < G; ++g) {
-      hv[g] = voff[g];
-      he[g] = eoff[g];
+    for (int32_t k = 0; k < K; ++k) {
+      const int32_t g = which[k];
       const int c = cls(g);
       ++count[c];
       const size_t d = small_smem(voff[g + 1] - voff[g], eoff[g + 1] - eoff[g]);
       if (d > need[c]) need[c] = d;
     }
-    hv[G] = voff[G];
-    he[G] = eoff[G];
     for (int c = 41; c >= 0; --c) {
       at[c] = run;
       run += count[c];
     }
-    for (int32_t g = 0; g < G; ++g) order[at[cls(g)]++] = g;
-    A.voff = hv;
-    A.eoff = he;
+    for (int32_t k = 0; k < K; ++k) order[at[cls(which[k])]++] = which[k];
+    int64_t entry = 0;
+    for (int32_t k = 0; k < K; ++k) {
+      const int32_t g = order[k];
+      hv[2 * k] = voff[g];
+      hv[2 * k + 1] = voff[g + 1];
+      he[2 * k] = eoff[g];
+      he[2 * k + 1] = eoff[g + 1];
+      hl[k] = entry;
+      entry += eoff[g + 1] - eoff[g] + 128;
+    }
     // one launch per block size, side by side: 1024 threads (one block per SM)
     // for graphs from 2^13 vertices and edges on (for all while every graph
     // has an SM), 512 from 2^11 on, 256 below
@@ -613,6 +595,9 @@ int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, 
     for (int t = 0; t < 3 && rc == MSF_OK; ++t) {
       if (blocks[t] == 0) continue;
       A.order = order + first;
+      A.voff = hv + 2 * first;
+      A.eoff = he + 2 * first;
+      A.loff = hl + first;
       first += blocks[t];
       cudaStream_t st = used ? fork.used[used - 1] : s;
       ++used;
@@ -627,8 +612,8 @@ int solve_small(int32_t G, const int64_t *voff, const int64_t *eoff, int64_t n, 
   if (rc) return rc;
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "forests of small graphs");
-  if (((volatile unsigned *)pin.p)[0]) return fail(MSF_ERR_INVALID_ARG, "vertex index out of range");
-  if (((volatile unsigned *)pin.p)[1]) return fail(MSF_ERR_INVALID_ARG, "NaN weight");
+  if (((volatile unsigned *)pin.p)[0]) *status |= 1u;
+  if (((volatile unsigned *)pin.p)[1]) *status |= 2u;
   return MSF_OK;
 }
 

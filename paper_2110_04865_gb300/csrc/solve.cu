@@ -105,7 +105,13 @@ struct Args {
   unsigned *front, *back;  // per warp: entries of the first and second class
   uint4 *list;          // (u, v, edge id, ordered weight), u | CAND
   uint32_t *mbits;
-  unsigned long long *bins;  // [256] long accumulators (zeroed with the control block)
+  // a batch (see Batch below); G = 0: one graph
+  int32_t G;
+  const int64_t *eL, *vL;  // [G + 1] first edge and vertex of each graph here
+  const int64_t *eA, *vA;  // [G] first edge and vertex of each graph in the call's arrays
+  const int32_t *id;       // [G] graph of the call
+  int32_t *giant;          // [G] root of each graph's giant component
+  unsigned long long *bins;  // [256] long accumulators (zeroed with the control block), [G][256] for a batch
   Ctrl *ctl;
   uint8_t *mask;
   int32_t *labels;
@@ -299,7 +305,7 @@ __device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const ui
 
 // Hooks along every entry that is the minimum of one of its ends (tie
 // breaking: of two roots that chose the same edge the smaller stays a root).
-__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, BlockSums &sums,
+__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, bool sum, BlockSums &sums,
                                           unsigned long long &usum) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 4;
@@ -330,12 +336,47 @@ __device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigne
       if (mu && (!mv || v < u)) A.p[u] = v;
       else A.p[v] = u;
       if (A.mbits) atomicOr(A.mbits + (x[j].z >> 5), 1u << (x[j].z & 31u));
-      if (A.totals) {
+      if (sum) {
         if (A.wtype == MSF_U32) usum += x[j].w;
         else sums.add(x[j].w);
       }
     }
   }
+}
+
+// A batch of graphs is solved as one graph whose edges and vertices are those
+// of its graphs, one after the other (eL, vL): positions there index parents,
+// lists and the bitmap, and order the edges of a graph as their own indices
+// do.  A warp's run of edges meets a few graphs; `f(g, x, k)` gets each piece:
+// graph g, its first position x and its k edges.
+template <class F>
+__device__ __forceinline__ void for_pieces(const Args &A, int64_t lo, int64_t hi, F f) {
+  if (lo >= hi) return;
+  int a = 0, b = A.G;  // eL[a] <= lo < eL[b]
+  while (b - a > 1) {
+    const int mid = (a + b) >> 1;
+    if (A.eL[mid] <= lo) a = mid;
+    else b = mid;
+  }
+  for (int64_t x = lo; x < hi; ++a) {
+    const int64_t end = A.eL[a + 1] < hi ? A.eL[a + 1] : hi;
+    if (end > x) f(a, x, (int)(end - x));
+    x = end;
+  }
+}
+// graph of vertex v, from a graph that is not behind it
+__device__ __forceinline__ int graph_from(const Args &A, int g, int64_t v) {
+  while (g + 1 < A.G && A.vL[g + 1] <= v) ++g;
+  return g;
+}
+__device__ __forceinline__ int graph_of_vertex(const Args &A, int64_t v) {
+  int a = 0, b = A.G;
+  while (b - a > 1) {
+    const int mid = (a + b) >> 1;
+    if (A.vL[mid] <= v) a = mid;
+    else b = mid;
+  }
+  return a;
 }
 
 // Four consecutive edges of a lane.
@@ -500,6 +541,103 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
   return out;
 }
 
+// The same passes over a batch, piece by piece (the thresholds' edge indices
+// are positions, compared edge by edge).
+template <bool F32>
+__device__ __forceinline__ void select_batch(const Args &A, bool vec, int64_t lo, int64_t hi, unsigned long long T0,
+                                             unsigned long long T1, uint4 *L, unsigned &front, unsigned &back,
+                                             unsigned &err) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  front = back = 0;
+  uint4 *LB = L + A.E - 1;
+  Limit<F32> l0(T0), l1(T1);
+  bool bad = false, nan = false;
+  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+    const int64_t a = A.eA[g] + (x - A.eL[g]), base = a & ~(int64_t)3;
+    const uint32_t vb = (uint32_t)A.vL[g], lim = (uint32_t)(A.vL[g + 1] - A.vL[g]);
+    const int first = (int)(a - base), end = first + k;
+    const int32_t *S = A.src + base, *D = A.dst + base;
+    const uint32_t *W = A.w + base;
+    auto load = [&](int64_t b) { return edge_quad<true>(S, D, W, vec, (int)b + 4 * lane, first, end); };
+    auto body = [&](const EdgeQuad &q, int64_t b) {
+      const int i = (int)b + 4 * lane;
+      const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
+      const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
+      const uint32_t w[4] = {q.w.x, q.w.y, q.w.z, q.w.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t e = x + (i + j - first);
+        bad |= max(u[j], v[j]) >= lim;
+        if (F32) nan |= __uint_as_float(w[j]) != __uint_as_float(w[j]);
+        const bool sel = u[j] != v[j] && l1.below(w[j], e);
+        const unsigned m = __ballot_sync(FULL, sel);
+        if (!m) continue;
+        const unsigned mf = __ballot_sync(FULL, sel && l0.below(w[j], e));
+        const bool fr = mf >> lane & 1u;
+        if (sel) {
+          uint4 *at = fr ? L + (front + __popc(mf & below)) : LB - (back + __popc(m & ~mf & below));
+          *at = make_uint4(u[j] + vb, v[j] + vb, (uint32_t)e, ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
+        }
+        front += __popc(mf);
+        back += __popc(m & ~mf);
+      }
+    };
+    stream2<EdgeQuad>(0, end, load, body);
+  });
+  err = (bad ? 1u : 0u) | (nan ? 2u : 0u);
+  __syncwarp();
+}
+
+template <bool SMEM>
+__device__ __forceinline__ unsigned filter_batch(const Args &A, bool vec, int64_t lo, int64_t hi, const uint32_t *bits,
+                                                 uint4 *L) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned out = 0;
+  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+    const int64_t a = A.eA[g] + (x - A.eL[g]), base = a & ~(int64_t)3;
+    const int32_t vb = (int32_t)A.vL[g];
+    const int first = (int)(a - base), end = first + k;
+    const int32_t *S = A.src + base, *D = A.dst + base;
+    const uint32_t *W = A.w + base;
+    auto load = [&](int64_t b) { return edge_quad<false>(S, D, W, vec, (int)b + 4 * lane, first, end); };
+    auto body = [&](const EdgeQuad &q, int64_t b) {
+      const int i = (int)b + 4 * lane;
+      int32_t u[4] = {q.s.x + vb, q.s.y + vb, q.s.z + vb, q.s.w + vb};
+      int32_t v[4] = {q.d.x + vb, q.d.y + vb, q.d.z + vb, q.d.w + vb};
+      uint32_t w[4];
+      bool on[4], any = false;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t bu = SMEM ? bits[u[j] >> 5] : __ldca(bits + (u[j] >> 5));
+        const uint32_t bv = SMEM ? bits[v[j] >> 5] : __ldca(bits + (v[j] >> 5));
+        on[j] = u[j] != v[j] && !(__funnelshift_r(bu, bu, u[j]) & __funnelshift_r(bv, bv, v[j]) & 1u);
+        any |= on[j];
+      }
+      if (!__any_sync(FULL, any)) return;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        w[j] = on[j] ? __ldcs(W + i + j) : 0u;
+        u[j] = on[j] ? __ldca(A.p + u[j]) : 0;
+        v[j] = on[j] ? __ldca(A.p + v[j]) : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool o = u[j] != v[j];
+        const unsigned bal = __ballot_sync(FULL, o);
+        if (o)
+          L[out + __popc(bal & below)] = make_uint4((uint32_t)u[j], (uint32_t)v[j], (uint32_t)(x + (i + j - first)),
+                                                    ord_weight_dev(w[j], A.wtype));
+        out += __popc(bal);
+      }
+    };
+    stream2<EdgeQuad>(0, end, load, body);
+  });
+  __syncwarp();
+  return out;
+}
+
 // The thresholds: the sample's keys (edge indices rounded down to a batch) of the two wanted ranks, found bit by bit
 // (one sample per thread, block 0).  The low half of a key, the edge index,
 // only matters where many samples share the threshold's weight.
@@ -509,7 +647,17 @@ __device__ void pick_thresholds(const Args &A) {
   const int64_t i = threadIdx.x;
   const uint32_t h = (uint32_t)i * 0x9E3779B1u;
   const int64_t e = i * A.m / SAMPLES + (int64_t)(((uint64_t)h * (uint64_t)step) >> 32);
-  const uint32_t w = ord_weight_dev(A.w[e], A.wtype);
+  int64_t ea = e;
+  if (A.G) {
+    int a = 0, b = A.G;
+    while (b - a > 1) {
+      const int mid = (a + b) >> 1;
+      if (A.eL[mid] <= e) a = mid;
+      else b = mid;
+    }
+    ea = A.eA[a] + (e - A.eL[a]);
+  }
+  const uint32_t w = ord_weight_dev(A.w[ea], A.wtype);
   const unsigned r0 = A.rank[0], r1 = A.rank[1];
   uint32_t w0 = 0, w1 = 0;
   for (int b = 31; b >= 0; --b) {
@@ -560,6 +708,26 @@ __device__ int32_t vote_giant(const Args &A) {
   return vote[best & 0xffffu];
 }
 
+// The same for every graph of a batch, a warp each (32 sampled ends).
+__device__ void vote_giants(const Args &A, int64_t warp, int64_t nwarps) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t g = warp; g < A.G; g += nwarps) {
+    const int64_t k = A.eL[g + 1] - A.eL[g], e = A.eA[g] + (int64_t)lane * k / 32;
+    int32_t x = -1;
+    if (k > 0) {
+      x = (int32_t)A.vL[g] + ((lane & 1) ? A.src[e] : A.dst[e]);
+      int32_t y = __ldca(A.p + x);
+      while (y != x) {
+        x = y;
+        y = __ldca(A.p + x);
+      }
+    }
+    const unsigned best = __reduce_max_sync(FULL, ((unsigned)__popc(__match_any_sync(FULL, x)) << 8) | (unsigned)lane);
+    x = __shfl_sync(FULL, x, (int)(best & 31u));
+    if (lane == 0) A.giant[g] = x;
+  }
+}
+
 // Parents, minima, root lists and the forest bitmap; the thresholds.
 __global__ void __launch_bounds__(ET, 1) k_prepare(Args A) {
   const int64_t tid = (int64_t)blockIdx.x * ET + threadIdx.x, nthr = (int64_t)gridDim.x * ET;
@@ -572,17 +740,19 @@ __global__ void __launch_bounds__(ET, 1) k_prepare(Args A) {
     const int64_t words = (A.m + 31) / 32 + 2;
     for (int64_t i = tid; i < words; i += nthr) A.mbits[i] = 0u;
   }
+  for (int64_t i = tid; i < (int64_t)A.G * 256; i += nthr) A.bins[i] = 0ull;
   if (A.classes > 1 && blockIdx.x == 0) pick_thresholds(A);
 }
 
-template <bool VEC, bool F32>
+template <bool VEC, bool F32, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_select(Args A) {
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
   const int64_t lo = warp * A.E, hi = lo + A.E < A.m ? lo + A.E : A.m;
   const unsigned long long T0 = A.classes > 1 ? A.ctl->thresh[0] : KEY_INF;
   const unsigned long long T1 = A.classes > 2 ? A.ctl->thresh[1] : KEY_INF;
   unsigned front, back, err = 0;
-  select_pass<VEC, F32>(A, lo, hi, T0, T1, A.list + lo, front, back, err);
+  if (BATCH) select_batch<F32>(A, VEC, lo, hi, T0, T1, A.list + lo, front, back, err);
+  else select_pass<VEC, F32>(A, lo, hi, T0, T1, A.list + lo, front, back, err);
   if (err) atomicOr(&A.ctl->err, err);
   if ((threadIdx.x & 31) == 0) {  // (an invalid edge ends the call: no list is used)
     A.front[warp] = front;
@@ -590,7 +760,7 @@ __global__ void __launch_bounds__(ET, 1) k_select(Args A) {
   }
 }
 
-template <bool VEC, bool SMEM>
+template <bool VEC, bool SMEM, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
   extern __shared__ uint32_t dyn_bits[];
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
@@ -602,14 +772,73 @@ __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
       for (int64_t i = threadIdx.x; i < words; i += ET) dyn_bits[i] = A.gbits[i];
       __syncthreads();
     }
-    front = filter_pass<VEC, SMEM>(A, lo, hi, SMEM ? dyn_bits : A.gbits, A.list + lo);
+    const uint32_t *bits = SMEM ? dyn_bits : A.gbits;
+    front = BATCH ? filter_batch<SMEM>(A, VEC, lo, hi, bits, A.list + lo)
+                  : filter_pass<VEC, SMEM>(A, lo, hi, bits, A.list + lo);
   }
   if ((threadIdx.x & 31) == 0) A.front[warp] = front;
+}
+
+// Mask bytes of the positions [lo, hi) of a batch, and the weights of the
+// forest edges among them into their graphs' accumulators: a piece's sums of
+// four exponents from its first forest weight's down are kept in registers.
+__device__ void batch_results(const Args &A, int64_t lo, int64_t hi) {
+  const int lane = threadIdx.x & 31;
+  constexpr int WIN = 4, U = 4;
+  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+    const int64_t a = A.eA[g] + (x - A.eL[g]);
+    if (A.mask) {
+      uint8_t *mask = A.mask + a;
+      const int head = (int)((16 - (reinterpret_cast<uintptr_t>(mask) & 15)) & 15);
+      const int h = head < k ? head : k, nq = (k - h) >> 4;
+      uint4 *q = reinterpret_cast<uint4 *>(mask + h);
+      auto bit = [&](int i) { return (uint8_t)((A.mbits[(x + i) >> 5] >> ((x + i) & 31)) & 1u); };
+      for (int i = lane; i < h; i += 32) mask[i] = bit(i);
+      for (int i = lane; i < nq; i += 32) q[i] = spread16(bits16(A.mbits, x + h + ((int64_t)i << 4)));
+      for (int i = h + (nq << 4) + lane; i < k; i += 32) mask[i] = bit(i);
+    }
+    if (!A.totals) return;
+    const uint32_t *W = A.w + a;
+    unsigned long long *bins = A.bins + (int64_t)g * 256;
+    long long acc[WIN];
+#pragma unroll
+    for (int i = 0; i < WIN; ++i) acc[i] = 0;
+    int top = -1;
+    for (int b0 = 0; b0 < k; b0 += 32 * U) {
+      bool on[U];
+      uint32_t w[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const int i = b0 + j * 32 + lane;
+        on[j] = i < k && ((A.mbits[(x + i) >> 5] >> ((x + i) & 31)) & 1u);
+        w[j] = on[j] ? W[i] : 0u;
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        int bin = 0;
+        long long val = 0;
+        if (on[j]) weight_bin(ord_weight_dev(w[j], A.wtype), A.wtype, &bin, &val);
+        if (top < 0 && __any_sync(FULL, on[j])) top = __reduce_max_sync(FULL, on[j] && bin < 255 ? bin : 0);
+        const int d = top - bin;
+        const bool in = on[j] && d >= 0 && d < WIN;
+#pragma unroll
+        for (int i = 0; i < WIN; ++i) acc[i] += in && d == i ? val : 0;
+        if (on[j] && !in) atomicAdd(bins + bin, (unsigned long long)val);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < WIN; ++i) {
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) acc[i] += __shfl_xor_sync(FULL, acc[i], d);
+      if (lane == 0 && acc[i]) atomicAdd(bins + (top - i), (unsigned long long)acc[i]);
+    }
+  });
 }
 
 // The rounds on the light classes (phase 0; the bitmap of the giant component
 // when a heavy class follows) or on the heavy edges left (phase 1); the
 // results at the end.
+template <bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   __shared__ BlockSums sums;
   __shared__ long long sbins[256];
@@ -729,6 +958,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   auto flatten = [&](bool bits, int32_t giant) -> bool {
     constexpr int U = 4;
     unsigned out = 0;
+    int gv = BATCH && bits && vlo < vhi ? graph_of_vertex(A, vlo) : 0;
     for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
       int32_t x[U], y[U];
 #pragma unroll
@@ -752,6 +982,10 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
         if (root) V[out + __popc(mr & below)] = a;
         out += __popc(mr);
         if (bits) {
+          if (BATCH && v < vhi) {
+            gv = graph_from(A, gv, v);
+            giant = A.giant[gv];
+          }
           const unsigned mg = __ballot_sync(FULL, v < vhi && a == giant);
           if (lane == 0 && v < vhi) A.gbits[v >> 5] = mg;
         }
@@ -769,7 +1003,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     unsigned long long live = total_live(cnt);
     for (int k = 0; k < ROUND_CAP && live; ++k) {
       const bool small = live <= SMALL;
-      hook_pass(A, L, cnt, small, sums, usum);
+      hook_pass(A, L, cnt, small, !BATCH && A.totals, sums, usum);
       if (!grid_barrier(C, phase, target)) return false;
       if (!small) {
         if (!settle_roots()) return false;
@@ -793,11 +1027,15 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   }
   const bool last = phase == 1 || A.classes < 3;
   if (!last) {
-    flatten(true, vote_giant(A));
+    if (BATCH) {
+      vote_giants(A, warp, nthr >> 5);
+      if (!grid_barrier(C, phase, target)) return;
+    }
+    flatten(true, BATCH ? 0 : vote_giant(A));
     if (lane == 0) A.back[warp] = vc;
   }
-  // the forest's weight so far
-  if (A.totals) {
+  // the forest's weight so far (a batch: from the bitmap, at the end)
+  if (!BATCH && A.totals) {
     if (A.wtype == MSF_U32) {
 #pragma unroll
       for (int d = 16; d >= 1; d >>= 1) usum += __shfl_xor_sync(FULL, usum, d);
@@ -846,7 +1084,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     }
   }
   if (!grid_barrier(C, phase, target)) return;
-  if (A.totals && blockIdx.x == 0) {
+  if (!BATCH && A.totals && blockIdx.x == 0) {
     for (int i = threadIdx.x; i < 256; i += ET) sbins[i] = (long long)ld_rel64(A.bins + i);
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -855,6 +1093,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     }
   }
   if (A.labels) {
+    int gv = BATCH && vlo < vhi ? graph_of_vertex(A, vlo) : 0;
     for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
       int32_t x[U];
       unsigned b[U];
@@ -864,8 +1103,30 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
       for (int j = 0; j < U; ++j) b[j] = __ldca(reinterpret_cast<const unsigned *>(A.r + x[j]));
 #pragma unroll
       for (int j = 0; j < U; ++j)
-        if (v0 + j * 32 + lane < vhi) A.labels[v0 + j * 32 + lane] = (int32_t)(b[j] < (unsigned)x[j] ? b[j] : (unsigned)x[j]);
+        if (v0 + j * 32 + lane < vhi) {
+          const int64_t v = v0 + j * 32 + lane;
+          const int32_t least = (int32_t)min(b[j], (unsigned)x[j]);
+          if (BATCH) {
+            gv = graph_from(A, gv, v);
+            A.labels[A.vA[gv] + (v - A.vL[gv])] = least - (int32_t)A.vL[gv];
+          } else {
+            A.labels[v] = least;
+          }
+        }
     }
+  }
+  if (BATCH) {
+    batch_results(A, warp * A.E, warp * A.E + A.E < A.m ? warp * A.E + A.E : A.m);
+    if (A.totals) {
+      if (!grid_barrier(C, phase, target)) return;
+      // a warp per graph rounds its total
+      for (int64_t g = warp; g < A.G; g += nthr >> 5) {
+        const double t = combine_bins_warp(reinterpret_cast<const long long *>(A.bins) + g * 256, A.wtype);
+        if (lane == 0) A.totals[A.id[g]] = t;
+      }
+    }
+    if (tid == 0) A.host[0] = *(volatile unsigned *)&C->err;
+    return;
   }
   if (A.mask) {
     const int64_t m = A.m;
@@ -885,10 +1146,22 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
-// Forest of one graph from its edge list (pointers the device can read).  Any
-// output may be NULL.  Synchronizes `s`.
-int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, const uint32_t *w, int wtype,
-                uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s) {
+// Forest of one graph from its edge list, or of K graphs of a batch, `which` of
+// the graphs with the host offsets voff, eoff (pointers the device can read).
+// Any output may be NULL.  Synchronizes `s`; *status: 1 = index out of range,
+// 2 = NaN weight.
+int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
+                unsigned *status, cudaStream_t s) {
+  int64_t n = 0, m = 0;
+  if (!which) {
+    n = voff[1];
+    m = eoff[1];
+  }
+  for (int32_t k = 0; which && k < K; ++k) {
+    n += voff[which[k] + 1] - voff[which[k]];
+    m += eoff[which[k] + 1] - eoff[which[k]];
+  }
   Args A;
   std::memset(&A, 0, sizeof(A));
   A.n = n;
@@ -928,6 +1201,9 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   };
   static_assert(sizeof(Ctrl) <= 256, "control block");
   const size_t ctl_bytes = 256 + 256 * 8;  // control block, long accumulators
+  const size_t tab_bytes = which ? (size_t)(K + 1) * 32 + (size_t)K * 4 : 0;  // eL, vL, eA, vA, id
+  const size_t o_tab = place(tab_bytes), o_giant = place((size_t)(which ? K : 0) * 4);
+  const size_t o_bbins = place((size_t)(which ? K : 0) * 256 * 8);
   const size_t o_ctl = place(ctl_bytes), o_p = place((size_t)(n + 1) * 4), o_r = place((size_t)(n + 1) * 8);
   const size_t o_roots = place((size_t)(n + 1) * 4), o_gbits = place(bit_bytes);
   const size_t o_bits = place(((size_t)(m + 31) / 32 + 2) * 4);
@@ -938,7 +1214,7 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   if (err) return err;
   PoolBlock back{base};
   PinnedWords pin;
-  if (int rc = pin.take(64)) return rc;
+  if (int rc = pin.take(64 + tab_bytes)) return rc;
   pin.p[0] = 0x80000000u;  // not finished
   A.ctl = (Ctrl *)(base + o_ctl);
   A.p = (int32_t *)(base + o_p);
@@ -954,23 +1230,56 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   A.labels = labels;
   A.totals = totals;
   A.host = pin.p;
+  if (which) {
+    int64_t *t = (int64_t *)(pin.p + 16);
+    int32_t *ids = (int32_t *)(t + 4 * (K + 1));
+    int64_t *eL = t, *vL = t + (K + 1), *eA = t + 2 * (K + 1), *vA = t + 3 * (K + 1);
+    eL[0] = vL[0] = 0;
+    for (int32_t k = 0; k < K; ++k) {
+      const int32_t g = which[k];
+      eL[k + 1] = eL[k] + (eoff[g + 1] - eoff[g]);
+      vL[k + 1] = vL[k] + (voff[g + 1] - voff[g]);
+      eA[k] = eoff[g];
+      vA[k] = voff[g];
+      ids[k] = g;
+    }
+    eA[K] = vA[K] = 0;
+    int64_t *d = (int64_t *)(base + o_tab);
+    MSF_CK(cudaMemcpyAsync(d, t, tab_bytes, cudaMemcpyHostToDevice, s));
+    A.G = K;
+    A.eL = d;
+    A.vL = d + (K + 1);
+    A.eA = d + 2 * (K + 1);
+    A.vA = d + 3 * (K + 1);
+    A.id = (int32_t *)(d + 4 * (K + 1));
+    A.giant = (int32_t *)(base + o_giant);
+    A.bins = (unsigned long long *)(base + o_bbins);
+  }
   MSF_CK(cudaMemsetAsync(A.ctl, 0, ctl_bytes, s));
   k_prepare<<<blocks, ET, 0, s>>>(A);
-  void (*select)(Args) = wtype == MSF_F32 ? (vec ? k_select<true, true> : k_select<false, true>)
-                                          : (vec ? k_select<true, false> : k_select<false, false>);
+  const bool f32 = wtype == MSF_F32;
+  void (*select)(Args) =
+      which ? (f32 ? (vec ? k_select<true, true, true> : k_select<false, true, true>)
+                   : (vec ? k_select<true, false, true> : k_select<false, false, true>))
+            : (f32 ? (vec ? k_select<true, true, false> : k_select<false, true, false>)
+                   : (vec ? k_select<true, false, false> : k_select<false, false, false>));
+  const void *rounds = which ? (const void *)k_rounds<true> : (const void *)k_rounds<false>;
   select<<<blocks, ET, 0, s>>>(A);
   int phase = 0;
   void *args[] = {&A, &phase};
-  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
+  cudaError_t e = cudaLaunchCooperativeKernel(rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
   if (e == cudaSuccess && A.classes > 2) {
-    void (*filter)(Args) = A.smem_bits ? (vec ? k_filter<true, true> : k_filter<false, true>)
-                                       : (vec ? k_filter<true, false> : k_filter<false, false>);
+    void (*filter)(Args) =
+        which ? (A.smem_bits ? (vec ? k_filter<true, true, true> : k_filter<false, true, true>)
+                             : (vec ? k_filter<true, false, true> : k_filter<false, false, true>))
+              : (A.smem_bits ? (vec ? k_filter<true, true, false> : k_filter<false, true, false>)
+                             : (vec ? k_filter<true, false, false> : k_filter<false, false, false>));
     if (A.smem_bits)
       e = cudaFuncSetAttribute(filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BITS);
     if (e == cudaSuccess) {
       filter<<<blocks, ET, dyn, s>>>(A);
       phase = 1;
-      e = cudaLaunchCooperativeKernel((const void *)k_rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
+      e = cudaLaunchCooperativeKernel(rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
     }
   }
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // (a share of the device that holds fewer blocks)
@@ -984,8 +1293,7 @@ int solve_edges(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, co
   if (e != cudaSuccess) return cuda_fail(e, "forest of an edge list");
   const unsigned st = *(volatile unsigned *)pin.p;
   if (st & 0x80000000u) return fail(MSF_ERR_CHECK, "device consistency check failed");
-  if (st & 1u) return fail(MSF_ERR_INVALID_ARG, "vertex index out of range");
-  if (st & 2u) return fail(MSF_ERR_INVALID_ARG, "NaN weight");
+  *status |= st;
   return MSF_OK;
 }
 
