@@ -108,10 +108,10 @@ int msf_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *total
  *
  * Graphs that each fit in one SM's shared memory (about 10 bytes a vertex and
  * a bit an edge: some 20 000 vertices) are solved side by side, one thread
- * block each; one larger graph (G = 1, the one-shot form of build, compute and
- * free) is solved from its edge list without a CSR; a batch with larger graphs
- * is stored as one disjoint union and solved by one launch of the round loop.
- * The forest, labels and total are the same, since they are unique.  An option
+ * block each; the larger ones (with G = 1 the one-shot form of build, compute
+ * and free) are solved together from their edge lists without a CSR.  The
+ * forest, labels and total are those of the round loop over the disjoint union,
+ * since they are unique.  An option
  * that asks for a schedule, a builder, a kernel form, the host-driven loop, or
  * a round or jump limit below its default always selects the round loop.
  *   voff, eoff  HOST int64[G+1] vertex and edge offsets, voff[0] = eoff[0] = 0,

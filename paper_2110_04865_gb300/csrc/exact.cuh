@@ -342,9 +342,9 @@ __device__ __forceinline__ EdgeQuad edge_quad(const int32_t *src, const int32_t 
 // is loaded again once its batch is done, while the other's is worked on, and
 // none is copied to the other.
 template <class Q, class Load, class Body>
-__device__ __forceinline__ void stream2(int64_t lo, int64_t hi, Load load, Body body) {
+__device__ __forceinline__ void stream2(int lo, int hi, Load load, Body body) {
   Q a = load(lo), b = load(lo + 128);
-  for (int64_t k = lo; k < hi; k += 256) {
+  for (int k = lo; k < hi; k += 256) {
     body(a, k);
     a = load(k + 256);
     if (k + 128 < hi) body(b, k + 128);

@@ -25,9 +25,9 @@
 // edge inside a component of the lighter edges' forest is not, so every step
 // is exact.
 //
-// Every warp owns a contiguous range of the edges and a region of the kept
-// list of the same capacity: it fills, reads, relabels and compacts its own
-// region in place, so the lists need no global counters and cannot overflow.
+// Every warp owns pages of the edges and a list of the same capacity in the
+// same pages: it fills, reads, relabels and compacts its own list in place, so
+// the lists need no global counters and cannot overflow.
 // The rounds kernel is cooperative, one block of 1024 threads per SM; its
 // phases meet at a grid barrier (about 2 us, bounded wait), which costs less
 // than the kernel boundaries and conditional nodes of a graph loop (about 60
@@ -60,6 +60,7 @@ constexpr int SAMPLES = 1024;   // sampled weights for the thresholds
 constexpr int VOTES = 128;      // sampled edge ends for the giant component
 constexpr int TS_BITS = 11;     // slots of the block's table of minima
 constexpr int TS = 1 << TS_BITS;
+constexpr unsigned TABLE_HITS = 16;  // of a batch's 256 ends: below, the table is not worth its instructions
 constexpr int HOPS = 16;        // hops of one settling pass
 constexpr int SHORT_CHAIN = 8;  // hops through L1 before a chain counts as long
 constexpr int ROUND_CAP = 64;   // Boruvka rounds at most (components at least halve)
@@ -77,6 +78,12 @@ constexpr int64_t TWO_CLASSES = 1 << 22;
 constexpr unsigned long long SMALL = 1 << 17;
 // Edges or vertices per block: a call that does not fill the device.
 constexpr int64_t BLOCK_SHARE = 1024;
+// Pages (see Pages) of 2^PAGE places at most, and smaller where a warp would get
+// fewer than EVEN of them (its share is even to one page).  4096 graphs of 20 M
+// edges: one range per warp 8.56 ms, pages of 128 7.0, by this rule 6.05, with
+// EVEN 4 6.18, with longer pages 6.12; R-MAT and lattice graphs 1-5 % faster
+// than with ranges.
+constexpr int PAGE = 10, EVEN = 16;
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
 struct Ctrl {
@@ -95,8 +102,7 @@ struct Args {
   int32_t classes;      // 1 = every edge in the first class, 2 = none heavy, 3
   int32_t second;       // there is a second class
   int32_t smem_bits;    // the giant component's bitmap fits in shared memory
-  int64_t E;            // edges per warp region (a multiple of 128)
-  int64_t VE;           // vertices per warp region (a multiple of 128)
+  int32_t es, vs;       // pages of 2^es edges and 2^vs vertices (see Pages)
   unsigned rank[2];     // the thresholds' ranks among SAMPLES
   int32_t *p;
   unsigned long long *r;
@@ -110,6 +116,7 @@ struct Args {
   const int64_t *eL, *vL;  // [G + 1] first edge and vertex of each graph here
   const int64_t *eA, *vA;  // [G] first edge and vertex of each graph in the call's arrays
   const int32_t *id;       // [G] graph of the call
+  int32_t *eg, *vg;        // graph of each page's first edge and first vertex
   int32_t *giant;          // [G] root of each graph's giant component
   unsigned long long *bins;  // [256] long accumulators (zeroed with the control block), [G][256] for a batch
   Ctrl *ctl;
@@ -129,6 +136,28 @@ __device__ __forceinline__ unsigned long long ld_rel64(const unsigned long long 
   return cuda::atomic_ref<unsigned long long, cuda::thread_scope_device>(*const_cast<unsigned long long *>(a))
       .load(cuda::memory_order_relaxed);
 }
+
+// Edges and vertices are dealt to the warps in pages: warp w of W takes pages
+// w, w + W, ..., so that all warps work on one window of the arrays at a time
+// (an input with locality -- a lattice, a batch -- then keeps the parents and
+// minima it gathers in L2; with one contiguous range per warp every range's
+// vicinity is live at once).  `at(i)` is the i-th of the warp's elements, in
+// order; `cap` counts the places of its pages, `len` the elements below total.
+struct Pages {
+  uint32_t s, w, W, cap, len;
+  __device__ Pages(int64_t total, int32_t shift, int64_t warp, int64_t warps)
+      : s((uint32_t)shift), w((uint32_t)warp), W((uint32_t)warps) {
+    const int64_t pages = (total + ((int64_t)1 << s) - 1) >> s;
+    const int64_t mine = warp < pages ? (pages - warp + warps - 1) / warps : 0;
+    cap = (uint32_t)(mine << s);
+    len = cap;
+    if (mine > 0 && (pages - 1) % warps == warp) len -= (uint32_t)((pages << s) - total);  // the last page
+  }
+  __device__ __forceinline__ uint32_t page(uint32_t i) const { return (i >> s) * W + w; }
+  __device__ __forceinline__ int64_t at(uint32_t i) const {
+    return ((int64_t)page(i) << s) + (i & ((1u << s) - 1u));
+  }
+};
 
 // All blocks meet; false (everywhere, sooner or later) when a wait ran out.
 __device__ bool grid_barrier(Ctrl *c, int phase, unsigned &target) {
@@ -200,10 +229,12 @@ __device__ __forceinline__ void table_clear(Table &t) {
     t.val[i] = KEY_INF;
   }
 }
-// The table's slot for a root, or -1 when another root holds it.
-__device__ __forceinline__ int table_slot(Table &t, int32_t root) {
+// The table's slot for a root, or -1 when another root holds it; `hit`: the
+// root held it already.
+__device__ __forceinline__ int table_slot(Table &t, int32_t root, bool &hit) {
   const int slot = (int)(((uint32_t)root * 0x9E3779B1u) >> (32 - TS_BITS));
   int k = *(volatile int32_t *)(t.key + slot);
+  hit = k == root;
   if (k == -1) {
     k = atomicCAS(t.key + slot, -1, root);
     if (k == -1) k = root;
@@ -221,18 +252,21 @@ __device__ __forceinline__ bool table_offer(Table &t, int slot, unsigned long lo
   return false;
 }
 
-// Minimum pass over `cnt` entries of the warp from S, which end up at L (the
-// same place, or S lies further back in the region): with RELABEL the ends
-// become their roots first (their parents) and the entries inside a component
-// are dropped.  Every end's minimum is lowered to the entry's key; an entry that
-// lowered one is marked CAND (the final minimum did).  Returns the entries
-// left.
-template <bool RELABEL, bool CHASE = false>
-__device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const uint4 *S, uint4 *L, unsigned cnt) {
+// Minimum pass over `cnt` entries of the warp's list from place `from` on,
+// which end up at its front: with RELABEL the ends become their roots first
+// (their parents) and the entries inside a component are dropped.  Every end's
+// minimum is lowered to the entry's key; it is read first, and only an entry
+// that was below it is marked CAND (the final minimum is; lowering them unread
+// took R-MAT 26 from 23 to 31 ms).  A warp leaves the block's table alone once
+// few of its ends are found there (many small graphs: 9.0 -> 8.6 ms).  Returns
+// the entries left.
+template <bool RELABEL, bool CHASE>
+__device__ __noinline__ unsigned min_pass(const Args &A, Table &tab, const Pages P, unsigned from, unsigned cnt) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   constexpr int U = 4;
   unsigned out = 0;
+  bool use = true;
   for (unsigned b0 = 0; b0 < cnt; b0 += 32 * U) {
     uint4 x[U];
     bool on[U];
@@ -241,7 +275,7 @@ __device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const ui
     for (int j = 0; j < U; ++j) {
       const unsigned i = b0 + j * 32 + lane;
       on[j] = i < cnt;
-      x[j] = on[j] ? S[i] : make_uint4(0u, 0u, 0u, 0u);
+      x[j] = on[j] ? A.list[P.at(from + i)] : make_uint4(0u, 0u, 0u, 0u);
       u[j] = (int32_t)(x[j].x & ~CAND);
       v[j] = (int32_t)x[j].y;
     }
@@ -263,39 +297,55 @@ __device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const ui
 #pragma unroll
       for (int j = 0; j < U; ++j) on[j] = on[j] && u[j] != v[j];
     }
-    // ends in the table; the others read their global minimum
-    bool cand[U];
-    unsigned long long ru[U], rv[U];
+    unsigned cand = 0u;
+    unsigned gu = 0, gv = 0;  // entries whose ends go to r directly
+    if (use) {
+      unsigned hits = 0;
 #pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
-      cand[j] = false;
-      ru[j] = rv[j] = 0ull;
-      if (on[j]) {
-        const int su = table_slot(tab, u[j]), sv = table_slot(tab, v[j]);
-        if (su < 0) ru[j] = ld_rel64(A.r + u[j]);
-        else cand[j] |= table_offer(tab, su, key);
-        if (sv < 0) rv[j] = ld_rel64(A.r + v[j]);
-        else cand[j] |= table_offer(tab, sv, key);
+      for (int j = 0; j < U; ++j) {
+        if (!on[j]) continue;
+        const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
+        bool hu, hv;
+        const int su = table_slot(tab, u[j], hu), sv = table_slot(tab, v[j], hv);
+        hits += (hu ? 1u : 0u) + (hv ? 1u : 0u);
+        if (su < 0) gu |= 1u << j;
+        else if (table_offer(tab, su, key)) cand |= 1u << j;
+        if (sv < 0) gv |= 1u << j;
+        else if (table_offer(tab, sv, key)) cand |= 1u << j;
       }
+      use = __reduce_add_sync(FULL, hits) >= TABLE_HITS;
+    } else {
+#pragma unroll
+      for (int j = 0; j < U; ++j)
+        if (on[j]) gu |= 1u << j;
+      gv = gu;
+    }
+    {
+      unsigned long long ru[U], rv[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        ru[j] = gu >> j & 1u ? ld_rel64(A.r + u[j]) : 0ull;
+        rv[j] = gv >> j & 1u ? ld_rel64(A.r + v[j]) : 0ull;
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
+        if (key >= ru[j]) gu &= ~(1u << j);
+        if (key >= rv[j]) gv &= ~(1u << j);
+      }
+      cand |= gu | gv;
     }
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
-      if (key < ru[j]) {
-        atomicMin(A.r + u[j], key);
-        cand[j] = true;
-      }
-      if (key < rv[j]) {
-        atomicMin(A.r + v[j], key);
-        cand[j] = true;
-      }
+      if (gu >> j & 1u) atomicMin(A.r + u[j], key);
+      if (gv >> j & 1u) atomicMin(A.r + v[j], key);
     }
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const unsigned bal = __ballot_sync(FULL, on[j]);
       const unsigned at = out + __popc(bal & below);
-      if (on[j]) L[at] = make_uint4((uint32_t)u[j] | (cand[j] ? CAND : 0u), (uint32_t)v[j], x[j].z, x[j].w);
+      if (on[j]) A.list[P.at(at)] = make_uint4((uint32_t)u[j] | (cand >> j & 1u ? CAND : 0u), (uint32_t)v[j], x[j].z, x[j].w);
       out += __popc(bal);
     }
   }
@@ -305,7 +355,7 @@ __device__ __forceinline__ unsigned min_pass(const Args &A, Table &tab, const ui
 
 // Hooks along every entry that is the minimum of one of its ends (tie
 // breaking: of two roots that chose the same edge the smaller stays a root).
-__device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigned cnt, bool small, bool sum, BlockSums &sums,
+__device__ __noinline__ void hook_pass(const Args &A, const Pages P, unsigned cnt, bool small, bool sum, BlockSums &sums,
                                           unsigned long long &usum) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 4;
@@ -315,7 +365,7 @@ __device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigne
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const unsigned i = b0 + j * 32 + lane;
-      x[j] = i < cnt ? L[i] : make_uint4(0u, 0u, 0u, 0u);
+      x[j] = i < cnt ? A.list[P.at(i)] : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int j = 0; j < U; ++j) {
@@ -347,20 +397,15 @@ __device__ __forceinline__ void hook_pass(const Args &A, const uint4 *L, unsigne
 // A batch of graphs is solved as one graph whose edges and vertices are those
 // of its graphs, one after the other (eL, vL): positions there index parents,
 // lists and the bitmap, and order the edges of a graph as their own indices
-// do.  A warp's run of edges meets a few graphs; `f(g, x, k)` gets each piece:
-// graph g, its first position x and its k edges.
+// do.  A page of edges meets one or a few graphs; `f(g, x, k)` gets each piece
+// of the page's: graph g, its first position x and its k edges.
 template <class F>
-__device__ __forceinline__ void for_pieces(const Args &A, int64_t lo, int64_t hi, F f) {
-  if (lo >= hi) return;
-  int a = 0, b = A.G;  // eL[a] <= lo < eL[b]
-  while (b - a > 1) {
-    const int mid = (a + b) >> 1;
-    if (A.eL[mid] <= lo) a = mid;
-    else b = mid;
-  }
-  for (int64_t x = lo; x < hi; ++a) {
-    const int64_t end = A.eL[a + 1] < hi ? A.eL[a + 1] : hi;
-    if (end > x) f(a, x, (int)(end - x));
+__device__ __forceinline__ void for_pieces(const Args &A, uint32_t page, F f) {
+  const int64_t lo = (int64_t)page << A.es, full = lo + ((int64_t)1 << A.es), hi = full < A.m ? full : A.m;
+  int g = A.eg[page];
+  for (int64_t x = lo; x < hi; ++g) {
+    const int64_t end = A.eL[g + 1] < hi ? A.eL[g + 1] : hi;
+    if (end > x) f(g, x, (int)(end - x));
     x = end;
   }
 }
@@ -369,11 +414,12 @@ __device__ __forceinline__ int graph_from(const Args &A, int g, int64_t v) {
   while (g + 1 < A.G && A.vL[g + 1] <= v) ++g;
   return g;
 }
-__device__ __forceinline__ int graph_of_vertex(const Args &A, int64_t v) {
-  int a = 0, b = A.G;
+// graph of position x, off[g] <= x < off[g + 1]
+__device__ __forceinline__ int graph_at(const int64_t *off, int G, int64_t x) {
+  int a = 0, b = G;
   while (b - a > 1) {
     const int mid = (a + b) >> 1;
-    if (A.vL[mid] <= v) a = mid;
+    if (off[mid] <= x) a = mid;
     else b = mid;
   }
   return a;
@@ -439,27 +485,27 @@ __device__ __forceinline__ Ends load_ends(const Args &A, int64_t e, int64_t hi) 
   return q;
 }
 
-// First pass over the warp's edges [lo, hi): validation; the non-loop edges
-// below T0 go to the front of the warp's list, those from T0 to T1 to its back
-// (growing downwards from the region's end).  The pass is bound by instruction issue, so an edge costs a
+// First pass over the warp's edges: validation; the non-loop edges below T0 go
+// to the front of the warp's list, those from T0 to T1 to its back (growing
+// downwards from its end).  The pass is bound by instruction issue, so an edge costs a
 // running maximum (the index check), a NaN test and one or two comparisons
 // until it is selected.
 template <bool VEC, bool F32>
-__device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t hi, unsigned long long T0,
-                                            unsigned long long T1, uint4 *L, unsigned &front, unsigned &back,
-                                            unsigned &err) {
+__device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsigned long long T0,
+                                            unsigned long long T1, unsigned &front, unsigned &back, unsigned &err) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   const uint32_t n = (uint32_t)A.n;
-  front = back = 0;
-  if (lo >= hi) return;
-  uint4 *LB = L + A.E - 1;
+  front = back = err = 0;
+  if (!P.cap) return;
+  const unsigned last = P.cap - 1u;
   Limit<F32> l0(T0), l1(T1);
   uint32_t top = 0;  // largest index seen
   bool nan = false;
-  auto load = [&](int64_t b) { return load_quad<VEC>(A, b + 4 * lane, hi); };  // (zeros past the end: self-loops)
-  auto body = [&](const Quad &q, int64_t b) {
-    const int64_t e0 = b + 4 * lane;
+  // (zeros past the end: self-loops)
+  auto load = [&](int b) { return load_quad<VEC>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
+  auto body = [&](const Quad &q, int i) {
+    const int64_t b = P.at((uint32_t)i), e0 = b + 4 * lane;
     const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
     const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
     const uint32_t w[4] = {q.w.x, q.w.y, q.w.z, q.w.w};
@@ -476,14 +522,14 @@ __device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t h
       const unsigned mf = __ballot_sync(FULL, sel && l0.below(w[j]));
       const bool fr = mf >> lane & 1u;
       if (sel) {
-        uint4 *at = fr ? L + (front + __popc(mf & below)) : LB - (back + __popc(m & ~mf & below));
-        *at = make_uint4(u[j], v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
+        const unsigned at = fr ? front + __popc(mf & below) : last - (back + __popc(m & ~mf & below));
+        A.list[P.at(at)] = make_uint4(u[j], v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
       }
       front += __popc(mf);
       back += __popc(m & ~mf);
     }
   };
-  stream2<Quad>(lo, hi, load, body);
+  stream2<Quad>(0, (int)P.cap, load, body);
   err = (top >= n ? 1u : 0u) | (nan ? 2u : 0u);
   __syncwarp();
 }
@@ -495,15 +541,14 @@ __device__ __forceinline__ void select_pass(const Args &A, int64_t lo, int64_t h
 // from shared memory when it fits there (a gather of parents is one L1
 // wavefront per lane; R-MAT 20: 30 M of them).
 template <bool VEC, bool SMEM>
-__device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64_t hi, const uint32_t *bits,
-                                                uint4 *L) {
+__device__ __forceinline__ unsigned filter_pass(const Args &A, const Pages P, const uint32_t *bits) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   unsigned out = 0;
-  if (lo >= hi) return 0;
-  auto load = [&](int64_t b) { return load_ends<VEC>(A, b + 4 * lane, hi); };  // (zeros past the end: self-loops)
-  auto body = [&](const Ends &q, int64_t b) {
-    const int64_t e0 = b + 4 * lane;
+  // (zeros past the end: self-loops)
+  auto load = [&](int b) { return load_ends<VEC>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
+  auto body = [&](const Ends &q, int i) {
+    const int64_t e0 = P.at((uint32_t)i) + 4 * lane, hi = A.m;
     int32_t u[4] = {q.s.x, q.s.y, q.s.z, q.s.w}, v[4] = {q.d.x, q.d.y, q.d.z, q.d.w};
     uint32_t bu[4], bv[4], w[4];
     bool on[4];
@@ -531,12 +576,12 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
       const bool o = u[j] != v[j];
       const unsigned bal = __ballot_sync(FULL, o);
       if (o)
-        L[out + __popc(bal & below)] =
+        A.list[P.at(out + __popc(bal & below))] =
             make_uint4((uint32_t)u[j], (uint32_t)v[j], (uint32_t)(e0 + j), ord_weight_dev(w[j], A.wtype));
       out += __popc(bal);
     }
   };
-  stream2<Ends>(lo, hi, load, body);
+  stream2<Ends>(0, (int)P.cap, load, body);
   __syncwarp();
   return out;
 }
@@ -544,24 +589,23 @@ __device__ __forceinline__ unsigned filter_pass(const Args &A, int64_t lo, int64
 // The same passes over a batch, piece by piece (the thresholds' edge indices
 // are positions, compared edge by edge).
 template <bool F32>
-__device__ __forceinline__ void select_batch(const Args &A, bool vec, int64_t lo, int64_t hi, unsigned long long T0,
-                                             unsigned long long T1, uint4 *L, unsigned &front, unsigned &back,
-                                             unsigned &err) {
+__device__ __forceinline__ void select_batch(const Args &A, bool vec, const Pages P, unsigned long long T0,
+                                             unsigned long long T1, unsigned &front, unsigned &back, unsigned &err) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   front = back = 0;
-  uint4 *LB = L + A.E - 1;
+  const unsigned last = P.cap - 1u;
   Limit<F32> l0(T0), l1(T1);
   bool bad = false, nan = false;
-  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+  auto piece = [&](int g, int64_t x, int k) {
     const int64_t a = A.eA[g] + (x - A.eL[g]), base = a & ~(int64_t)3;
     const uint32_t vb = (uint32_t)A.vL[g], lim = (uint32_t)(A.vL[g + 1] - A.vL[g]);
     const int first = (int)(a - base), end = first + k;
     const int32_t *S = A.src + base, *D = A.dst + base;
     const uint32_t *W = A.w + base;
-    auto load = [&](int64_t b) { return edge_quad<true>(S, D, W, vec, (int)b + 4 * lane, first, end); };
-    auto body = [&](const EdgeQuad &q, int64_t b) {
-      const int i = (int)b + 4 * lane;
+    auto load = [&](int b) { return edge_quad<true>(S, D, W, vec, b + 4 * lane, first, end); };
+    auto body = [&](const EdgeQuad &q, int b) {
+      const int i = b + 4 * lane;
       const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
       const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
       const uint32_t w[4] = {q.w.x, q.w.y, q.w.z, q.w.w};
@@ -576,34 +620,34 @@ __device__ __forceinline__ void select_batch(const Args &A, bool vec, int64_t lo
         const unsigned mf = __ballot_sync(FULL, sel && l0.below(w[j], e));
         const bool fr = mf >> lane & 1u;
         if (sel) {
-          uint4 *at = fr ? L + (front + __popc(mf & below)) : LB - (back + __popc(m & ~mf & below));
-          *at = make_uint4(u[j] + vb, v[j] + vb, (uint32_t)e, ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
+          const unsigned at = fr ? front + __popc(mf & below) : last - (back + __popc(m & ~mf & below));
+          A.list[P.at(at)] = make_uint4(u[j] + vb, v[j] + vb, (uint32_t)e, ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
         }
         front += __popc(mf);
         back += __popc(m & ~mf);
       }
     };
     stream2<EdgeQuad>(0, end, load, body);
-  });
+  };
+  for (uint32_t i = 0; i < P.cap; i += 1u << P.s) for_pieces(A, P.page(i), piece);
   err = (bad ? 1u : 0u) | (nan ? 2u : 0u);
   __syncwarp();
 }
 
 template <bool SMEM>
-__device__ __forceinline__ unsigned filter_batch(const Args &A, bool vec, int64_t lo, int64_t hi, const uint32_t *bits,
-                                                 uint4 *L) {
+__device__ __forceinline__ unsigned filter_batch(const Args &A, bool vec, const Pages P, const uint32_t *bits) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   unsigned out = 0;
-  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+  auto piece = [&](int g, int64_t x, int k) {
     const int64_t a = A.eA[g] + (x - A.eL[g]), base = a & ~(int64_t)3;
     const int32_t vb = (int32_t)A.vL[g];
     const int first = (int)(a - base), end = first + k;
     const int32_t *S = A.src + base, *D = A.dst + base;
     const uint32_t *W = A.w + base;
-    auto load = [&](int64_t b) { return edge_quad<false>(S, D, W, vec, (int)b + 4 * lane, first, end); };
-    auto body = [&](const EdgeQuad &q, int64_t b) {
-      const int i = (int)b + 4 * lane;
+    auto load = [&](int b) { return edge_quad<false>(S, D, W, vec, b + 4 * lane, first, end); };
+    auto body = [&](const EdgeQuad &q, int b) {
+      const int i = b + 4 * lane;
       int32_t u[4] = {q.s.x + vb, q.s.y + vb, q.s.z + vb, q.s.w + vb};
       int32_t v[4] = {q.d.x + vb, q.d.y + vb, q.d.z + vb, q.d.w + vb};
       uint32_t w[4];
@@ -627,13 +671,14 @@ __device__ __forceinline__ unsigned filter_batch(const Args &A, bool vec, int64_
         const bool o = u[j] != v[j];
         const unsigned bal = __ballot_sync(FULL, o);
         if (o)
-          L[out + __popc(bal & below)] = make_uint4((uint32_t)u[j], (uint32_t)v[j], (uint32_t)(x + (i + j - first)),
-                                                    ord_weight_dev(w[j], A.wtype));
+          A.list[P.at(out + __popc(bal & below))] = make_uint4(
+              (uint32_t)u[j], (uint32_t)v[j], (uint32_t)(x + (i + j - first)), ord_weight_dev(w[j], A.wtype));
         out += __popc(bal);
       }
     };
     stream2<EdgeQuad>(0, end, load, body);
-  });
+  };
+  for (uint32_t i = 0; i < P.cap; i += 1u << P.s) for_pieces(A, P.page(i), piece);
   __syncwarp();
   return out;
 }
@@ -649,13 +694,8 @@ __device__ void pick_thresholds(const Args &A) {
   const int64_t e = i * A.m / SAMPLES + (int64_t)(((uint64_t)h * (uint64_t)step) >> 32);
   int64_t ea = e;
   if (A.G) {
-    int a = 0, b = A.G;
-    while (b - a > 1) {
-      const int mid = (a + b) >> 1;
-      if (A.eL[mid] <= e) a = mid;
-      else b = mid;
-    }
-    ea = A.eA[a] + (e - A.eL[a]);
+    const int g = graph_at(A.eL, A.G, e);
+    ea = A.eA[g] + (e - A.eL[g]);
   }
   const uint32_t w = ord_weight_dev(A.w[ea], A.wtype);
   const unsigned r0 = A.rank[0], r1 = A.rank[1];
@@ -740,19 +780,23 @@ __global__ void __launch_bounds__(ET, 1) k_prepare(Args A) {
     const int64_t words = (A.m + 31) / 32 + 2;
     for (int64_t i = tid; i < words; i += nthr) A.mbits[i] = 0u;
   }
-  for (int64_t i = tid; i < (int64_t)A.G * 256; i += nthr) A.bins[i] = 0ull;
+  if (A.G) {
+    for (int64_t i = tid; i < (int64_t)A.G * 256; i += nthr) A.bins[i] = 0ull;
+    for (int64_t i = tid; i << A.es < A.m; i += nthr) A.eg[i] = graph_at(A.eL, A.G, i << A.es);
+    for (int64_t i = tid; i << A.vs < A.n; i += nthr) A.vg[i] = graph_at(A.vL, A.G, i << A.vs);
+  }
   if (A.classes > 1 && blockIdx.x == 0) pick_thresholds(A);
 }
 
 template <bool VEC, bool F32, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_select(Args A) {
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
-  const int64_t lo = warp * A.E, hi = lo + A.E < A.m ? lo + A.E : A.m;
+  const Pages P(A.m, A.es, warp, (int64_t)gridDim.x * EW);
   const unsigned long long T0 = A.classes > 1 ? A.ctl->thresh[0] : KEY_INF;
   const unsigned long long T1 = A.classes > 2 ? A.ctl->thresh[1] : KEY_INF;
   unsigned front, back, err = 0;
-  if (BATCH) select_batch<F32>(A, VEC, lo, hi, T0, T1, A.list + lo, front, back, err);
-  else select_pass<VEC, F32>(A, lo, hi, T0, T1, A.list + lo, front, back, err);
+  if (BATCH) select_batch<F32>(A, VEC, P, T0, T1, front, back, err);
+  else select_pass<VEC, F32>(A, P, T0, T1, front, back, err);
   if (err) atomicOr(&A.ctl->err, err);
   if ((threadIdx.x & 31) == 0) {  // (an invalid edge ends the call: no list is used)
     A.front[warp] = front;
@@ -764,7 +808,7 @@ template <bool VEC, bool SMEM, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
   extern __shared__ uint32_t dyn_bits[];
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
-  const int64_t lo = warp * A.E, hi = lo + A.E < A.m ? lo + A.E : A.m;
+  const Pages P(A.m, A.es, warp, (int64_t)gridDim.x * EW);
   unsigned front = 0;
   if (!A.ctl->err && !A.ctl->abort) {  // (an invalid edge's index must not be used)
     if (SMEM) {
@@ -773,19 +817,18 @@ __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
       __syncthreads();
     }
     const uint32_t *bits = SMEM ? dyn_bits : A.gbits;
-    front = BATCH ? filter_batch<SMEM>(A, VEC, lo, hi, bits, A.list + lo)
-                  : filter_pass<VEC, SMEM>(A, lo, hi, bits, A.list + lo);
+    front = BATCH ? filter_batch<SMEM>(A, VEC, P, bits) : filter_pass<VEC, SMEM>(A, P, bits);
   }
   if ((threadIdx.x & 31) == 0) A.front[warp] = front;
 }
 
-// Mask bytes of the positions [lo, hi) of a batch, and the weights of the
+// Mask bytes of the warp's positions of a batch, and the weights of the
 // forest edges among them into their graphs' accumulators: a piece's sums of
 // four exponents from its first forest weight's down are kept in registers.
-__device__ void batch_results(const Args &A, int64_t lo, int64_t hi) {
+__device__ void batch_results(const Args &A, const Pages P) {
   const int lane = threadIdx.x & 31;
   constexpr int WIN = 4, U = 4;
-  for_pieces(A, lo, hi, [&](int g, int64_t x, int k) {
+  auto piece = [&](int g, int64_t x, int k) {
     const int64_t a = A.eA[g] + (x - A.eL[g]);
     if (A.mask) {
       uint8_t *mask = A.mask + a;
@@ -832,14 +875,15 @@ __device__ void batch_results(const Args &A, int64_t lo, int64_t hi) {
       for (int d = 16; d >= 1; d >>= 1) acc[i] += __shfl_xor_sync(FULL, acc[i], d);
       if (lane == 0 && acc[i]) atomicAdd(bins + (top - i), (unsigned long long)acc[i]);
     }
-  });
+  };
+  for (uint32_t i = 0; i < P.cap; i += 1u << P.s) for_pieces(A, P.page(i), piece);
 }
 
 // The rounds on the light classes (phase 0; the bitmap of the giant component
 // when a heavy class follows) or on the heavy edges left (phase 1); the
 // results at the end.
 template <bool BATCH>
-__global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
+__global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A, int phase) {
   __shared__ BlockSums sums;
   __shared__ long long sbins[256];
   __shared__ Table tab;
@@ -862,10 +906,8 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   __syncthreads();
   // the warp's vertices and its list of roots (all of them, or what the
   // flattening before the filter left)
-  const int64_t vlo = warp * A.VE < A.n ? warp * A.VE : A.n, vhi = vlo + A.VE < A.n ? vlo + A.VE : A.n;
-  int32_t *V = A.roots + vlo;
-  unsigned vc = phase == 0 ? (unsigned)(vhi - vlo) : A.back[warp];
-  uint4 *L = A.list + warp * A.E;
+  const Pages P(A.m, A.es, warp, nthr >> 5), Q(A.n, A.vs, warp, nthr >> 5);
+  unsigned vc = phase == 0 ? Q.len : A.back[warp];
   unsigned it = 0;  // counter of the grid sums
   auto aborted = [&]() { return *(volatile unsigned *)&C->abort != 0; };
   // The block's table goes to r; then the grid meets and the warps' counts are
@@ -906,7 +948,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
 #pragma unroll
         for (int j = 0; j < U; ++j) {
           const unsigned i = b0 + j * 32 + lane;
-          k[j] = i < vc ? (uint32_t)V[i] : 0xffffffffu;
+          k[j] = i < vc ? (uint32_t)A.roots[Q.at(i)] : 0xffffffffu;
         }
 #pragma unroll
         for (int j = 0; j < U; ++j) {
@@ -940,7 +982,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
             k[j] = (uint32_t)v | LONG;
           }
           const unsigned bal = __ballot_sync(FULL, keep);
-          if (keep) V[out + __popc(bal & below)] = (int32_t)k[j];
+          if (keep) A.roots[Q.at(out + __popc(bal & below))] = (int32_t)k[j];
           out += __popc(bal);
         }
       }
@@ -958,8 +1000,10 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   auto flatten = [&](bool bits, int32_t giant) -> bool {
     constexpr int U = 4;
     unsigned out = 0;
-    int gv = BATCH && bits && vlo < vhi ? graph_of_vertex(A, vlo) : 0;
-    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+    int gv = 0;
+    for (uint32_t i = 0; i < Q.cap; i += 32 * U) {
+      const int64_t v0 = Q.at(i), vhi = A.n;
+      if (BATCH && bits && !(i & ((1u << Q.s) - 1u))) gv = A.vg[Q.page(i)];
       int32_t x[U], y[U];
 #pragma unroll
       for (int j = 0; j < U; ++j) {
@@ -979,7 +1023,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
         if (a != x[j]) st_rel(A.p + v, a);
         const bool root = v < vhi && a == (int32_t)v;
         const unsigned mr = __ballot_sync(FULL, root);
-        if (root) V[out + __popc(mr & below)] = a;
+        if (root) A.roots[Q.at(out + __popc(mr & below))] = a;
         out += __popc(mr);
         if (bits) {
           if (BATCH && v < vhi) {
@@ -1003,13 +1047,13 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     unsigned long long live = total_live(cnt);
     for (int k = 0; k < ROUND_CAP && live; ++k) {
       const bool small = live <= SMALL;
-      hook_pass(A, L, cnt, small, !BATCH && A.totals, sums, usum);
+      hook_pass(A, P, cnt, small, !BATCH && A.totals, sums, usum);
       if (!grid_barrier(C, phase, target)) return false;
       if (!small) {
         if (!settle_roots()) return false;
-        cnt = min_pass<true>(A, tab, L, L, cnt);
+        cnt = min_pass<true, false>(A, tab, P, 0u, cnt);
       } else {
-        cnt = min_pass<true, true>(A, tab, L, L, cnt);
+        cnt = min_pass<true, true>(A, tab, P, 0u, cnt);
       }
       live = total_live(cnt);
     }
@@ -1017,12 +1061,12 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   };
 
   unsigned cnt = A.front[warp];
-  cnt = min_pass<false>(A, tab, L, L, cnt);
+  cnt = min_pass<false, false>(A, tab, P, 0u, cnt);
   if (!rounds(cnt)) return;
   if (phase == 0 && A.second) {
     if (!flatten(false, 0)) return;
     const unsigned back = A.back[warp];
-    cnt = min_pass<true>(A, tab, L + A.E - back, L, back);
+    cnt = min_pass<true, false>(A, tab, P, P.cap - back, back);
     if (!rounds(cnt)) return;
   }
   const bool last = phase == 1 || A.classes < 3;
@@ -1055,7 +1099,8 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
   // root.
   constexpr int U = 4;
   if (A.labels) {
-    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+    for (uint32_t i = 0; i < Q.cap; i += 32 * U) {
+      const int64_t v0 = Q.at(i), vhi = A.n;
       int32_t x[U], y[U];
 #pragma unroll
       for (int j = 0; j < U; ++j) x[j] = v0 + j * 32 + lane < vhi ? ld_rel(A.p + v0 + j * 32 + lane) : 0;
@@ -1072,7 +1117,8 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
         }
         if (a != x[j]) st_rel(A.p + v, a);
         if (a <= (int32_t)v) continue;  // (the root itself is added when read)
-        const int slot = table_slot(tab, a);
+        bool hit;
+        const int slot = table_slot(tab, a, hit);
         unsigned *low = reinterpret_cast<unsigned *>(slot < 0 ? A.r + a : tab.val + slot);
         if (slot < 0 || (unsigned)v < *(volatile unsigned *)low) atomicMin(low, (unsigned)v);
       }
@@ -1093,8 +1139,10 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     }
   }
   if (A.labels) {
-    int gv = BATCH && vlo < vhi ? graph_of_vertex(A, vlo) : 0;
-    for (int64_t v0 = vlo; v0 < vhi; v0 += 32 * U) {
+    int gv = 0;
+    for (uint32_t i = 0; i < Q.cap; i += 32 * U) {
+      const int64_t v0 = Q.at(i), vhi = A.n;
+      if (BATCH && !(i & ((1u << Q.s) - 1u))) gv = A.vg[Q.page(i)];
       int32_t x[U];
       unsigned b[U];
 #pragma unroll
@@ -1116,7 +1164,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(Args A, int phase) {
     }
   }
   if (BATCH) {
-    batch_results(A, warp * A.E, warp * A.E + A.E < A.m ? warp * A.E + A.E : A.m);
+    batch_results(A, P);
     if (A.totals) {
       if (!grid_barrier(C, phase, target)) return;
       // a warp per graph rounds its total
@@ -1178,8 +1226,10 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   const int64_t cap = (int64_t)sm_count();
   const int blocks = (int)(want < cap ? want : cap);
   const int64_t warps = (int64_t)blocks * EW;
-  A.E = ((m + warps - 1) / warps + 127) / 128 * 128;
-  A.VE = ((n + warps - 1) / warps + 127) / 128 * 128;
+  A.es = A.vs = 7;
+  while (A.es < PAGE && ((warps * EVEN) << (A.es + 1)) <= m) ++A.es;
+  while (A.vs < PAGE && ((warps * EVEN) << (A.vs + 1)) <= n) ++A.vs;
+  const int64_t epages = (m + ((int64_t)1 << A.es) - 1) >> A.es, vpages = (n + ((int64_t)1 << A.vs) - 1) >> A.vs;
   A.classes = 1;
   if (m >= 64 * SAMPLES) {
     double la = CLASS1, lb = CLASS2;
@@ -1190,7 +1240,7 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
     A.rank[0] = (unsigned)(la * (double)n / (double)m * SAMPLES);
     A.rank[1] = (unsigned)(lb * (double)n / (double)m * SAMPLES);
   }
-  const size_t bit_bytes = (size_t)((n + 31) / 32) * 4;
+  const size_t bit_bytes = (size_t)((n + 127) / 128) * 16;
   A.smem_bits = A.classes > 2 && bit_bytes <= SMEM_BITS;
   const size_t dyn = A.smem_bits ? bit_bytes : 0;
   size_t off = 0;
@@ -1205,10 +1255,11 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   const size_t o_tab = place(tab_bytes), o_giant = place((size_t)(which ? K : 0) * 4);
   const size_t o_bbins = place((size_t)(which ? K : 0) * 256 * 8);
   const size_t o_ctl = place(ctl_bytes), o_p = place((size_t)(n + 1) * 4), o_r = place((size_t)(n + 1) * 8);
-  const size_t o_roots = place((size_t)(n + 1) * 4), o_gbits = place(bit_bytes);
+  const size_t o_roots = place(((size_t)vpages << A.vs) * 4), o_gbits = place(bit_bytes);
   const size_t o_bits = place(((size_t)(m + 31) / 32 + 2) * 4);
   const size_t o_front = place((size_t)warps * 4), o_back = place((size_t)warps * 4);
-  const size_t o_list = place((size_t)warps * (size_t)A.E * 16);
+  const size_t o_eg = place(which ? (size_t)epages * 4 : 0), o_vg = place(which ? (size_t)vpages * 4 : 0);
+  const size_t o_list = place(((size_t)epages << A.es) * 16);
   int err = MSF_OK;
   char *base = (char *)pool_alloc(off, &err);
   if (err) return err;
@@ -1253,6 +1304,8 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
     A.vA = d + 3 * (K + 1);
     A.id = (int32_t *)(d + 4 * (K + 1));
     A.giant = (int32_t *)(base + o_giant);
+    A.eg = (int32_t *)(base + o_eg);
+    A.vg = (int32_t *)(base + o_vg);
     A.bins = (unsigned long long *)(base + o_bbins);
   }
   MSF_CK(cudaMemsetAsync(A.ctl, 0, ctl_bytes, s));
