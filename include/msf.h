@@ -86,8 +86,12 @@ int msf_build_csr(int64_t n, int64_t m, const int32_t *src, const int32_t *dst,
 
 /*
  * msf_compute -- minimum spanning forest of a built graph (Algorithm 2 with
- * complete shortcutting, Sec. 4.2).  The round loop runs on the device as a
- * CUDA graph with a conditional while node; the host waits once at the end.
+ * complete shortcutting, Sec. 4.2).  The forest is solved from the edges (light
+ * ones first, the others filtered), and the algorithm's rounds are counted for
+ * the statistics.  With an option that asks for a schedule, a builder, a
+ * compaction threshold, a kernel form, the host-driven loop or a limit below its
+ * default, the round loop over the CSR runs, as a CUDA graph with a conditional
+ * while node.  The host waits once at the end.
  *
  *   edge_mask  uint8[m]: 1 for forest edges, 0 otherwise (indexed like the
  *              input edges, or like the slots in CSR form).

@@ -117,6 +117,7 @@ void free_buf(CsrBuf &b) {
 void free_graph(msf_graph *g) {
   if (!g) return;
   pool_free(g->ends);
+  pool_free(g->w);
   pool_free(g->voff_d);
   pool_free(g->eoff_d);
   free_buf(g->csr0);
@@ -261,9 +262,57 @@ int check_weights_type(int wtype) {
   return MSF_OK;
 }
 
+// The one-shot solver gives the forest alone: a caller that asked for a
+// schedule, a builder, a kernel form or tighter limits than the defaults gets
+// the round loop over a CSR, whose steps those options are about.
+bool one_shot_allowed() {
+  const Options &o = options();
+  return o.exec_mode == 0 && o.shortcut_mode == MSF_SHORTCUT_CSP && !o.pairwise && o.build_mode == 0 &&
+         o.sweep == 0 && o.round_limit >= 64 && o.jump_limit >= 64;
+}
+
+// One graph's forest from the edges the build kept instead of the loop over the
+// CSR, with the loop's statistics (see k_rounds): every sweep of the loop reads
+// 12 bytes a slot and gathers a parent for each.  msf_compute, loop / this: R-MAT
+// 20 (2^24 edges) 1385 / 710 us, uniform 2^24 edges 1587 / 826, R-MAT 16 341 /
+// 202, 96^3 lattice 831 / 480, 1296 vertices 329 / 53.  MSF_ERR_OOM or
+// SOLVE_NOT_RUN: no room or no place for it, the loop runs.
+int edges_compute(msf_graph *g, uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s) {
+  LoopCounts c;
+  const int rc = small_counted(g->n, g->m)
+                     ? solve_small_pairs(g->n, g->m, g->ends, g->w, g->wtype, mask, labels, totals, &c, s)
+                     : solve_pairs(g->n, g->m, g->ends, g->w, g->wtype, mask, labels, totals, &c, s);
+  if (rc) return rc;
+  // the loop stops without a confirming round when one tree is left
+  g->stats.rounds = c.hooked + (c.hooked && options().early_stop && c.left <= 1 ? 0 : 1);
+  g->stats.compactions = 0;
+  g->stats.forest_edges = (int64_t)c.edges;
+  g->stats.jump_steps = c.passes;
+  g->stats.kernels = g->build_kernels + c.kernels;
+  return MSF_OK;
+}
+
 int graph_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *totals, int64_t ntot,
                   cudaStream_t s) {
-  int rc = ensure_workspace(g);
+  int rc;
+  if (g->G == 1 && g->w && one_shot_allowed() && options().tau == Options().tau) {
+    Staged sm, sl, st;
+    if ((rc = sm.output(edge_mask, (size_t)g->m)) || (rc = sl.output(labels, (size_t)g->n * 4)) ||
+        (rc = st.output(totals, 8)))
+      return rc;
+    rc = edges_compute(g, (uint8_t *)sm.dev, (int32_t *)sl.dev, (double *)st.dev, s);
+    if (rc != MSF_ERR_OOM && rc != SOLVE_NOT_RUN) {
+      if (rc || (rc = sm.copy_back(s)) || (rc = sl.copy_back(s)) || (rc = st.copy_back(s))) return rc;
+      if (sm.owned || sl.owned || st.owned) MSF_CK(cudaStreamSynchronize(s));
+      g->stats.n = g->n;
+      g->stats.m = g->m;
+      g->stats.nnz = g->nnz0;
+      g->stats.rows = g->nrows0;
+      return MSF_OK;
+    }
+    set_error("");
+  }
+  rc = ensure_workspace(g);
   if (rc) return rc;
   if ((rc = ensure_pairwise(g))) return rc;
   Staged sm, sl, st;
@@ -373,6 +422,22 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
       return cuda_fail(e, "copying offsets");
     }
   }
+  if (G == 1) {
+    // msf_compute reads the edges (4 bytes an edge more, 25 us of 770 us at 2^24
+    // edges); without room for them it runs the loop over the CSR
+    int err = MSF_OK;
+    g->w = (uint32_t *)pool_alloc((size_t)(m > 0 ? m : 1) * 4, &err);
+    if (err) {
+      g->w = nullptr;
+      set_error("");
+    } else if (m > 0) {
+      const cudaError_t e = cudaMemcpyAsync(g->w, sw.dev, (size_t)m * 4, cudaMemcpyDeviceToDevice, s);
+      if (e != cudaSuccess) {
+        free_graph(g);
+        return cuda_fail(e, "copying weights");
+      }
+    }
+  }
   rc = build_csr_device(n, m, (const int32_t *)ss.dev, (const int32_t *)sd.dev, (const int64_t *)sr.dev, sw.dev,
                         wtype, G, g->eoff_d, g->voff_d, s, g);
   if (rc) {
@@ -381,15 +446,6 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
   }
   *out = g;
   return MSF_OK;
-}
-
-// The one-shot solver gives the forest alone: a caller that asked for a
-// schedule, a builder, a kernel form or tighter limits than the defaults gets
-// the round loop over a CSR, whose steps those options are about.
-bool one_shot_allowed() {
-  const Options &o = options();
-  return o.exec_mode == 0 && o.shortcut_mode == MSF_SHORTCUT_CSP && !o.pairwise && o.build_mode == 0 &&
-         o.sweep == 0 && o.round_limit >= 64 && o.jump_limit >= 64;
 }
 
 int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t *src, const int32_t *dst,

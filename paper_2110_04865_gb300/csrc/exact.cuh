@@ -338,6 +338,31 @@ __device__ __forceinline__ EdgeQuad edge_quad(const int32_t *src, const int32_t 
   return q;
 }
 
+// The same from pairs of ends (16-byte aligned, as w), edges [i, hi) of four.
+__device__ __forceinline__ EdgeQuad pair_quad(const int2 *ends, const uint32_t *w, int i, int hi) {
+  EdgeQuad q;
+  q.s = q.d = make_int4(0, 0, 0, 0);
+  q.w = make_uint4(0u, 0u, 0u, 0u);
+  if (i + 4 <= hi) {
+    const int4 a = reinterpret_cast<const int4 *>(ends + i)[0], b = reinterpret_cast<const int4 *>(ends + i)[1];
+    q.s = make_int4(a.x, a.z, b.x, b.z);
+    q.d = make_int4(a.y, a.w, b.y, b.w);
+    q.w = *reinterpret_cast<const uint4 *>(w + i);
+    return q;
+  }
+  int32_t *s = &q.s.x, *d = &q.d.x;
+  uint32_t *v = &q.w.x;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (i + j < hi) {
+      const int2 uv = ends[i + j];
+      s[j] = uv.x;
+      d[j] = uv.y;
+      v[j] = w[i + j];
+    }
+  return q;
+}
+
 // Batches of 128 edges [lo, hi) through two register buffers in turn: a buffer
 // is loaded again once its batch is done, while the other's is worked on, and
 // none is copied to the other.

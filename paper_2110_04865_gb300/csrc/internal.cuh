@@ -303,6 +303,19 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
                 unsigned *status, cudaStream_t s);
 
+// One graph given as pairs of validated ends, with what the round loop of
+// Algorithm 2 takes on it (its statistics); may return MSF_ERR_OOM before any
+// work, or SOLVE_NOT_RUN.
+struct LoopCounts {
+  int32_t hooked;  // rounds in which roots hooked
+  uint32_t left;   // trees with edges after the last of them
+  uint32_t edges;  // forest edges
+  int32_t passes;  // passes that settle the hooked roots
+  int32_t kernels;
+};
+int solve_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+                double *totals, LoopCounts *counts, cudaStream_t s);
+
 // small.cu
 // The same for graphs that each fit in one SM's shared memory (small_fits),
 // one block per graph.
@@ -311,6 +324,9 @@ bool small_single(int64_t n, int64_t m);  // one graph: faster so than by solve_
 int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
                 unsigned *status, cudaStream_t s);
+bool small_counted(int64_t n, int64_t m);  // one graph with its counts: faster so than by solve_pairs
+int solve_small_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask,
+                      int32_t *labels, double *totals, LoopCounts *counts, cudaStream_t s);
 
 // exec.cu
 int enqueue_msf_graph(const DevState &hs, cudaStream_t s, const DevState **host_state);
@@ -330,6 +346,7 @@ struct msf_graph {
   int64_t nnz0, nrows0;
   int32_t build_kernels;  // kernels launched by the build
   int2 *ends;
+  uint32_t *w;  // weights of one graph, or NULL (no memory left for them)
   int64_t *voff_d, *eoff_d;
   msf::CsrBuf csr0;
   // workspace (allocated on the first compute)

@@ -37,8 +37,10 @@ constexpr int ROUND_CAP = 64;  // Boruvka rounds at most (components at least ha
 
 struct SmallArgs {
   const int32_t *src, *dst;
+  const int2 *ends;        // instead of src and dst: validated ends
   const uint32_t *w;
   int32_t wtype;
+  int32_t count;           // the loop's rounds are counted (no edges filtered)
   int32_t vec;             // the three arrays are 16-byte aligned
   const int64_t *voff, *eoff;  // [2 * block]: its graph's offsets (pinned host memory, read in place)
   const int32_t *order;    // graph of each block, or NULL
@@ -48,7 +50,7 @@ struct SmallArgs {
   uint8_t *mask;
   int32_t *labels;
   double *totals;
-  unsigned *host;          // pinned: [0] index out of range, [1] NaN weight
+  unsigned *host;          // pinned: [0] index out of range, [1] NaN weight, [2..4] LoopCounts
 };
 
 // Dynamic shared memory of a graph: minima, parents, forest bitmap.
@@ -71,6 +73,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
   __shared__ BlockSums sums;
   __shared__ long long sbins[256];
   __shared__ unsigned long long s_usum, s_thresh;
+  __shared__ unsigned s_pairs[2], s_edges;  // trees formed, by round modulo 2; forest edges
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned below = (1u << lane) - 1u;
   const int at = 2 * (int)blockIdx.x;
@@ -92,7 +95,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
   }
   for (int i = threadIdx.x; i < (m + 31) / 32 + 2; i += NT) bits[i] = 0u;
   sums.clear();
-  if (threadIdx.x == 0) s_usum = 0;
+  if (threadIdx.x == 0) s_usum = s_edges = 0;
+  int hooked = 0;  // rounds with hooks
   unsigned long long usum = 0;  // uint32 weights of the thread's forest edges
   uint32_t top = 0;             // largest endpoint seen
   bool nan = false;
@@ -106,10 +110,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
   };
   // hook along a minimum (tie breaking as in Algorithm 2: of two roots that
   // chose the same edge the smaller stays a root)
+  unsigned pairs = 0;  // roots of the thread's edges that chose each other
   auto hook = [&](uint32_t uv, uint32_t e, uint32_t ow) -> bool {
     const uint32_t u = uv & 0xffffu, v = uv >> 16;
     const bool mu = rw[u] == ow && re[u] == e, mv = rw[v] == ow && re[v] == e;
     if (!(mu || mv)) return false;
+    pairs += mu && mv;
     if (mu && (!mv || v < u)) p[u] = (uint16_t)v;
     else p[v] = (uint16_t)u;
     return true;
@@ -126,6 +132,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     const uint32_t u = uv & 0xffffu, v = uv >> 16;
     if (rw[u] == ow) atomicMin(re + u, e);
     if (rw[v] == ow) atomicMin(re + v, e);
+  };
+  // A round's hooks are counted (its slot was cleared before its first barrier).
+  auto count_round = [&]() {
+    if (!A.count) return;
+    const unsigned t = __reduce_add_sync(FULL, pairs);
+    if (lane == 0 && t) atomicAdd(&s_pairs[hooked & 1], t);
+    pairs = 0;
+    ++hooked;
   };
   // Every parent a root (a vertex's parent is written by its own thread only),
   // the minima cleared; four vertices' chains side by side.
@@ -166,6 +180,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     unsigned in = 0;  // kept entries in the forest
     for (int k = 0; k < ROUND_CAP; ++k) {
       uint32_t left = 0;
+      if (threadIdx.x == 0) s_pairs[hooked & 1] = 0;
 #pragma unroll
       for (int j = 0; j < KEEP; ++j) {
         if (!kuv[j]) continue;
@@ -184,6 +199,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
           in |= 1u << j;
           kuv[j] = 0u;
         }
+      count_round();
       __syncthreads();
       settle();
     }
@@ -210,6 +226,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
         return;
       }
       int out = 0;
+      if (threadIdx.x == 0) s_pairs[hooked & 1] = 0;
       for (int b0 = 0; b0 < cnt; b0 += 32 * U) {
         uint4 x[U];
 #pragma unroll
@@ -227,7 +244,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       }
       __syncwarp();
       cnt = out;
-      __syncthreads();
+      if (!__syncthreads_or(cnt > 0)) return;
       for (int b0 = 0; b0 < cnt; b0 += 32 * U) {
         uint4 x[U];
 #pragma unroll
@@ -245,6 +262,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
         for (int j = 0; j < U; ++j)
           if (x[j].x && hook(x[j].x, x[j].z, x[j].w)) mark(x[j].z, x[j].w);
       }
+      count_round();
       __syncthreads();
       settle();
     }
@@ -264,8 +282,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       const int i = j * NT + threadIdx.x;
       uint32_t u = 0, v = 0, w = 0;
       if (i < m) {
-        u = (uint32_t)A.src[e0 + i];
-        v = (uint32_t)A.dst[e0 + i];
+        const int2 uv = A.ends ? A.ends[e0 + i] : make_int2(A.src[e0 + i], A.dst[e0 + i]);
+        u = (uint32_t)uv.x;
+        v = (uint32_t)uv.y;
         w = A.w[e0 + i];
       }
       top = max(top, max(u, v));
@@ -280,7 +299,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     // The threshold: about the key of the wanted rank in a sample of warp 0,
     // found bit by bit with ballots -- twelve bits below the samples' common
     // prefix; any threshold is a valid one.
-    const bool filter = (double)m > 1.5 * LIGHT * (double)n;
+    const bool filter = !A.count && (double)m > 1.5 * LIGHT * (double)n;
     if (wid == 0 && filter) {
       constexpr int PER = 8;
       uint32_t w[PER], e[PER], lo = NONE, up = 0u;
@@ -332,7 +351,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     L = A.list + (A.loff ? A.loff[blockIdx.x] : 0) + lo;
     int cnt = 0;
     {
-      auto load = [&](int b) { return edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi); };
+      auto load = [&](int b) { return A.ends ? pair_quad(A.ends, W, b + 4 * lane, hi) : edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi); };
       auto body = [&](const EdgeQuad &q, int b) {
         const int i = b + 4 * lane;
         limit.batch(a0 + b);
@@ -380,6 +399,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       stream2<EdgeQuad>(lo, hi, load, body);
       __syncwarp();
       rounds(cnt);
+    }
+  }
+  if (A.count) {
+    __syncthreads();
+    unsigned c = 0;
+    for (int i = threadIdx.x; i < (m + 31) / 32; i += NT) c += __popc(bits[i]);
+    c = __reduce_add_sync(FULL, c);
+    if (lane == 0 && c) atomicAdd(&s_edges, c);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      A.host[2] = (unsigned)hooked;
+      A.host[3] = hooked ? s_pairs[(hooked - 1) & 1] : 0u;
+      A.host[4] = s_edges;
     }
   }
   // Results (parents are roots, the minima clear).  The last warp rounds the
@@ -502,18 +534,24 @@ bool small_fits(int64_t n, int64_t m) {
 // 235, (8000, 200000) 265 / 225, (4000, 200000) 176 / 230, (4000, 65536) 147 / 300.
 bool small_single(int64_t n, int64_t m) { return small_fits(n, m) && m + 8 * n <= ((int64_t)1 << 18); }
 
-// Forests of one graph (which = NULL), or of K graphs that fit (small_fits),
-// `which` of the graphs with the host offsets voff, eoff.  Synchronizes `s`;
-// *status: 1 = index out of range, 2 = NaN weight.
-int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
-                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                unsigned *status, cudaStream_t s) {
+// The same with the loop's rounds counted, which needs every edge in every round:
+// (8000, 16000) 115 / 166, (1500, 15000) 109 / 147, (1500, 40000) 207 / 153,
+// (8000, 60000) 345 / 195.
+bool small_counted(int64_t n, int64_t m) { return small_fits(n, m) && m <= ((int64_t)3 << 13); }
+
+namespace {
+
+int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+          const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+          double *totals, unsigned *status, LoopCounts *counts, cudaStream_t s) {
   const int64_t n = which ? 0 : voff[1], m = which ? 0 : eoff[1];
   const int32_t G = which ? K : 1;
   SmallArgs A;
   std::memset(&A, 0, sizeof(A));
   A.src = src;
   A.dst = dst;
+  A.ends = ends;
+  A.count = counts != nullptr;
   A.w = w;
   A.wtype = wtype;
   A.vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
@@ -612,9 +650,34 @@ int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int6
   if (rc) return rc;
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "forests of small graphs");
-  if (((volatile unsigned *)pin.p)[0]) *status |= 1u;
-  if (((volatile unsigned *)pin.p)[1]) *status |= 2u;
+  const volatile unsigned *st = (volatile unsigned *)pin.p;
+  if (st[0]) *status |= 1u;
+  if (st[1]) *status |= 2u;
+  if (counts) {
+    counts->hooked = counts->passes = (int32_t)st[2];
+    counts->left = st[3];
+    counts->edges = st[4];
+    counts->kernels = 1;
+  }
   return MSF_OK;
+}
+
+}  // namespace
+
+// Forests of one graph (which = NULL), or of K graphs that fit (small_fits),
+// `which` of the graphs with the host offsets voff, eoff.  Synchronizes `s`;
+// *status: 1 = index out of range, 2 = NaN weight.
+int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
+                unsigned *status, cudaStream_t s) {
+  return solve(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, status, nullptr, s);
+}
+
+int solve_small_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask,
+                      int32_t *labels, double *totals, LoopCounts *counts, cudaStream_t s) {
+  const int64_t voff[2] = {0, n}, eoff[2] = {0, m};
+  unsigned status = 0;
+  return solve(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, &status, counts, s);
 }
 
 }  // namespace msf

@@ -71,6 +71,11 @@ constexpr double CLASS1 = 0.75, CLASS2 = 1.5;
 // Below this the light edges form one class: a second one saves less than its
 // rounds' barriers cost (R-MAT 16, m = 2^20: 197 us with one, 212 with two).
 constexpr int64_t TWO_CLASSES = 1 << 22;
+// With the loop's rounds counted one class up to here (its rounds are the
+// loop's), classes and a replay of the rounds on the forest from here on: in us,
+// one class / classes, R-MAT 2^20 edges 202 / 260, 2^21 266 / 297, 2^22 381 / 354;
+// uniform 2^20 282 / 325, 2^22 635 / 484; lattice 10^6 298 / 424.
+constexpr int64_t COUNT_CLASSES = 3 << 20;
 // Edges left from which a round's roots are settled in a step of their own:
 // below, all of them are in flight at once (155 648 threads) and the minimum
 // pass follows the chains itself, one barrier and about 5 us less per round
@@ -87,16 +92,19 @@ constexpr int PAGE = 10, EVEN = 16;
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
 struct Ctrl {
-  unsigned arrive[2];  // grid barriers of the two rounds kernels
+  unsigned arrive[3];  // grid barriers of the rounds kernels
   unsigned abort;      // a barrier wait ran out
   unsigned err;        // 1 = index out of range, 2 = NaN weight
-  unsigned long long live[2][4];  // edges left, by round modulo 4, of the two rounds kernels
+  unsigned long long live[3][4];  // edges left, by round modulo 4, of the rounds kernels
+  unsigned pairs[4];   // trees formed, by round modulo 4
+  unsigned edges;      // forest edges
   unsigned long long thresh[2];  // keys of the first class lie below [0], of the second below [1]
 };
 
 struct Args {
   int64_t n, m;
   const int32_t *src, *dst;
+  const int2 *ends;     // instead of src and dst: validated ends
   const uint32_t *w;
   int32_t wtype;
   int32_t classes;      // 1 = every edge in the first class, 2 = none heavy, 3
@@ -123,7 +131,7 @@ struct Args {
   uint8_t *mask;
   int32_t *labels;
   double *totals;
-  unsigned *host;       // pinned: [0] status bits
+  unsigned *host;       // pinned: [0] status bits, [1..4] rounds with hooks, trees the last left, edges, passes
 };
 
 __device__ __forceinline__ int ld_rel(const int32_t *a) {
@@ -355,10 +363,13 @@ __device__ __noinline__ unsigned min_pass(const Args &A, Table &tab, const Pages
 
 // Hooks along every entry that is the minimum of one of its ends (tie
 // breaking: of two roots that chose the same edge the smaller stays a root).
-__device__ __noinline__ void hook_pass(const Args &A, const Pages P, unsigned cnt, bool small, bool sum, BlockSums &sums,
+// Returns the hooks of the thread in the low half and those of two roots that
+// chose each other, one for every tree formed, in the high half.
+__device__ __noinline__ unsigned hook_pass(const Args &A, const Pages P, unsigned cnt, bool small, bool mark, bool sum, BlockSums &sums,
                                           unsigned long long &usum) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 4;
+  unsigned hooks = 0;
   for (unsigned b0 = 0; b0 < cnt; b0 += 32 * U) {
     uint4 x[U];
     unsigned long long ru[U], rv[U];
@@ -379,19 +390,21 @@ __device__ __noinline__ void hook_pass(const Args &A, const Pages P, unsigned cn
       const unsigned long long key = ((unsigned long long)x[j].w << 32) | x[j].z;
       const bool mu = ru[j] == key, mv = rv[j] == key;
       if (!((x[j].x & CAND) && (mu || mv))) continue;
+      hooks += mu && mv ? 0x10001u : 1u;
       if (small) {  // the minima are cleared here (no other entry's key equals them, before or after)
         if (mu) A.r[u] = KEY_INF;
         if (mv) A.r[v] = KEY_INF;
       }
       if (mu && (!mv || v < u)) A.p[u] = v;
       else A.p[v] = u;
-      if (A.mbits) atomicOr(A.mbits + (x[j].z >> 5), 1u << (x[j].z & 31u));
+      if (mark) atomicOr(A.mbits + (x[j].z >> 5), 1u << (x[j].z & 31u));
       if (sum) {
         if (A.wtype == MSF_U32) usum += x[j].w;
         else sums.add(x[j].w);
       }
     }
   }
+  return hooks;
 }
 
 // A batch of graphs is solved as one graph whose edges and vertices are those
@@ -430,12 +443,38 @@ struct Quad {
   int4 s, d;
   uint4 w;
 };
-template <bool VEC>
+// Forms of the edges: separate arrays of ends, aligned or not, or pairs.
+enum Form { SCALAR = 0, VECTOR = 1, PAIRS = 2 };
+__device__ __forceinline__ void load_pairs(const int2 *ends, int64_t e, int64_t hi, int4 &s, int4 &d) {
+  if (e + 4 <= hi) {
+    const int4 a = __ldcs(reinterpret_cast<const int4 *>(ends + e)), b = __ldcs(reinterpret_cast<const int4 *>(ends + e) + 1);
+    s = make_int4(a.x, a.z, b.x, b.z);
+    d = make_int4(a.y, a.w, b.y, b.w);
+    return;
+  }
+  int32_t *x = &s.x, *y = &d.x;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (e + j < hi) {
+      const int2 a = ends[e + j];
+      x[j] = a.x;
+      y[j] = a.y;
+    }
+}
+template <int FORM>
 __device__ __forceinline__ Quad load_quad(const Args &A, int64_t e, int64_t hi) {
   Quad q;
   q.s = q.d = make_int4(0, 0, 0, 0);
   q.w = make_uint4(0u, 0u, 0u, 0u);
-  if (VEC && e + 4 <= hi) {
+  if (FORM == PAIRS) {
+    load_pairs(A.ends, e, hi, q.s, q.d);
+    uint32_t *w = &q.w.x;
+    if (e + 4 <= hi) q.w = __ldcs(reinterpret_cast<const uint4 *>(A.w + e));
+    else
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (e + j < hi) w[j] = A.w[e + j];
+  } else if (FORM == VECTOR && e + 4 <= hi) {
     q.s = __ldcs(reinterpret_cast<const int4 *>(A.src + e));
     q.d = __ldcs(reinterpret_cast<const int4 *>(A.dst + e));
     q.w = __ldcs(reinterpret_cast<const uint4 *>(A.w + e));
@@ -466,11 +505,13 @@ __device__ __forceinline__ Quad load_quad(const Args &A, int64_t e, int64_t hi) 
 struct Ends {
   int4 s, d;
 };
-template <bool VEC>
+template <int FORM>
 __device__ __forceinline__ Ends load_ends(const Args &A, int64_t e, int64_t hi) {
   Ends q;
   q.s = q.d = make_int4(0, 0, 0, 0);
-  if (VEC && e + 4 <= hi) {
+  if (FORM == PAIRS) {
+    load_pairs(A.ends, e, hi, q.s, q.d);
+  } else if (FORM == VECTOR && e + 4 <= hi) {
     q.s = __ldcs(reinterpret_cast<const int4 *>(A.src + e));
     q.d = __ldcs(reinterpret_cast<const int4 *>(A.dst + e));
   } else if (e < hi) {
@@ -490,7 +531,7 @@ __device__ __forceinline__ Ends load_ends(const Args &A, int64_t e, int64_t hi) 
 // downwards from its end).  The pass is bound by instruction issue, so an edge costs a
 // running maximum (the index check), a NaN test and one or two comparisons
 // until it is selected.
-template <bool VEC, bool F32>
+template <int FORM, bool F32>
 __device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsigned long long T0,
                                             unsigned long long T1, unsigned &front, unsigned &back, unsigned &err) {
   const int lane = threadIdx.x & 31;
@@ -503,7 +544,7 @@ __device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsign
   uint32_t top = 0;  // largest index seen
   bool nan = false;
   // (zeros past the end: self-loops)
-  auto load = [&](int b) { return load_quad<VEC>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
+  auto load = [&](int b) { return load_quad<FORM>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
   auto body = [&](const Quad &q, int i) {
     const int64_t b = P.at((uint32_t)i), e0 = b + 4 * lane;
     const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
@@ -513,8 +554,10 @@ __device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsign
     l1.batch(b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      top = max(top, max(u[j], v[j]));
-      if (F32) nan |= __uint_as_float(w[j]) != __uint_as_float(w[j]);
+      if (FORM != PAIRS) {
+        top = max(top, max(u[j], v[j]));
+        if (F32) nan |= __uint_as_float(w[j]) != __uint_as_float(w[j]);
+      }
       const bool sel = l1.below(w[j]) && u[j] != v[j];
       const unsigned m = __ballot_sync(FULL, sel);
       if (!m) continue;
@@ -530,7 +573,7 @@ __device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsign
     }
   };
   stream2<Quad>(0, (int)P.cap, load, body);
-  err = (top >= n ? 1u : 0u) | (nan ? 2u : 0u);
+  if (FORM != PAIRS) err = (top >= n ? 1u : 0u) | (nan ? 2u : 0u);
   __syncwarp();
 }
 
@@ -540,13 +583,13 @@ __device__ __forceinline__ void select_pass(const Args &A, const Pages P, unsign
 // Most edges lie inside the giant component: two bits of its bitmap tell,
 // from shared memory when it fits there (a gather of parents is one L1
 // wavefront per lane; R-MAT 20: 30 M of them).
-template <bool VEC, bool SMEM>
+template <int FORM, bool SMEM>
 __device__ __forceinline__ unsigned filter_pass(const Args &A, const Pages P, const uint32_t *bits) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   unsigned out = 0;
   // (zeros past the end: self-loops)
-  auto load = [&](int b) { return load_ends<VEC>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
+  auto load = [&](int b) { return load_ends<FORM>(A, P.at((uint32_t)b) + 4 * lane, (uint32_t)b < P.cap ? A.m : 0); };
   auto body = [&](const Ends &q, int i) {
     const int64_t e0 = P.at((uint32_t)i) + 4 * lane, hi = A.m;
     int32_t u[4] = {q.s.x, q.s.y, q.s.z, q.s.w}, v[4] = {q.d.x, q.d.y, q.d.z, q.d.w};
@@ -729,7 +772,7 @@ __device__ int32_t vote_giant(const Args &A) {
   if (threadIdx.x == 0) best = 0;
   if (threadIdx.x < VOTES) {
     const int64_t e = (int64_t)((unsigned long long)threadIdx.x * (unsigned long long)A.m / VOTES);
-    int32_t x = (threadIdx.x & 1) ? A.src[e] : A.dst[e];
+    int32_t x = A.ends ? ((threadIdx.x & 1) ? A.ends[e].x : A.ends[e].y) : (threadIdx.x & 1) ? A.src[e] : A.dst[e];
     if ((uint32_t)x >= (uint32_t)A.n) x = 0;  // (an invalid edge: the call fails later)
     int32_t y = __ldca(A.p + x);
     while (y != x) {
@@ -788,15 +831,15 @@ __global__ void __launch_bounds__(ET, 1) k_prepare(Args A) {
   if (A.classes > 1 && blockIdx.x == 0) pick_thresholds(A);
 }
 
-template <bool VEC, bool F32, bool BATCH>
+template <int FORM, bool F32, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_select(Args A) {
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
   const Pages P(A.m, A.es, warp, (int64_t)gridDim.x * EW);
   const unsigned long long T0 = A.classes > 1 ? A.ctl->thresh[0] : KEY_INF;
   const unsigned long long T1 = A.classes > 2 ? A.ctl->thresh[1] : KEY_INF;
   unsigned front, back, err = 0;
-  if (BATCH) select_batch<F32>(A, VEC, P, T0, T1, front, back, err);
-  else select_pass<VEC, F32>(A, P, T0, T1, front, back, err);
+  if (BATCH) select_batch<F32>(A, FORM == VECTOR, P, T0, T1, front, back, err);
+  else select_pass<FORM, F32>(A, P, T0, T1, front, back, err);
   if (err) atomicOr(&A.ctl->err, err);
   if ((threadIdx.x & 31) == 0) {  // (an invalid edge ends the call: no list is used)
     A.front[warp] = front;
@@ -804,7 +847,7 @@ __global__ void __launch_bounds__(ET, 1) k_select(Args A) {
   }
 }
 
-template <bool VEC, bool SMEM, bool BATCH>
+template <int FORM, bool SMEM, bool BATCH>
 __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
   extern __shared__ uint32_t dyn_bits[];
   const int64_t warp = ((int64_t)blockIdx.x * ET + threadIdx.x) >> 5;
@@ -817,7 +860,7 @@ __global__ void __launch_bounds__(ET, 1) k_filter(Args A) {
       __syncthreads();
     }
     const uint32_t *bits = SMEM ? dyn_bits : A.gbits;
-    front = BATCH ? filter_batch<SMEM>(A, VEC, P, bits) : filter_pass<VEC, SMEM>(A, P, bits);
+    front = BATCH ? filter_batch<SMEM>(A, FORM == VECTOR, P, bits) : filter_pass<FORM, SMEM>(A, P, bits);
   }
   if ((threadIdx.x & 31) == 0) A.front[warp] = front;
 }
@@ -879,15 +922,54 @@ __device__ void batch_results(const Args &A, const Pages P) {
   for (uint32_t i = 0; i < P.cap; i += 1u << P.s) for_pieces(A, P.page(i), piece);
 }
 
+// The forest's edges into the warp's list, the state of its vertices as at the
+// start; returns the entries.
+__device__ __noinline__ unsigned list_forest(const Args &A, const Pages P, const Pages Q) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  for (uint32_t i = lane; i < Q.cap; i += 32) {
+    const int64_t v = Q.at(i);
+    if (v >= A.n) continue;
+    st_rel(A.p + v, (int32_t)v);
+    A.r[v] = KEY_INF;
+    A.roots[v] = (int32_t)v;
+  }
+  unsigned out = 0;
+  constexpr int U = 4;
+  for (uint32_t i = 0; i < P.cap; i += 32 * U) {
+    const int64_t e0 = P.at(i);
+    if (e0 >= A.m) continue;
+    uint4 x[U];
+    bool on[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {  // (the bitmap's words end at most 128 edges behind the last)
+      const int64_t e = e0 + j * 32 + lane;
+      on[j] = e < A.m && (__ldcg(A.mbits + (e0 >> 5) + j) >> lane & 1u);
+      const int2 uv = on[j] ? A.ends[e] : make_int2(0, 0);
+      x[j] = make_uint4((uint32_t)uv.x, (uint32_t)uv.y, (uint32_t)e, on[j] ? ord_weight_dev(A.w[e], A.wtype) : 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned bal = __ballot_sync(FULL, on[j]);
+      if (on[j]) A.list[P.at(out + __popc(bal & below))] = x[j];
+      out += __popc(bal);
+    }
+  }
+  __syncwarp();
+  return out;
+}
+
 // The rounds on the light classes (phase 0; the bitmap of the giant component
 // when a heavy class follows) or on the heavy edges left (phase 1); the
-// results at the end.
-template <bool BATCH>
+// results at the end.  Phase 2 counts the rounds that the loop takes without
+// classes: they are those on the forest's own edges (the lightest edge that
+// leaves a component is one of them, so every round hooks the same roots).
+template <bool BATCH, bool COUNT>
 __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A, int phase) {
   __shared__ BlockSums sums;
   __shared__ long long sbins[256];
   __shared__ Table tab;
-  __shared__ unsigned s_live;
+  __shared__ unsigned s_live, s_pairs, s_edges;
   Ctrl *C = A.ctl;
   if (C->abort) return;  // (phase 0 did not finish)
   if (C->err) {          // an invalid edge: its indices must not be used
@@ -901,14 +983,26 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   const unsigned below = (1u << lane) - 1u;
   unsigned long long usum = 0;  // uint32 weights of the thread's forest edges
   sums.clear();
-  if (threadIdx.x == 0) s_live = 0;
+  if (threadIdx.x == 0) s_live = s_pairs = s_edges = 0;
   table_clear(tab);
   __syncthreads();
   // the warp's vertices and its list of roots (all of them, or what the
   // flattening before the filter left)
   const Pages P(A.m, A.es, warp, nthr >> 5), Q(A.n, A.vs, warp, nthr >> 5);
-  unsigned vc = phase == 0 ? Q.len : A.back[warp];
+  unsigned vc = phase == 1 ? A.back[warp] : Q.len;
   unsigned it = 0;  // counter of the grid sums
+  // the rounds are counted: those of phase 2, or of the only class
+  const bool counting = COUNT && (phase == 2 || A.classes == 1);
+  unsigned *pair_slot = C->pairs;
+  int hooked = 0;       // rounds with hooks
+  unsigned passes = 0;  // settling passes and chases
+  auto counted = [&]() {  // (behind a grid barrier)
+    if (!counting || tid != 0) return;
+    A.host[1] = (unsigned)hooked;
+    A.host[2] = hooked ? *(volatile unsigned *)&C->pairs[(hooked - 1) & 3] : 0u;
+    A.host[3] = *(volatile unsigned *)&C->edges;
+    A.host[4] = passes;
+  };
   auto aborted = [&]() { return *(volatile unsigned *)&C->abort != 0; };
   // The block's table goes to r; then the grid meets and the warps' counts are
   // summed (0 when the wait ran out).
@@ -924,6 +1018,11 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     if (threadIdx.x == 0) {
       if (s_live) atomicAdd(&C->live[phase][it & 3u], (unsigned long long)s_live);
       s_live = 0;
+      if (COUNT) {
+        if (s_pairs) atomicAdd(pair_slot, s_pairs);
+        if (s_edges) atomicAdd(&C->edges, s_edges);
+        s_pairs = s_edges = 0;
+      }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) C->live[phase][(it + 2) & 3u] = 0;
     if (!grid_barrier(C, phase, target)) return 0;
@@ -939,6 +1038,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   auto settle_roots = [&]() -> bool {
     constexpr int U = 4;
     for (int pass = 0; pass < ROUND_CAP; ++pass) {
+      ++passes;
       unsigned out = 0;
       bool more = false;
       for (unsigned b0 = 0; b0 < vc; b0 += 32 * U) {
@@ -1047,12 +1147,21 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     unsigned long long live = total_live(cnt);
     for (int k = 0; k < ROUND_CAP && live; ++k) {
       const bool small = live <= SMALL;
-      hook_pass(A, P, cnt, small, !BATCH && A.totals, sums, usum);
+      const unsigned h = hook_pass(A, P, cnt, small, A.mbits && !(COUNT && phase == 2), !BATCH && A.totals && !(COUNT && phase == 2), sums, usum);
+      if (counting) {  // (added up with the edges left; the round's slot was cleared two rounds before)
+        const unsigned t = __reduce_add_sync(FULL, h & 0xffffu), q = __reduce_add_sync(FULL, h >> 16);
+        if (lane == 0 && q) atomicAdd(&s_pairs, q);
+        if (lane == 0 && t) atomicAdd(&s_edges, t);
+        pair_slot = &C->pairs[k & 3];
+        if (tid == 0) C->pairs[(k + 2) & 3] = 0;
+        ++hooked;
+      }
       if (!grid_barrier(C, phase, target)) return false;
       if (!small) {
         if (!settle_roots()) return false;
         cnt = min_pass<true, false>(A, tab, P, 0u, cnt);
       } else {
+        ++passes;
         cnt = min_pass<true, true>(A, tab, P, 0u, cnt);
       }
       live = total_live(cnt);
@@ -1060,9 +1169,19 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     return !aborted();
   };
 
-  unsigned cnt = A.front[warp];
+  unsigned cnt;
+  if (COUNT && phase == 2) {
+    cnt = list_forest(A, P, Q);
+    if (!grid_barrier(C, phase, target)) return;
+  } else {
+    cnt = A.front[warp];
+  }
   cnt = min_pass<false, false>(A, tab, P, 0u, cnt);
   if (!rounds(cnt)) return;
+  if (COUNT && phase == 2) {
+    counted();
+    return;
+  }
   if (phase == 0 && A.second) {
     if (!flatten(false, 0)) return;
     const unsigned back = A.back[warp];
@@ -1187,20 +1306,17 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     for (int64_t e = h + (nq << 4) + tid; e < m; e += nthr)
       A.mask[e] = (uint8_t)((A.mbits[e >> 5] >> (e & 31)) & 1u);
   }
+  counted();
   if (tid == 0) A.host[0] = *(volatile unsigned *)&C->err;
 }
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-}  // namespace
-
-// Forest of one graph from its edge list, or of K graphs of a batch, `which` of
-// the graphs with the host offsets voff, eoff (pointers the device can read).
-// Any output may be NULL.  Synchronizes `s`; *status: 1 = index out of range,
-// 2 = NaN weight.
-int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
-                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                unsigned *status, cudaStream_t s) {
+// The edges as separate arrays (src, dst) or as pairs of validated ends; with
+// `counts` (one graph, pairs) the rounds of the loop without classes too.
+int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+          const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+          double *totals, unsigned *status, LoopCounts *counts, cudaStream_t s) {
   int64_t n = 0, m = 0;
   if (!which) {
     n = voff[1];
@@ -1216,6 +1332,7 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   A.m = m;
   A.src = src;
   A.dst = dst;
+  A.ends = ends;
   A.w = w;
   A.wtype = wtype;
   const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
@@ -1231,7 +1348,7 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   while (A.vs < PAGE && ((warps * EVEN) << (A.vs + 1)) <= n) ++A.vs;
   const int64_t epages = (m + ((int64_t)1 << A.es) - 1) >> A.es, vpages = (n + ((int64_t)1 << A.vs) - 1) >> A.vs;
   A.classes = 1;
-  if (m >= 64 * SAMPLES) {
+  if (m >= (counts ? COUNT_CLASSES : 64 * SAMPLES)) {
     double la = CLASS1, lb = CLASS2;
     if (m < TWO_CLASSES) la = lb;
     if ((double)m > 1.25 * la * (double)n && la < lb) A.classes = 2;
@@ -1267,12 +1384,13 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   PinnedWords pin;
   if (int rc = pin.take(64 + tab_bytes)) return rc;
   pin.p[0] = 0x80000000u;  // not finished
+  pin.p[1] = counts ? 0x80000000u : 0u;
   A.ctl = (Ctrl *)(base + o_ctl);
   A.p = (int32_t *)(base + o_p);
   A.r = (unsigned long long *)(base + o_r);
   A.roots = (int32_t *)(base + o_roots);
   A.gbits = (uint32_t *)(base + o_gbits);
-  A.mbits = mask ? (uint32_t *)(base + o_bits) : nullptr;
+  A.mbits = mask || (counts && A.classes > 1) ? (uint32_t *)(base + o_bits) : nullptr;
   A.bins = (unsigned long long *)(base + o_ctl + 256);
   A.front = (unsigned *)(base + o_front);
   A.back = (unsigned *)(base + o_back);
@@ -1312,21 +1430,25 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   k_prepare<<<blocks, ET, 0, s>>>(A);
   const bool f32 = wtype == MSF_F32;
   void (*select)(Args) =
-      which ? (f32 ? (vec ? k_select<true, true, true> : k_select<false, true, true>)
-                   : (vec ? k_select<true, false, true> : k_select<false, false, true>))
-            : (f32 ? (vec ? k_select<true, true, false> : k_select<false, true, false>)
-                   : (vec ? k_select<true, false, false> : k_select<false, false, false>));
-  const void *rounds = which ? (const void *)k_rounds<true> : (const void *)k_rounds<false>;
+      which  ? (f32 ? (vec ? k_select<VECTOR, true, true> : k_select<SCALAR, true, true>)
+                    : (vec ? k_select<VECTOR, false, true> : k_select<SCALAR, false, true>))
+      : ends ? (f32 ? k_select<PAIRS, true, false> : k_select<PAIRS, false, false>)
+             : (f32 ? (vec ? k_select<VECTOR, true, false> : k_select<SCALAR, true, false>)
+                    : (vec ? k_select<VECTOR, false, false> : k_select<SCALAR, false, false>));
+  const void *rounds = which    ? (const void *)k_rounds<true, false>
+                       : counts ? (const void *)k_rounds<false, true>
+                                : (const void *)k_rounds<false, false>;
   select<<<blocks, ET, 0, s>>>(A);
   int phase = 0;
   void *args[] = {&A, &phase};
   cudaError_t e = cudaLaunchCooperativeKernel(rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
   if (e == cudaSuccess && A.classes > 2) {
     void (*filter)(Args) =
-        which ? (A.smem_bits ? (vec ? k_filter<true, true, true> : k_filter<false, true, true>)
-                             : (vec ? k_filter<true, false, true> : k_filter<false, false, true>))
-              : (A.smem_bits ? (vec ? k_filter<true, true, false> : k_filter<false, true, false>)
-                             : (vec ? k_filter<true, false, false> : k_filter<false, false, false>));
+        which  ? (A.smem_bits ? (vec ? k_filter<VECTOR, true, true> : k_filter<SCALAR, true, true>)
+                              : (vec ? k_filter<VECTOR, false, true> : k_filter<SCALAR, false, true>))
+        : ends ? (A.smem_bits ? k_filter<PAIRS, true, false> : k_filter<PAIRS, false, false>)
+               : (A.smem_bits ? (vec ? k_filter<VECTOR, true, false> : k_filter<SCALAR, true, false>)
+                              : (vec ? k_filter<VECTOR, false, false> : k_filter<SCALAR, false, false>));
     if (A.smem_bits)
       e = cudaFuncSetAttribute(filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BITS);
     if (e == cudaSuccess) {
@@ -1334,6 +1456,10 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
       phase = 1;
       e = cudaLaunchCooperativeKernel(rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
     }
+  }
+  if (e == cudaSuccess && counts && A.classes > 1) {
+    phase = 2;
+    e = cudaLaunchCooperativeKernel(rounds, dim3((unsigned)blocks), dim3(ET), args, 0, s);
   }
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // (a share of the device that holds fewer blocks)
     cudaGetLastError();
@@ -1345,9 +1471,35 @@ int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int6
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "forest of an edge list");
   const unsigned st = *(volatile unsigned *)pin.p;
-  if (st & 0x80000000u) return fail(MSF_ERR_CHECK, "device consistency check failed");
+  if ((st | pin.p[1]) & 0x80000000u) return fail(MSF_ERR_CHECK, "device consistency check failed");
   *status |= st;
+  if (counts) {
+    counts->hooked = (int32_t)pin.p[1];
+    counts->left = pin.p[2];
+    counts->edges = pin.p[3];
+    counts->passes = (int32_t)pin.p[4];
+    counts->kernels = 3 + (A.classes > 2 ? 2 : 0) + (A.classes > 1 ? 1 : 0);
+  }
   return MSF_OK;
+}
+
+}  // namespace
+
+// Forest of one graph from its edge list, or of K graphs of a batch, `which` of
+// the graphs with the host offsets voff, eoff (pointers the device can read).
+// Any output may be NULL.  Synchronizes `s`; *status: 1 = index out of range,
+// 2 = NaN weight.
+int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+                const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
+                unsigned *status, cudaStream_t s) {
+  return solve(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, status, nullptr, s);
+}
+
+int solve_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+                double *totals, LoopCounts *counts, cudaStream_t s) {
+  const int64_t voff[2] = {0, n}, eoff[2] = {0, m};
+  unsigned status = 0;
+  return solve(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, &status, counts, s);
 }
 
 }  // namespace msf
