@@ -709,10 +709,24 @@ int msf_connected_components(msf_graph *g, int32_t *labels, void *stream) {
   if (!g || !labels) return fail(MSF_ERR_INVALID_ARG, "NULL argument");
   DeviceGuard dg(g->device);
   cudaStream_t s = (cudaStream_t)stream;
-  int rc = ensure_workspace(g);
-  if (rc) return rc;
+  int rc;
   Staged sl;
   if ((rc = sl.output(labels, (size_t)g->n * 4))) return rc;
+  if (options().round_limit >= 64 && options().jump_limit >= 64) {
+    // the kernel over the edges stops at no round of the caller's and counts no
+    // jumps; the loop over the CSR takes those calls
+    int32_t rounds = 0;
+    rc = components_pairs(g->n, g->m, g->ends, (int32_t *)sl.dev, &rounds, s);
+    if (rc != MSF_ERR_OOM && rc != SOLVE_NOT_RUN) {
+      if (rc) return rc;
+      g->stats.cc_rounds = rounds;
+      if ((rc = sl.copy_back(s))) return rc;
+      if (sl.owned) MSF_CK(cudaStreamSynchronize(s));
+      return MSF_OK;
+    }
+    set_error("");
+  }
+  if ((rc = ensure_workspace(g))) return rc;
   DevState hs = make_state(g);
   hs.labels = (int32_t *)sl.dev;
   hs.mask = nullptr;

@@ -316,6 +316,11 @@ struct LoopCounts {
 int solve_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
                 double *totals, LoopCounts *counts, cudaStream_t s);
 
+// cc.cu
+// Connected components (smallest vertices) and the rounds the loop over the CSR
+// takes, from pairs of validated ends; MSF_ERR_OOM and SOLVE_NOT_RUN as above.
+int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, int32_t *rounds, cudaStream_t s);
+
 // small.cu
 // The same for graphs that each fit in one SM's shared memory (small_fits),
 // one block per graph.

@@ -42,11 +42,10 @@
 // ms.  Fractions around these (CLASS1 0.25 to 1, CLASS2 1.2 to 3): R-MAT 26
 // 20.7 to 22.9 ms, the grid 2.3 to 4.4, uniform 0.52 to 0.70, R-MAT 20 0.48 to
 // 0.54; a single light class of 1.5 n: 28.4, 3.2, 0.68 and 0.57 ms.
-#include <cuda/atomic>
-
 #include <cstring>
 
 #include "exact.cuh"
+#include "grid.cuh"
 #include "internal.cuh"
 
 namespace msf {
@@ -83,12 +82,7 @@ constexpr int64_t COUNT_CLASSES = 3 << 20;
 constexpr unsigned long long SMALL = 1 << 17;
 // Edges or vertices per block: a call that does not fill the device.
 constexpr int64_t BLOCK_SHARE = 1024;
-// Pages (see Pages) of 2^PAGE places at most, and smaller where a warp would get
-// fewer than EVEN of them (its share is even to one page).  4096 graphs of 20 M
-// edges: one range per warp 8.56 ms, pages of 128 7.0, by this rule 6.05, with
-// EVEN 4 6.18, with longer pages 6.12; R-MAT and lattice graphs 1-5 % faster
-// than with ranges.
-constexpr int PAGE = 10, EVEN = 16;
+
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
 struct Ctrl {
@@ -134,66 +128,9 @@ struct Args {
   unsigned *host;       // pinned: [0] status bits, [1..4] rounds with hooks, trees the last left, edges, passes
 };
 
-__device__ __forceinline__ int ld_rel(const int32_t *a) {
-  return cuda::atomic_ref<int, cuda::thread_scope_device>(*const_cast<int32_t *>(a)).load(cuda::memory_order_relaxed);
-}
-__device__ __forceinline__ void st_rel(int32_t *a, int v) {
-  cuda::atomic_ref<int, cuda::thread_scope_device>(*a).store(v, cuda::memory_order_relaxed);
-}
 __device__ __forceinline__ unsigned long long ld_rel64(const unsigned long long *a) {
   return cuda::atomic_ref<unsigned long long, cuda::thread_scope_device>(*const_cast<unsigned long long *>(a))
       .load(cuda::memory_order_relaxed);
-}
-
-// Edges and vertices are dealt to the warps in pages: warp w of W takes pages
-// w, w + W, ..., so that all warps work on one window of the arrays at a time
-// (an input with locality -- a lattice, a batch -- then keeps the parents and
-// minima it gathers in L2; with one contiguous range per warp every range's
-// vicinity is live at once).  `at(i)` is the i-th of the warp's elements, in
-// order; `cap` counts the places of its pages, `len` the elements below total.
-struct Pages {
-  uint32_t s, w, W, cap, len;
-  __device__ Pages(int64_t total, int32_t shift, int64_t warp, int64_t warps)
-      : s((uint32_t)shift), w((uint32_t)warp), W((uint32_t)warps) {
-    const int64_t pages = (total + ((int64_t)1 << s) - 1) >> s;
-    const int64_t mine = warp < pages ? (pages - warp + warps - 1) / warps : 0;
-    cap = (uint32_t)(mine << s);
-    len = cap;
-    if (mine > 0 && (pages - 1) % warps == warp) len -= (uint32_t)((pages << s) - total);  // the last page
-  }
-  __device__ __forceinline__ uint32_t page(uint32_t i) const { return (i >> s) * W + w; }
-  __device__ __forceinline__ int64_t at(uint32_t i) const {
-    return ((int64_t)page(i) << s) + (i & ((1u << s) - 1u));
-  }
-};
-
-// All blocks meet; false (everywhere, sooner or later) when a wait ran out.
-__device__ bool grid_barrier(Ctrl *c, int phase, unsigned &target) {
-  if (gridDim.x == 1) {
-    __syncthreads();
-    return true;
-  }
-  __shared__ unsigned ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    target += gridDim.x;
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> a(c->arrive[phase]), ab(c->abort);
-    __threadfence();
-    a.fetch_add(1u, cuda::memory_order_acq_rel);
-    unsigned good = 0;
-    for (unsigned it = 0; it < (1u << 25); ++it) {
-      if ((int)(a.load(cuda::memory_order_acquire) - target) >= 0) {
-        good = 1;
-        break;
-      }
-      if ((it & 1023u) == 1023u && ab.load(cuda::memory_order_relaxed)) break;
-    }
-    if (!good) ab.store(1u, cuda::memory_order_relaxed);
-    __threadfence();
-    ok = good;
-  }
-  __syncthreads();
-  return ok != 0;
 }
 
 // Root of x, whose parent y was read, by its chain.  Hooks happen in other
@@ -445,22 +382,6 @@ struct Quad {
 };
 // Forms of the edges: separate arrays of ends, aligned or not, or pairs.
 enum Form { SCALAR = 0, VECTOR = 1, PAIRS = 2 };
-__device__ __forceinline__ void load_pairs(const int2 *ends, int64_t e, int64_t hi, int4 &s, int4 &d) {
-  if (e + 4 <= hi) {
-    const int4 a = __ldcs(reinterpret_cast<const int4 *>(ends + e)), b = __ldcs(reinterpret_cast<const int4 *>(ends + e) + 1);
-    s = make_int4(a.x, a.z, b.x, b.z);
-    d = make_int4(a.y, a.w, b.y, b.w);
-    return;
-  }
-  int32_t *x = &s.x, *y = &d.x;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (e + j < hi) {
-      const int2 a = ends[e + j];
-      x[j] = a.x;
-      y[j] = a.y;
-    }
-}
 template <int FORM>
 __device__ __forceinline__ Quad load_quad(const Args &A, int64_t e, int64_t hi) {
   Quad q;
@@ -1025,7 +946,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
       }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) C->live[phase][(it + 2) & 3u] = 0;
-    if (!grid_barrier(C, phase, target)) return 0;
+    if (!grid_barrier(C->arrive + phase, &C->abort, target)) return 0;
     const unsigned long long t = ld_rel64(&C->live[phase][it & 3u]);
     ++it;
     return t;
@@ -1137,7 +1058,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     }
     __syncwarp();
     vc = out;
-    return grid_barrier(C, phase, target);
+    return grid_barrier(C->arrive + phase, &C->abort, target);
   };
   // Rounds on the warp's `cnt` entries until no edge is left; the minima of
   // the first one have been offered.  With few edges left the roots are not
@@ -1156,7 +1077,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
         if (tid == 0) C->pairs[(k + 2) & 3] = 0;
         ++hooked;
       }
-      if (!grid_barrier(C, phase, target)) return false;
+      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return false;
       if (!small) {
         if (!settle_roots()) return false;
         cnt = min_pass<true, false>(A, tab, P, 0u, cnt);
@@ -1172,7 +1093,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   unsigned cnt;
   if (COUNT && phase == 2) {
     cnt = list_forest(A, P, Q);
-    if (!grid_barrier(C, phase, target)) return;
+    if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
   } else {
     cnt = A.front[warp];
   }
@@ -1192,7 +1113,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   if (!last) {
     if (BATCH) {
       vote_giants(A, warp, nthr >> 5);
-      if (!grid_barrier(C, phase, target)) return;
+      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
     }
     flatten(true, BATCH ? 0 : vote_giant(A));
     if (lane == 0) A.back[warp] = vc;
@@ -1248,7 +1169,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
       if (tab.key[i] >= 0 && b != 0xffffffffu) atomicMin(reinterpret_cast<unsigned *>(A.r + tab.key[i]), b);
     }
   }
-  if (!grid_barrier(C, phase, target)) return;
+  if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
   if (!BATCH && A.totals && blockIdx.x == 0) {
     for (int i = threadIdx.x; i < 256; i += ET) sbins[i] = (long long)ld_rel64(A.bins + i);
     __syncthreads();
@@ -1285,7 +1206,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   if (BATCH) {
     batch_results(A, P);
     if (A.totals) {
-      if (!grid_barrier(C, phase, target)) return;
+      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
       // a warp per graph rounds its total
       for (int64_t g = warp; g < A.G; g += nthr >> 5) {
         const double t = combine_bins_warp(reinterpret_cast<const long long *>(A.bins) + g * 256, A.wtype);
@@ -1343,10 +1264,9 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   const int64_t cap = (int64_t)sm_count();
   const int blocks = (int)(want < cap ? want : cap);
   const int64_t warps = (int64_t)blocks * EW;
-  A.es = A.vs = 7;
-  while (A.es < PAGE && ((warps * EVEN) << (A.es + 1)) <= m) ++A.es;
-  while (A.vs < PAGE && ((warps * EVEN) << (A.vs + 1)) <= n) ++A.vs;
-  const int64_t epages = (m + ((int64_t)1 << A.es) - 1) >> A.es, vpages = (n + ((int64_t)1 << A.vs) - 1) >> A.vs;
+  A.es = page_shift(m, warps);
+  A.vs = page_shift(n, warps);
+  const int64_t epages = page_count(m, A.es), vpages = page_count(n, A.vs);
   A.classes = 1;
   if (m >= (counts ? COUNT_CLASSES : 64 * SAMPLES)) {
     double la = CLASS1, lb = CLASS2;
