@@ -361,9 +361,9 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
         int32_t x[U], y[U], a[U];
         bool any = false;
 #pragma unroll
-        for (int j = 0; j < U; ++j) x[j] = v0 + j * 32 + lane < n ? ld_rel(p + v0 + j * 32 + lane) : 0;
+        for (int j = 0; j < U; ++j) x[j] = v0 + j * 32 + lane < n ? ld_rel(p + v0 + j * 32 + lane) : -1;
 #pragma unroll
-        for (int j = 0; j < U; ++j) y[j] = __ldca(p + x[j]);
+        for (int j = 0; j < U; ++j) y[j] = x[j] >= 0 ? __ldca(p + x[j]) : -1;  // (no vertex: no chain)
 #pragma unroll
         for (int j = 0; j < U; ++j) {
           const int64_t v = v0 + j * 32 + lane;

@@ -72,3 +72,21 @@ def test_shapes(shape):
         d = np.concatenate([v[:-1].ravel(), v[:, :-1].ravel(), v[:, :, :-1].ravel()]).astype(np.int32)
         n = k ** 3
     check(n, s, d)
+
+
+def test_small_sparse_graphs():
+    """Many trees and rounds, vertex 0 often no root, the last page of the
+    vertices partly filled: labels and rounds of the step oracle."""
+    from oracle import as_cc
+    from paper_2110_04865_gb300 import api
+    rng = np.random.default_rng(0)
+    for _ in range(120):
+        n = int(rng.integers(2, 3000))
+        m = int(rng.integers(1, 3 * n))
+        s, d = (rng.integers(0, n, m).astype(np.int32) for _ in range(2))
+        g = api.Graph(n, to_dev(s), to_dev(d), to_dev(np.ones(m, np.float32)))
+        lb = g.components().cpu().numpy()
+        rounds = g.stats().cc_rounds
+        g.free()
+        ref = as_cc.as_cc(n, s, d)
+        assert np.array_equal(lb, ref["labels"]) and rounds == ref["rounds"]
