@@ -265,7 +265,7 @@ def ingest_traffic(args):
     """profiles/min_edge_traffic.json from the ncu CSV of
     `bench.py --profile-min-edge --workload W` run with the sweep shape in
     MSF_SPL / MSF_PREFETCH / MSF_BPS / MSF_SWEEP (the shape the autotuner
-    picks on W): the mean DRAM bytes (read + write) per captured k_sweep
+    picks on W): the mean DRAM bytes (read + write) per captured sweep
     launch, each after an L2 flush.  Entries for other shapes of the same
     workload and sources are kept."""
     import csv
@@ -275,16 +275,15 @@ def ingest_traffic(args):
     with open(args.ingest_traffic) as f:
         lines = [ln for ln in f if ln.startswith('"')]
     for r in csv.DictReader(lines):
-        # the sweep proper, not its relabelling instantiation (launched beside it,
-        # it returns at once outside the second round of a round loop)
-        if "k_sweep" not in r["Kernel Name"] or ", 1>(" in r["Kernel Name"]:
+        # msf_min_edge's own sweep, or the form that the shape asks for
+        if "k_min_sweep" not in r["Kernel Name"] and "k_sweep" not in r["Kernel Name"]:
             continue
         unit = {"byte": 1, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}.get(r.get("Metric Unit", "byte"), None)
         if r["Metric Name"] in ("dram__bytes_read.sum", "dram__bytes_write.sum") and unit:
             key = int(r["ID"])
             per[key] = per.get(key, 0.0) + float(r["Metric Value"].replace(",", "")) * unit
     if not per:
-        raise SystemExit("no k_sweep DRAM counters in the capture")
+        raise SystemExit("no sweep DRAM counters in the capture")
     shape = env_shape()
     src_hash = build_lib.source_hash(SWEEP_SOURCES)
     path = os.path.join(ROOT, "profiles", "min_edge_traffic.json")
@@ -301,10 +300,8 @@ def ingest_traffic(args):
                                                 ("BPS", shape["blocks_per_sm"]), ("SWEEP", shape["sweep"])))
     out = {"workload": args.workload, "source_hash": src_hash, "sources": list(SWEEP_SOURCES),
            "command": f"{env} ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
-                      f"--clock-control none -k regex:k_sweep -s 1 -c 4 --csv python bench.py --profile-min-edge "
-                      f"--workload {args.workload} --no-autotune  (each msf_min_edge call launches the sweep and "
-                      f"its relabelling instantiation, which returns at once outside a round loop's second "
-                      f"round and is left out: the 4 captured launches hold 2 sweeps)",
+                      f"--clock-control none -k regex:'k_min_sweep|k_sweep' -s 1 -c 2 --csv python bench.py "
+                      f"--profile-min-edge --workload {args.workload} --no-autotune",
            "captures": caps}
     with open(path, "w") as f:
         json.dump(out, f, indent=1)
@@ -326,7 +323,7 @@ def main():
                     help="only build the graph and run the min-edge sweep 4 times (for ncu)")
     ap.add_argument("--ingest-traffic", metavar="CSV",
                     help="read an ncu CSV of a --profile-min-edge capture (dram__bytes_read.sum, "
-                         "dram__bytes_write.sum of k_sweep, the shape in MSF_SPL/MSF_PREFETCH/MSF_BPS/"
+                         "dram__bytes_write.sum of the sweep, the shape in MSF_SPL/MSF_PREFETCH/MSF_BPS/"
                          "MSF_SWEEP) and write profiles/min_edge_traffic.json")
     ap.add_argument("--profile-build", action="store_true",
                     help="only build (and free) the CSR 3 times (for ncu)")

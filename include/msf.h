@@ -292,9 +292,11 @@ enum msf_option {
   MSF_OPT_COMPACT_TAU = 0,   /* compact when live slots < tau * slots (0 < tau < 1; default 0.5; 0 = never) */
   MSF_OPT_ROUND_LIMIT = 1,   /* maximum rounds (default 64) */
   MSF_OPT_JUMP_LIMIT = 2,    /* maximum shortcut passes per round (default 64) */
-  MSF_OPT_SLOTS_PER_LANE = 3,/* min-edge tile: slots per lane, 4, 8 or 16 (default 4) */
+  MSF_OPT_SLOTS_PER_LANE = 3,/* min-edge tile: slots per lane, 4, 8 or 16 (default 4;
+                                msf_min_edge then takes 8 where rows are long enough) */
   MSF_OPT_BLOCKS_PER_SM = 4, /* min-edge grid: resident blocks per SM (1..8, default 4) */
-  MSF_OPT_PREFETCH = 5,      /* min-edge sweep loads the next tile early: 0 or 1 (default 0) */
+  MSF_OPT_PREFETCH = 5,      /* the round loop's sweep loads the next tile early: 0 or 1
+                                (default 0) */
   MSF_OPT_EXEC_MODE = 6,     /* 0 = device round loop in a CUDA graph (default); 1 = host-driven
                                 loop, one launch per kernel and a host wait per decision (for
                                 profiling kernels individually) */

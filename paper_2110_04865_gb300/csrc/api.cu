@@ -448,6 +448,57 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
   return MSF_OK;
 }
 
+// msf_min_edge by the sweep made for it (whole call, loop's sweep with a state, two
+// waits and a copy around it / this: R-MAT 20 203 / 131 us, uniform 2^24 edges 222
+// / 134, 5000 vertices 79 / 43); an option that asks for another form gets that
+// one.  The loop's tile prefetch would cost it registers and time (104 us against
+// 90 in the kernel), so that option is the loop's alone.
+bool plain_sweep() {
+  const Options &o = options();
+  return !o.pairwise && o.sweep == 0;
+}
+
+// One application over the slots [s0, s1) of the graph's CSR (s0 a multiple of
+// SLOT_PAD).  One wait: the check of the parents is read with the result.
+int min_edge_slots(msf_graph *g, const int32_t *p, int64_t s0, int64_t s1, uint64_t *r, cudaStream_t s) {
+  if (g->n == 0) return MSF_OK;
+  int err = MSF_OK;
+  char *base = (char *)pool_alloc((size_t)(g->nrows0 + 1) * 4 + 256, &err);
+  if (err) return err;
+  PoolBlock back{base};
+  PinnedWords pin;
+  if (int rc = pin.take(64)) return rc;
+  unsigned *bad = (unsigned *)base;
+  int32_t *prow = (int32_t *)(base + 256);
+  CsrBuf B = g->csr0;
+  B.col += s0;
+  B.key += s0;
+  B.tile_row += s0 / TB;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaError_t e = cudaMemsetAsync(bad, 0, 8, s);
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
+  if (e == cudaSuccess) {
+    launch_min_check(p, g->n, B, g->nrows0, prow, bad, pin.p, r, s);
+    e = cudaEventRecord(ev[0], s);
+  }
+  if (e == cudaSuccess && s1 > s0)
+    launch_min_sweep(p, g->n, B, s1 - s0, g->nrows0, prow, bad, pin.p, r, options().spl, options().blocks_per_sm, s);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaEventRecord(ev[1], s);
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
+  float ms = 0.f;
+  if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+  for (cudaEvent_t x : ev)
+    if (x) cudaEventDestroy(x);
+  if (e != cudaSuccess) return cuda_fail(e, "min-edge sweep");
+  const volatile unsigned *st = pin.p;
+  if (st[0]) return fail(MSF_ERR_INVALID_ARG, "parent value outside [0, n)");
+  if (st[1]) return fail(MSF_ERR_CHECK, "min-edge sweep reported an inconsistent CSR");
+  if (s1 > s0) g->stats.min_edge_ms = ms;
+  return MSF_OK;
+}
+
 int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t *src, const int32_t *dst,
              const void *w, int wtype, uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
   const int64_t n = voff[G], m = eoff[G];
@@ -558,6 +609,12 @@ int msf_min_edge(msf_graph *g, const int32_t *parent, uint64_t *r, void *stream)
   Staged sp, sr;
   if ((rc = sp.input(parent, (size_t)g->n * 4, s))) return rc;
   if ((rc = sr.output(r, (size_t)g->n * 8))) return rc;
+  if (plain_sweep()) {
+    if ((rc = min_edge_slots(g, (const int32_t *)sp.dev, 0, g->nnz0, (uint64_t *)sr.dev, s))) return rc;
+    if ((rc = sr.copy_back(s))) return rc;
+    if (sr.owned) MSF_CK(cudaStreamSynchronize(s));
+    return MSF_OK;
+  }
   int err = MSF_OK;
   int *flag = (int *)pool_alloc(16, &err);
   if (err) return err;
@@ -609,6 +666,21 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
   Staged sp, sr;
   if ((rc = sp.input(parent, (size_t)g->n * 4, s))) return rc;
   if ((rc = sr.output(r, (size_t)g->n * 8))) return rc;
+  // the part's slots [s0, s1): cuts at multiples of SLOT_PAD, so that every
+  // tile of the sweep (at most SLOT_PAD slots) lies inside one part
+  const int64_t nnz = g->nnz0;
+  auto cut = [&](int64_t k) -> int64_t {
+    if (k >= nparts) return nnz;
+    const int64_t c = (int64_t)((__int128)k * nnz / nparts);
+    return c / SLOT_PAD * SLOT_PAD;
+  };
+  const int64_t s0 = cut(part), s1 = cut((int64_t)part + 1);
+  if (plain_sweep()) {
+    if ((rc = min_edge_slots(g, (const int32_t *)sp.dev, s0, s1, (uint64_t *)sr.dev, s))) return rc;
+    if ((rc = sr.copy_back(s))) return rc;
+    if (sr.owned) MSF_CK(cudaStreamSynchronize(s));
+    return MSF_OK;
+  }
   int err = MSF_OK;
   int *flag = (int *)pool_alloc(16, &err);
   if (err) return err;
@@ -624,15 +696,6 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
   if (e != cudaSuccess) return cuda_fail(e, "checking parent");
   if (hflag) return fail(MSF_ERR_INVALID_ARG, "parent value outside [0, n)");
   if (g->n > 0) MSF_CK(cudaMemsetAsync(sr.dev, 0xff, (size_t)g->n * 8, s));
-  // the part's slots [s0, s1): cuts at multiples of SLOT_PAD, so that every
-  // tile of the sweep (at most SLOT_PAD slots) lies inside one part
-  const int64_t nnz = g->nnz0;
-  auto cut = [&](int64_t k) -> int64_t {
-    if (k >= nparts) return nnz;
-    const int64_t c = (int64_t)((__int128)k * nnz / nparts);
-    return c / SLOT_PAD * SLOT_PAD;
-  };
-  const int64_t s0 = cut(part), s1 = cut((int64_t)part + 1);
   if (s1 > s0) {
     if ((rc = ensure_workspace(g))) return rc;
     DevState hs;

@@ -264,6 +264,13 @@ int radix_build_csr(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, i
 // change of p and before the sweep (use_star: rows outside stars get -1).
 void launch_prow(DevState *st, int use_star, cudaStream_t s);
 void launch_min_edge(DevState *st, int spl, int blocks_per_sm, int prefetch, cudaStream_t s, int pairwise = 0);
+// msf_min_edge without a loop's state: the parents checked (*bad, *host) and the
+// rows' parents, r cleared; then the sweep of the slots of B (host[1]: the CSR is
+// inconsistent).  Both leave r alone when *bad is set.
+void launch_min_check(const int32_t *p, int64_t n, const CsrBuf &B, int64_t nrows, int32_t *prow, unsigned *bad,
+                      unsigned *host, uint64_t *r, cudaStream_t s);
+void launch_min_sweep(const int32_t *p, int64_t n, const CsrBuf &B, int64_t nnz, int64_t nrows, const int32_t *prow,
+                      const unsigned *bad, unsigned *host, uint64_t *r, int spl, int blocks_per_sm, cudaStream_t s);
 void launch_compact(DevState *st, int spl, int blocks_per_sm, cudaStream_t s);
 
 // rounds.cu

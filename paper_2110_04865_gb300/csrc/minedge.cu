@@ -939,6 +939,182 @@ __global__ void __launch_bounds__(256) k_pair_gather(DevState *st) {
   }
 }
 
+// ---- one application on its own (msf_min_edge) -------------------------------------
+
+// Range check of the parents, and the parents of the CSR's rows.
+__global__ void __launch_bounds__(256) k_min_check(const int32_t *p, int64_t n, const int32_t *rows, int64_t nrows,
+                                                   int32_t *prow, unsigned *bad, unsigned *host) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  bool out = false;
+  for (int64_t i = i0; i < n; i += stride) out |= (uint32_t)p[i] >= (uint32_t)n;
+  for (int64_t k = i0; k < nrows; k += stride) prow[k] = p[rows[k]];
+  if (out) bad[0] = *host = 1u;
+  if (blockIdx.x == 0) {
+    // bad[1]: the most frequent of 256 sampled parents makes a sixteenth of them
+    __shared__ int32_t sample[256];
+    sample[threadIdx.x] = p[(int64_t)((uint64_t)threadIdx.x * (uint64_t)n >> 8)];
+    __syncthreads();
+    int c = 0;
+    for (int i = 0; i < 256; ++i) c += sample[i] == sample[threadIdx.x];
+    if (__syncthreads_or(c >= 16) && threadIdx.x == 0) bad[1] = 1u;
+  }
+}
+__global__ void __launch_bounds__(256) k_min_clear(uint64_t *r, int64_t n, const unsigned *bad) {
+  if (*bad) return;  // (a refused call leaves r as it was)
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) r[i] = KEY_INF;
+}
+
+// The sweep without a loop around it: no count of live slots is wanted, so a
+// lane takes the smallest key of its slots of a row first and gathers the parent
+// of that column only; the other columns' parents matter where that slot lies
+// inside a tree, and then the warp goes through the tile slot by slot (and
+// through the next ones, without trying first).  A gathered parent is one L1
+// wavefront per lane: 33.5 M of them were the sweep's bound (R-MAT 20, a seventh
+// of the vertices roots).
+struct MinArgs {
+  const int32_t *col, *tile_row, *prow, *p;
+  const uint64_t *key;
+  unsigned long long *r;
+  int64_t nnz, nrows;
+  uint32_t nv;
+  const unsigned *bad;  // [0] a parent is out of range, [1] there is a large tree
+  unsigned *host;       // pinned: [1] inconsistent CSR
+};
+constexpr int SLOT_BY_SLOT = 8;  // tiles gone through slot by slot after a failed try
+template <int V, bool LARGE>
+__device__ __forceinline__ void min_sweep(const MinArgs &A) {
+  constexpr int S = 32 * V;
+  constexpr int F = S / TB;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t ntiles = (A.nnz + S - 1) / S, tstride = (int64_t)gridDim.x * WARPS;
+  const int32_t *__restrict__ p = A.p;
+  unsigned long long *r = A.r;
+  CsrBuf B{};
+  B.key = const_cast<uint64_t *>(A.key);
+  // (a large tree's root keeps its minimum in L1: what is not below the copy needs
+  // no atomic)
+  auto emit = [&](int32_t root, unsigned long long v) {
+    if (!LARGE || v < __ldca(r + root)) atomicMin(r + root, v);
+  };
+  int slow = 0;  // tiles left to go through slot by slot
+  for (int64_t t = (int64_t)blockIdx.x * WARPS + wid; t < ntiles; t += tstride) {
+    const int64_t sl = t * S + (int64_t)lane * V;
+    int32_t c[V];
+    uint64_t k[V];
+    load_tile<V, true>(B, A.col, sl, c, k);
+    int32_t k0 = A.tile_row[t * F];
+    // row starts among the lane's slots; its first slot's row
+    uint32_t hv = 0;
+#pragma unroll
+    for (int j = 0; j < V; ++j) hv |= ((uint32_t)c[j] >> 31) << j;
+    const int cnt = __popc(hv);
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(FULL, incl, d);
+      if (lane >= d) incl += o;
+    }
+    const int head0 = __shfl_sync(FULL, (int)(hv & 1u), 0);
+    int R = 1 + __shfl_sync(FULL, incl, 31) - head0;  // rows meeting the tile
+    const int rbase = incl - cnt + (int)(hv & 1u) - head0;
+    const int nxt = __shfl_down_sync(FULL, (int)(hv & 1u), 1);
+    const bool next_head = (lane == 31) || nxt;
+    const bool first_head = (lane == 0) || (hv & 1u);
+    if (k0 < 0 || (int64_t)k0 + R > A.nrows) {  // impossible for a consistent CSR
+      A.host[1] = 1u;
+      k0 = k0 < 0 ? 0 : (k0 >= A.nrows ? (int32_t)(A.nrows - 1) : k0);
+      R = (int)((int64_t)k0 + R > A.nrows ? A.nrows - k0 : R);
+    }
+    const int32_t *prow_t = A.prow + k0;
+    const int rb0 = rbase < 0 ? 0 : rbase;
+    auto row_parent = [&](int i) { return __ldg(prow_t + (i < R ? i : R - 1)); };
+    const int32_t pi0 = row_parent(rb0);
+    unsigned long long lead, cur;
+    bool brk;
+    int32_t pi;
+#pragma unroll 1
+    for (bool by_slot = slow > 0;;) {
+      if (by_slot) {  // slots inside a tree out
+        int32_t pj[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) pj[j] = __ldg(p + (c[j] & (int32_t)COL_MASK));
+        int rb = rb0;
+        pi = pi0;
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          if (j > 0 && ((hv >> j) & 1u)) pi = row_parent(++rb);
+          if (pj[j] == pi) k[j] = KEY_INF;
+        }
+      }
+      // running minima of the rows; the columns of the last ones' parents
+      int32_t pj[V];
+#pragma unroll
+      for (int j = 1; j < V; ++j) {
+        if (!((hv >> j) & 1u) && k[j - 1] < k[j]) {
+          k[j] = k[j - 1];
+          c[j] = c[j - 1];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        const bool end = j == V - 1 || ((hv >> (j + 1)) & 1u);
+        pj[j] = end && !by_slot && k[j] != KEY_INF ? __ldg(p + (c[j] & (int32_t)COL_MASK)) : -1;
+      }
+      bool inside = false;  // a row's smallest slot lies inside a tree
+      int rb = rb0;
+      lead = KEY_INF;
+      brk = false;
+      pi = pi0;
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        if (j > 0 && ((hv >> j) & 1u)) {
+          const bool in = pj[j - 1] == pi;
+          inside |= in;
+          if (!brk) lead = k[j - 1];
+          else if (!in && k[j - 1] != KEY_INF && (uint32_t)pi < A.nv) emit(pi, k[j - 1]);
+          brk = true;
+          pi = row_parent(++rb);
+        }
+      }
+      inside |= pj[V - 1] == pi;
+      cur = k[V - 1];
+      if (by_slot || !__any_sync(FULL, inside)) break;
+      by_slot = true;
+      slow = SLOT_BY_SLOT + 1;
+      load_tile<V, true>(B, A.col, sl, c, k);
+    }
+    if (slow > 0) --slow;
+    // segmented inclusive min-scan of the trailing segments across lanes
+    unsigned long long agg = cur;
+    int f = (brk || first_head) ? 1 : 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long oa = __shfl_up_sync(FULL, agg, d);
+      const int of = __shfl_up_sync(FULL, f, d);
+      if (lane >= d) {
+        if (!f) agg = umin64(agg, oa);
+        f |= of;
+      }
+    }
+    unsigned long long prev = __shfl_up_sync(FULL, agg, 1);
+    if (lane == 0) prev = KEY_INF;
+    if (brk) {
+      const unsigned long long v = first_head ? lead : umin64(prev, lead);
+      if (v != KEY_INF && (uint32_t)pi0 < A.nv) emit(pi0, v);
+    }
+    if (next_head && agg != KEY_INF && (uint32_t)pi < A.nv) emit(pi, agg);
+  }
+}
+// With a large tree (half of the vertices in one, R-MAT 20: 343 -> 184 us for the
+// look before the atomic) and without (the look costs 12 us of 131 there).
+template <int V>
+__global__ void __launch_bounds__(THREADS, (V >= 16 ? 2 : 4)) k_min_sweep(const __grid_constant__ MinArgs A) {
+  if (A.bad[0]) return;
+  if (A.bad[1]) min_sweep<V, true>(A);
+  else min_sweep<V, false>(A);
+}
+
 // ---- compaction helpers ---------------------------------------------------------
 
 __global__ void k_cmp_prep(DevState *st, int S) {
@@ -1108,6 +1284,30 @@ void launch_min_edge(DevState *st, int spl, int blocks_per_sm, int prefetch, cud
       case 16: launch_sweep<16, MIN_EDGE, 0>(st, grid, b, s); break;
       default: launch_sweep<8, MIN_EDGE, 0>(st, grid, b, s); break;
     }
+  }
+}
+
+void launch_min_check(const int32_t *p, int64_t n, const CsrBuf &B, int64_t nrows, int32_t *prow, unsigned *bad,
+                      unsigned *host, uint64_t *r, cudaStream_t s) {
+  const int64_t work = (n > nrows ? n : nrows) / 256 + 1, cap = (int64_t)sm_count() * 8;
+  const int grid = (int)(work < cap ? work : cap);
+  k_min_check<<<grid, 256, 0, s>>>(p, n, B.rows, nrows, prow, bad, host);
+  k_min_clear<<<grid, 256, 0, s>>>(r, n, bad);
+}
+
+void launch_min_sweep(const int32_t *p, int64_t n, const CsrBuf &B, int64_t nnz, int64_t nrows, const int32_t *prow,
+                      const unsigned *bad, unsigned *host, uint64_t *r, int spl, int blocks_per_sm, cudaStream_t s) {
+  const MinArgs A{B.col, B.tile_row, prow, p, B.key, (unsigned long long *)r, nnz, nrows, (uint32_t)n, bad, host};
+  // 8 slots a lane by default (R-MAT 20 90 us, 4 slots 120; a 96^3 lattice 22 and
+  // 26), 4 where rows have fewer slots than that (12 us at 2.4 a row, 8 slots 14)
+  if (spl == 4 && nnz >= 4 * nrows) spl = 8;
+  const int64_t tiles = (nnz + 32 * spl - 1) / (32 * spl), want = (tiles + WARPS - 1) / WARPS;
+  const int64_t cap = (int64_t)sm_count() * blocks_per_sm;
+  const int grid = (int)(want < cap ? (want > 0 ? want : 1) : cap);
+  switch (spl) {
+    case 4: k_min_sweep<4><<<grid, THREADS, 0, s>>>(A); break;
+    case 16: k_min_sweep<16><<<grid, THREADS, 0, s>>>(A); break;
+    default: k_min_sweep<8><<<grid, THREADS, 0, s>>>(A); break;
   }
 }
 
