@@ -819,12 +819,24 @@ int msf_weight_backward(int64_t m, int32_t G, const int64_t *eoff, const uint8_t
   cudaStream_t s = (cudaStream_t)stream;
   int rc;
   Staged se, sm, sg, sw;
-  if (G > 1 && (rc = se.input(eoff, (size_t)(G + 1) * 8, s))) return rc;
+  // few graphs: their offsets go with the launch (eoff is read here)
+  const bool few = G <= BACKWARD_GRAPHS && m <= MAX_M && !(G > 1 && is_device_ptr(eoff));
+  if (!few && G > 1 && (rc = se.input(eoff, (size_t)(G + 1) * 8, s))) return rc;
   if ((rc = sm.input(edge_mask, (size_t)m, s))) return rc;
   if ((rc = sg.input(grad_total, (size_t)G * 8, s))) return rc;
   if ((rc = sw.output(grad_w, (size_t)m * 4))) return rc;
-  launch_backward(m, G, (const int64_t *)se.dev, (const uint8_t *)sm.dev, (const double *)sg.dev,
-                  (float *)sw.dev, s);
+  if (few) {
+    BackwardOffsets off;
+    for (int32_t g = 0; g + 1 < G; ++g) {
+      const int64_t e = eoff[g + 1];
+      off.end[g] = e < 0 ? 0u : e > MAX_M ? 0xffffffffu : (uint32_t)e;
+    }
+    off.end[G - 1] = 0xffffffffu;
+    launch_backward_few(off, m, G, (const uint8_t *)sm.dev, (const double *)sg.dev, (float *)sw.dev, s);
+  } else {
+    launch_backward(m, G, (const int64_t *)se.dev, (const uint8_t *)sm.dev, (const double *)sg.dev,
+                    (float *)sw.dev, s);
+  }
   MSF_CK(cudaGetLastError());
   if ((rc = sw.copy_back(s))) return rc;
   if (se.owned || sm.owned || sg.owned || sw.owned) MSF_CK(cudaStreamSynchronize(s));

@@ -296,6 +296,13 @@ void launch_mask_from_keys(DevState *st, cudaStream_t s);
 void launch_load_state(DevState *slot, const DevState &host, cudaStream_t s);
 void launch_backward(int64_t m, int32_t G, const int64_t *eoff_d, const uint8_t *mask,
                      const double *gt, float *gw, cudaStream_t s);
+// The same for G <= BACKWARD_GRAPHS graphs and m < 2^32 - 1.
+constexpr int BACKWARD_GRAPHS = 960;  // with the other arguments within 4 KB of parameters
+struct BackwardOffsets {
+  uint32_t end[BACKWARD_GRAPHS];  // first edge behind each graph
+};
+void launch_backward_few(const BackwardOffsets &off, int64_t m, int32_t G, const uint8_t *mask, const double *gt,
+                         float *gw, cudaStream_t s);
 void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cudaStream_t s);
 
 // solve.cu
