@@ -44,13 +44,13 @@ constexpr int ROUND_CAP = 64;
 constexpr size_t CC_BITS = 224 << 10;  // largest bitmap kept in shared memory
 // Entries of the lists from which a round's first step reads the giant tree's
 // bitmap before the parents (its making costs about 7 us at 2^20 vertices).
-constexpr unsigned LONG_LIST = 1u << 20;
+constexpr unsigned LONG_LIST = 1u << 12;  // (in units of 256)
 constexpr uint32_t NONE = 0xffffffffu;
 constexpr int64_t BLOCK_SHARE = 1024;  // edges or vertices per block: a call that does not fill the device
 
 struct CcCtrl {
-  unsigned arrive, abort;
-  unsigned sum[4], list[4];  // grid sums, by number modulo 4
+  unsigned long long arrive[2];
+  unsigned abort;
 };
 
 struct CcArgs {
@@ -93,7 +93,7 @@ __device__ __forceinline__ void offer(uint32_t *q, int32_t root, int32_t parent)
 
 __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ CcArgs A) {
   extern __shared__ uint32_t dyn[];
-  __shared__ unsigned s_sum, s_list;
+  __shared__ unsigned s_list;
   __shared__ int32_t vote[VOTES];
   __shared__ unsigned best;
   CcCtrl *C = A.ctl;
@@ -105,37 +105,34 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
   const int64_t n = A.n, m = A.m;
   int32_t *p = A.p;
   uint32_t *q = A.q;
-  unsigned target = 0, it = 0;
+  __shared__ GridBarrier bar;
   constexpr int U = 4;
-  auto barrier = [&]() { return grid_barrier(&C->arrive, &C->abort, target); };
-  // Barrier with the sums of the threads' counts and of the warps' lists.
+  auto barrier = [&]() { return bar.meet(); };
+  // Barrier; whether a thread of the grid has `some`, and the length of all lists
+  // in units of 256 entries a block.
   unsigned cnt = 0;   // entries of the warp's list
-  unsigned live = 0;  // of all
+  unsigned live = 0;  // of all, in those units
   int32_t giant = -1;
-  auto total = [&](unsigned c, unsigned &sum) -> bool {
-    c = __reduce_add_sync(FULL, c);
-    if (lane == 0 && c) atomicAdd(&s_sum, c);
+  auto total = [&](bool some, bool &any) -> bool {
     if (lane == 0 && cnt) atomicAdd(&s_list, cnt);
-    __syncthreads();
+    some = __syncthreads_or(some);
+    unsigned long long mine = 0;
     if (threadIdx.x == 0) {
-      if (s_sum) atomicAdd(&C->sum[it & 3u], s_sum);
-      if (s_list) atomicAdd(&C->list[it & 3u], s_list);
-      s_sum = s_list = 0;
-      if (blockIdx.x == 0) C->sum[(it + 2) & 3u] = C->list[(it + 2) & 3u] = 0;
+      mine = ((unsigned long long)(some ? 1u : 0u) << 36) + (s_list >> 8);
+      s_list = 0;
     }
-    if (!barrier()) return false;
-    sum = *(volatile unsigned *)&C->sum[it & 3u];
-    live = *(volatile unsigned *)&C->list[it & 3u];
-    ++it;
+    if (!bar.meet(mine)) return false;
+    any = bar.sum >> 36 != 0;
+    live = (unsigned)(bar.sum & ((1ull << 36) - 1ull));
     return true;
   };
   // The warp's vertices in groups of U * 32 (a group lies in one page).
   auto vertices = [&](auto f) {
     for (uint32_t i = 0; i < Q.cap; i += 32 * U) f(Q.at(i));
   };
-  // Roots with an offer take it; returns their number.
-  auto hook = [&]() -> unsigned {
-    unsigned c = 0;
+  // Roots with an offer take it; whether one of the thread's did.
+  auto hook = [&]() -> bool {
+    bool c = false;
     vertices([&](int64_t v0) {
       uint32_t x[U];
 #pragma unroll
@@ -146,7 +143,7 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
         const int64_t v = v0 + j * 32 + lane;
         q[v] = NONE;
         p[v] = (int32_t)x[j];
-        ++c;
+        c = true;
       }
     });
     return c;
@@ -205,7 +202,10 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
     return out;
   };
 
-  if (threadIdx.x == 0) s_sum = s_list = 0;
+  if (threadIdx.x == 0) {
+    s_list = 0;
+    bar.init(C->arrive, &C->abort);
+  }
   vertices([&](int64_t v0) {
 #pragma unroll
     for (int j = 0; j < U; ++j) {
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
       cnt = conditional_list();
     }
     if (!barrier()) return;
-    unsigned hooks;
+    bool hooks;
     if (!total(hook(), hooks)) return;
     if (!hooks) break;  // (every tree is a star: the second step finds no other)
     // starcheck: a vertex whose parent is no root marks its grandparent; a tree
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
         for (int j = 0; j < U; ++j)
           if (a[j] != x[j]) st_rel(p + v0 + j * 32 + lane, a[j]);
       });
-      unsigned left;
+      bool left;
       if (!total(more, left)) return;
       if (!left) break;
     }

@@ -52,34 +52,62 @@ struct Pages {
   }
 };
 
-// All blocks meet; false (everywhere, sooner or later) when a wait ran out.
-__device__ bool grid_barrier(unsigned *arrive, unsigned *abort, unsigned &target) {
-  if (gridDim.x == 1) {
+// Barriers of a cooperative grid's blocks, with a sum on the way: an arrival adds 1
+// above the block's addend, so the word that says that all have come also holds the
+// sum (two words in turn: a block arrives at the next barrier but one only after all
+// have read this one's).  An arrival takes the block's addend of the word's last
+// barrier out again, so a sum is that of one barrier; until all have come it may be
+// negative, which makes the count above too small, never too large.  The wait is
+// bounded.  One block's barrier is about 2 us of
+// latency; what the words save is measured on whole calls, fences around the
+// arrival, a counter and its read beside it before, this after: R-MAT 16
+// 203 -> 173 us, R-MAT 20 500 -> 455, uniform m = 16 n 553 -> 505.
+struct GridBarrier {  // in shared memory
+  static constexpr int SHIFT = 46;  // arrivals above (1700 barriers of 152 blocks), sums below
+  unsigned long long *word;         // [2], zero at the start
+  unsigned *abort;                  // a wait ran out somewhere
+  unsigned long long come[2], added[2], sum;  // arrivals awaited, the block's addends
+  unsigned k, ok;
+  __device__ void init(unsigned long long *w, unsigned *a) {  // (one thread; the block meets behind it)
+    word = w;
+    abort = a;
+    come[0] = come[1] = added[0] = added[1] = 0;
+    k = 0;
+  }
+  // All blocks meet; thread 0's `add` (below 2^38) summed up over them into `sum`.  False
+  // (everywhere, sooner or later) when a wait ran out.
+  __device__ bool meet(unsigned long long add = 0) {
     __syncthreads();
-    return true;
-  }
-  __shared__ unsigned ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    target += gridDim.x;
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> a(*arrive), ab(*abort);
-    __threadfence();
-    a.fetch_add(1u, cuda::memory_order_acq_rel);
-    unsigned good = 0;
-    for (unsigned it = 0; it < (1u << 25); ++it) {
-      if ((int)(a.load(cuda::memory_order_acquire) - target) >= 0) {
-        good = 1;
-        break;
+    if (threadIdx.x == 0) {
+      if (gridDim.x == 1) {
+        sum = add;
+        ok = 1;
+      } else {
+        cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> a(word[k & 1u]);
+        cuda::atomic_ref<unsigned, cuda::thread_scope_device> ab(*abort);
+        const unsigned long long all = come[k & 1u] += gridDim.x;
+        // (released with the block's writes: it met before)
+        a.fetch_add((1ull << SHIFT) + add - added[k & 1u], cuda::memory_order_release);
+        added[k & 1u] = add;
+        unsigned good = 0;
+        for (unsigned it = 0; it < (1u << 25); ++it) {
+          const unsigned long long v = a.load(cuda::memory_order_acquire);
+          if ((v >> SHIFT) >= all) {
+            sum = v & ((1ull << SHIFT) - 1ull);
+            good = 1;
+            break;
+          }
+          if ((it & 1023u) == 1023u && ab.load(cuda::memory_order_relaxed)) break;
+        }
+        if (!good) ab.store(1u, cuda::memory_order_relaxed);
+        ++k;
+        ok = good;
       }
-      if ((it & 1023u) == 1023u && ab.load(cuda::memory_order_relaxed)) break;
     }
-    if (!good) ab.store(1u, cuda::memory_order_relaxed);
-    __threadfence();
-    ok = good;
+    __syncthreads();
+    return ok != 0;
   }
-  __syncthreads();
-  return ok != 0;
-}
+};
 
 // Edges e to e + 4 (or hi) of pairs of ends, 16-byte aligned.
 __device__ __forceinline__ void load_pairs(const int2 *ends, int64_t e, int64_t hi, int4 &s, int4 &d) {

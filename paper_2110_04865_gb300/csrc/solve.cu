@@ -86,10 +86,9 @@ constexpr int64_t BLOCK_SHARE = 1024;
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
 struct Ctrl {
-  unsigned arrive[3];  // grid barriers of the rounds kernels
+  unsigned long long arrive[3][2];  // grid barriers of the rounds kernels
   unsigned abort;      // a barrier wait ran out
   unsigned err;        // 1 = index out of range, 2 = NaN weight
-  unsigned long long live[3][4];  // edges left, by round modulo 4, of the rounds kernels
   unsigned pairs[4];   // trees formed, by round modulo 4
   unsigned edges;      // forest edges
   unsigned long long thresh[2];  // keys of the first class lie below [0], of the second below [1]
@@ -897,21 +896,23 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     if (blockIdx.x == 0 && threadIdx.x == 0) A.host[0] = C->err;
     return;
   }
-  unsigned target = 0;
+  __shared__ GridBarrier bar;
   const int64_t tid = (int64_t)blockIdx.x * ET + threadIdx.x, nthr = (int64_t)gridDim.x * ET;
   const int64_t warp = tid >> 5;
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
   unsigned long long usum = 0;  // uint32 weights of the thread's forest edges
   sums.clear();
-  if (threadIdx.x == 0) s_live = s_pairs = s_edges = 0;
+  if (threadIdx.x == 0) {
+    s_live = s_pairs = s_edges = 0;
+    bar.init(C->arrive[phase], &C->abort);
+  }
   table_clear(tab);
   __syncthreads();
   // the warp's vertices and its list of roots (all of them, or what the
   // flattening before the filter left)
   const Pages P(A.m, A.es, warp, nthr >> 5), Q(A.n, A.vs, warp, nthr >> 5);
   unsigned vc = phase == 1 ? A.back[warp] : Q.len;
-  unsigned it = 0;  // counter of the grid sums
   // the rounds are counted: those of phase 2, or of the only class
   const bool counting = COUNT && (phase == 2 || A.classes == 1);
   unsigned *pair_slot = C->pairs;
@@ -936,8 +937,9 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
       if (k >= 0 && v < ld_rel64(A.r + k)) atomicMin(A.r + k, v);
     }
     table_clear(tab);  // (the thread's own slots)
+    unsigned mine = 0;
     if (threadIdx.x == 0) {
-      if (s_live) atomicAdd(&C->live[phase][it & 3u], (unsigned long long)s_live);
+      mine = s_live;
       s_live = 0;
       if (COUNT) {
         if (s_pairs) atomicAdd(pair_slot, s_pairs);
@@ -945,11 +947,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
         s_pairs = s_edges = 0;
       }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) C->live[phase][(it + 2) & 3u] = 0;
-    if (!grid_barrier(C->arrive + phase, &C->abort, target)) return 0;
-    const unsigned long long t = ld_rel64(&C->live[phase][it & 3u]);
-    ++it;
-    return t;
+    return bar.meet(mine) ? bar.sum : 0ull;
   };
   // The roots that hooked point to their new roots (Algorithm 3's chase of
   // the changed roots): passes of up to HOPS hops, each parent written by its
@@ -1058,7 +1056,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     }
     __syncwarp();
     vc = out;
-    return grid_barrier(C->arrive + phase, &C->abort, target);
+    return bar.meet();
   };
   // Rounds on the warp's `cnt` entries until no edge is left; the minima of
   // the first one have been offered.  With few edges left the roots are not
@@ -1077,7 +1075,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
         if (tid == 0) C->pairs[(k + 2) & 3] = 0;
         ++hooked;
       }
-      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return false;
+      if (!bar.meet()) return false;
       if (!small) {
         if (!settle_roots()) return false;
         cnt = min_pass<true, false>(A, tab, P, 0u, cnt);
@@ -1093,7 +1091,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   unsigned cnt;
   if (COUNT && phase == 2) {
     cnt = list_forest(A, P, Q);
-    if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
+    if (!bar.meet()) return;
   } else {
     cnt = A.front[warp];
   }
@@ -1113,7 +1111,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   if (!last) {
     if (BATCH) {
       vote_giants(A, warp, nthr >> 5);
-      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
+      if (!bar.meet()) return;
     }
     flatten(true, BATCH ? 0 : vote_giant(A));
     if (lane == 0) A.back[warp] = vc;
@@ -1169,7 +1167,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
       if (tab.key[i] >= 0 && b != 0xffffffffu) atomicMin(reinterpret_cast<unsigned *>(A.r + tab.key[i]), b);
     }
   }
-  if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
+  if (!bar.meet()) return;
   if (!BATCH && A.totals && blockIdx.x == 0) {
     for (int i = threadIdx.x; i < 256; i += ET) sbins[i] = (long long)ld_rel64(A.bins + i);
     __syncthreads();
@@ -1206,7 +1204,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   if (BATCH) {
     batch_results(A, P);
     if (A.totals) {
-      if (!grid_barrier(C->arrive + phase, &C->abort, target)) return;
+      if (!bar.meet()) return;
       // a warp per graph rounds its total
       for (int64_t g = warp; g < A.G; g += nthr >> 5) {
         const double t = combine_bins_warp(reinterpret_cast<const long long *>(A.bins) + g * 256, A.wtype);
