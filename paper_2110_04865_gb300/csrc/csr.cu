@@ -31,22 +31,42 @@ int grid_for(int64_t work, int per_sm = 8) {
   return (int)b;
 }
 
+// Rows of CSR slots.  A search per slot costs 20 dependent loads of row_ptr (R-MAT
+// 20, 2^25 slots: 475 us); here a warp looks for the rows of its first and last
+// slot, a lane for that of the first of its 16 between them, and walks on from
+// there (about 60 us).  Rows that are not non-decreasing are reported (err 4); the
+// searches end on them too.
+constexpr int COO_PER = 16;
 __global__ void __launch_bounds__(BT) k_csr_to_coo(const int64_t *row_ptr, const int32_t *col,
                                                    int64_t n, int64_t m, int32_t *src_out, int *err) {
-  const int64_t stride = (int64_t)gridDim.x * BT;
-  for (int64_t s = (int64_t)blockIdx.x * BT + threadIdx.x; s < m; s += stride) {
-    // row of slot s: largest i with row_ptr[i] <= s
-    int64_t lo = 0, hi = n;
+  const int64_t tid = (int64_t)blockIdx.x * BT + threadIdx.x, stride = (int64_t)gridDim.x * BT;
+  const int lane = threadIdx.x & 31;
+  // largest i in [lo, hi) with row_ptr[i] <= s, row_ptr[lo] <= s taken for granted
+  auto row_of = [&](int64_t lo, int64_t hi, int64_t s) {
     while (hi - lo > 1) {
-      int64_t mid = (lo + hi) >> 1;
-      if (row_ptr[mid] <= s) lo = mid; else hi = mid;
+      const int64_t mid = (lo + hi) >> 1;
+      if (row_ptr[mid] <= s) lo = mid;
+      else hi = mid;
     }
-    const int32_t c = col[s];
-    if (c < 0 || c >= n) { atomicOr(err, 1); src_out[s] = 0; continue; }
-    // slots with row >= column are not edges: make them self-loops
-    src_out[s] = (lo < c) ? (int32_t)lo : c;
+    return lo;
+  };
+  for (int64_t s0 = (tid - lane) * COO_PER; s0 < m; s0 += stride * COO_PER) {
+    const int64_t s1 = s0 + 32 * COO_PER < m ? s0 + 32 * COO_PER : m;
+    const int64_t r0 = row_of(0, n, s0), r1 = row_of(r0, n, s1 - 1);
+    const int64_t a = s0 + (int64_t)lane * COO_PER, b = a + COO_PER < s1 ? a + COO_PER : s1;
+    if (a >= s1) continue;
+    int64_t r = row_of(r0, r1 + 1, a);
+    int64_t end = row_ptr[r + 1];
+    for (int64_t s = a; s < b; ++s) {
+      while (s >= end && r + 1 < n) end = row_ptr[++r + 1];
+      const int32_t c = col[s];
+      int32_t u = 0;
+      if (c < 0 || c >= n) atomicOr(err, 1);
+      else u = r < c ? (int32_t)r : c;  // slots with row >= column are not edges: make them self-loops
+      src_out[s] = u;
+    }
   }
-  for (int64_t i = (int64_t)blockIdx.x * BT + threadIdx.x; i < n; i += stride)
+  for (int64_t i = tid; i < n; i += stride)
     if (row_ptr[i + 1] < row_ptr[i]) atomicOr(err, 4);
 }
 
@@ -108,20 +128,21 @@ __global__ void __launch_bounds__(BT) k_validate(const int32_t *__restrict__ src
 __global__ void k_slots_from_edges(long long *small) { small[4] = 2 * small[5]; }
 
 // Consecutive pairs among LOCALITY_SAMPLES evenly spread edges whose sources
-// or destinations lie more than `win` vertices apart (none for CSR input,
-// whose rows come in order).  Where few pairs do -- a lattice listed vertex
+// or destinations lie more than `win` vertices apart (of a CSR, whose rows come
+// in order, the columns).  Where few pairs do -- a lattice listed vertex
 // by vertex, a batch of small graphs listed graph by graph -- the
 // per-vertex atomic cursors write within a window of the slot arrays that
 // stays in L2.
 constexpr int64_t LOCALITY_SAMPLES = 1 << 13;
+constexpr int64_t BUCKET_EDGES = 1 << 21, BUCKET_SLOTS = 12 << 20;  // see build_csr_device
 __global__ void __launch_bounds__(BT) k_count_scattered(const int32_t *src, const int32_t *dst, int64_t m,
                                                         int64_t win, unsigned long long *out) {
-  if (!src || m < 2) return;
+  if (m < 2) return;
   unsigned c = 0;
   for (int64_t k = (int64_t)blockIdx.x * BT + threadIdx.x; k + 1 < LOCALITY_SAMPLES;
        k += (int64_t)gridDim.x * BT) {
     const int64_t i = k * (m - 1) / LOCALITY_SAMPLES, j = (k + 1) * (m - 1) / LOCALITY_SAMPLES;
-    const int64_t ds = (int64_t)src[i] - (int64_t)src[j], dd = (int64_t)dst[i] - (int64_t)dst[j];
+    const int64_t ds = src ? (int64_t)src[i] - (int64_t)src[j] : 0, dd = (int64_t)dst[i] - (int64_t)dst[j];
     c += (ds > win || -ds > win || dd > win || -dd > win);
   }
 #pragma unroll
@@ -468,15 +489,20 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
     coo_src = (int32_t *)tmp.get((size_t)(m > 0 ? m : 1) * sizeof(int32_t), &err);
     if (err) return err;
   }
-  // builder (measured on GB300): bucketed from 2^20 edges (R-MAT scale 20
-  // and 26, the uniform graph) unless the edge list has locality (the 256^3
-  // grid, a batch of small graphs, CSR input: per-vertex atomic cursors then
-  // write within an L2-sized window); per-vertex atomics for small graphs;
-  // radix on request
+  // builder: bucketed for many edges unless they have locality (the 256^3 grid, a
+  // batch of small graphs: per-vertex atomic cursors then write within an
+  // L2-sized window); per-vertex atomics for fewer, whose slots stay in L2; radix
+  // on request.  Whole builds in us, atomic / bucketed (with the sample's 22): COO
+  // of 2^21 edges 172-217 / 221-253, 3 * 2^20 241-306 / 259-294, 2^22 324-393 /
+  // 279-338; CSR of 2^23 slots 381-460 / 393-448, 3 * 2^22 529-737 / 514-562, 2^25
+  // 1362-1707 / 1053-1145 (a CSR's rows come in order, so half of its slots are
+  // written in order; beyond 2^22 vertices the buckets would be split twice).
   const int mode = options().build_mode;
   const bool radix = mode == 2;
   bool bucket = !radix && bucket_build_fits(n) && mode == 3;
-  if (mode == 0 && m >= ((int64_t)1 << 20) && bucket_build_fits(n)) {
+  const bool sampled = mode == 0 && bucket_build_fits(n) &&
+                       (row_ptr ? m >= BUCKET_SLOTS && n <= ((int64_t)1 << 22) : m >= BUCKET_EDGES);
+  if (sampled) {
     // window: the vertices whose slots (12 bytes each, 2m / n per vertex on
     // average) fill a quarter of L2
     int dev = 0, l2 = 0;
@@ -496,27 +522,37 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
     MSF_CK(cudaStreamSynchronize(s));
     bucket = far > (unsigned long long)(LOCALITY_SAMPLES / 16);
   }
-  uint32_t *deg = nullptr;
-  if (!radix && !bucket) {
-    deg = (uint32_t *)tmp.get((size_t)(n + 1) * 4, &err);
-    if (err) return err;
-    MSF_CK(cudaMemsetAsync(deg, 0, (size_t)(n + 1) * 4, s));
-  }
   MSF_CK(cudaMemsetAsync(small, 0, 64, s));
   int *errw = (int *)(small + 3);
   if (row_ptr) {
     k_csr_to_coo<<<grid_for(m), BT, 0, s>>>(row_ptr, dst, n, m, coo_src, errw);
     src = coo_src;
   }
-  if (m > 0 && !bucket) {  // (the bucketed builder validates in its first pass)
+  int rc = MSF_OK;
+  if (bucket) {  // (validates in its first pass; allocates before any)
+    rc = bucket_build_csr(n, m, src, dst, (const uint32_t *)w, wtype, G, eoff_d, voff_d, g->ends, small, g->csr0, s);
+    if (rc == MSF_ERR_OOM && sampled) {  // its records take 24 bytes an edge; the cursors take none
+      bucket = false;
+      set_error("");
+    } else if (rc) {
+      return rc;
+    }
+  }
+  uint32_t *deg = nullptr;
+  if (!radix && !bucket) {
+    deg = (uint32_t *)tmp.get((size_t)(n + 1) * 4, &err);
+    if (err) return err;
+    MSF_CK(cudaMemsetAsync(deg, 0, (size_t)(n + 1) * 4, s));
+  }
+  if (m > 0 && !bucket) {
     const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
                        reinterpret_cast<uintptr_t>(w)) & 15) == 0;
     auto *nl = (unsigned long long *)(small + 5);
     const uint32_t *wu = (const uint32_t *)w;
     const int gb = grid_for(vec ? (m + 3) / 4 : m);
-    if ((radix || bucket) && vec)
+    if (radix && vec)
       k_validate<false, true><<<gb, BT, 0, s>>>(src, dst, wu, wtype, m, n, G, eoff_d, voff_d, g->ends, errw, nl, deg);
-    else if (radix || bucket)
+    else if (radix)
       k_validate<false, false><<<gb, BT, 0, s>>>(src, dst, wu, wtype, m, n, G, eoff_d, voff_d, g->ends, errw, nl, deg);
     else if (vec)
       k_validate<true, true><<<gb, BT, 0, s>>>(src, dst, wu, wtype, m, n, G, eoff_d, voff_d, g->ends, errw, nl, deg);
@@ -525,16 +561,12 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
   }
   if (radix) k_slots_from_edges<<<1, 1, 0, s>>>(small);
   MSF_CK(cudaGetLastError());
-  int rc;
   bool marked = false;  // row-start marks already written by the builder
   if (radix) {
     rc = radix_build_csr(n, m, g->ends, (const uint32_t *)w, wtype, small + 4, small + 2, g->csr0, s);
     if (rc) return rc;
     MSF_CK(cudaMemcpyAsync(small + 1, small + 4, 8, cudaMemcpyDeviceToDevice, s));
-  } else if (bucket) {
-    rc = bucket_build_csr(n, m, src, dst, (const uint32_t *)w, wtype, G, eoff_d, voff_d, g->ends, small, g->csr0, s);
-    if (rc) return rc;
-  } else {
+  } else if (!bucket) {
     rc = atomic_build_csr(n, m, g->ends, (const uint32_t *)w, wtype, small, deg, g->csr0, s, &marked);
     if (rc) return rc;
   }
@@ -570,7 +602,7 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
                                                                               // 2^22 edges; rows (5)
   g->stats.builder = bucket ? 3 : (radix ? 2 : 1);
   g->build_kernels = (row_ptr ? 1 : 0) + (radix ? 1 : 0) /* slot count */ + builder + 1 /* tile map */ +
-                     ((mode == 0 && m >= ((int64_t)1 << 20) && bucket_build_fits(n)) ? 1 : 0);
+                     (sampled ? 1 : 0);
   return MSF_OK;
 }
 
