@@ -313,9 +313,10 @@ void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cuda
 // the device cannot hold the kernel's blocks at once; the outputs are
 // untouched.
 constexpr int SOLVE_NOT_RUN = -1;
+// It leaves `spare` SMs to blocks that run beside it.
 int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                unsigned *status, cudaStream_t s);
+                unsigned *status, int32_t spare, cudaStream_t s);
 
 // One graph given as pairs of validated ends, with what the round loop of
 // Algorithm 2 takes on it (its statistics); may return MSF_ERR_OOM before any
@@ -343,6 +344,22 @@ bool small_single(int64_t n, int64_t m);  // one graph: faster so than by solve_
 int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
                 unsigned *status, cudaStream_t s);
+// The same in two steps: start() queues the blocks (beside what is queued on `s`
+// later, with `beside`: K graphs of at most one per SM), finish() waits for them.
+class SmallRun {
+ public:
+  int start(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+            const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+            double *totals, bool count, bool beside, cudaStream_t s);
+  int finish(unsigned *status, LoopCounts *counts);
+  ~SmallRun();
+
+ private:
+  PinnedWords pin;
+  void *list = nullptr;
+  cudaStream_t stream = nullptr, side = nullptr;
+  bool queued = false;
+};
 bool small_counted(int64_t n, int64_t m);  // one graph with its counts: faster so than by solve_pairs
 int solve_small_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask,
                       int32_t *labels, double *totals, LoopCounts *counts, cudaStream_t s);

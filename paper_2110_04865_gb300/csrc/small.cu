@@ -539,11 +539,11 @@ bool small_single(int64_t n, int64_t m) { return small_fits(n, m) && m + 8 * n <
 // (8000, 60000) 345 / 195.
 bool small_counted(int64_t n, int64_t m) { return small_fits(n, m) && m <= ((int64_t)3 << 13); }
 
-namespace {
-
-int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
-          const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
-          double *totals, unsigned *status, LoopCounts *counts, cudaStream_t s) {
+// With `beside` the blocks are queued on a side stream that starts after the work
+// queued on `s` so far.
+int SmallRun::start(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
+                    const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
+                    double *totals, bool count, bool beside, cudaStream_t s) {
   const int64_t n = which ? 0 : voff[1], m = which ? 0 : eoff[1];
   const int32_t G = which ? K : 1;
   SmallArgs A;
@@ -551,7 +551,7 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   A.src = src;
   A.dst = dst;
   A.ends = ends;
-  A.count = counts != nullptr;
+  A.count = count;
   A.w = w;
   A.wtype = wtype;
   A.vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
@@ -563,14 +563,14 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   int err = MSF_OK;
   // pinned: status words, then the offsets and the blocks' graphs, which the
   // blocks read in place (a copy would cost a call more than their one read)
-  PinnedWords pin;
   if (int rc = pin.take(64 + (which ? (size_t)K * 44 : 0))) return rc;
   A.host = pin.p;
   int64_t entries = m + 256;
   for (int32_t k = 0; which && k < K; ++k) entries += eoff[which[k] + 1] - eoff[which[k]] + 128;
   char *base = (char *)pool_alloc((size_t)entries * 16, &err);
   if (err) return err;
-  PoolBlock back{base};
+  list = base;
+  stream = s;
   A.list = (uint4 *)base;
   int rc = MSF_OK;
   if (!which) {
@@ -627,9 +627,9 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
       tiers += blocks[t] > 0;
     }
     Fork fork(s);
-    for (int i = 1; i < tiers && rc == MSF_OK; ++i) rc = fork.branch();
+    for (int i = beside ? 0 : 1; i < tiers && rc == MSF_OK; ++i) rc = fork.branch();
     int64_t first = 0;
-    int used = 0;
+    int used = beside ? 1 : 0;
     for (int t = 0; t < 3 && rc == MSF_OK; ++t) {
       if (blocks[t] == 0) continue;
       A.order = order + first;
@@ -643,11 +643,24 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
            : t == 1 ? launch_small<512>(A, (int)blocks[t], dyn[t], st)
                     : launch_small<256>(A, (int)blocks[t], dyn[t], st);
     }
-    if (const int rj = fork.join()) rc = rc ? rc : rj;
+    if (beside) {
+      if (fork.n) side = fork.used[0];
+    } else if (const int rj = fork.join()) {
+      rc = rc ? rc : rj;
+    }
   }
-  cudaError_t e = rc ? cudaSuccess : cudaGetLastError();
-  const cudaError_t e2 = cudaStreamSynchronize(s);
+  queued = true;
   if (rc) return rc;
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? MSF_OK : cuda_fail(e, "forests of small graphs");
+}
+
+// (the side stream's work is waited for here: nothing of it is left when the call
+// returns)
+int SmallRun::finish(unsigned *status, LoopCounts *counts) {
+  queued = false;
+  cudaError_t e = side ? cudaStreamSynchronize(side) : cudaSuccess;
+  const cudaError_t e2 = cudaStreamSynchronize(stream);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "forests of small graphs");
   const volatile unsigned *st = (volatile unsigned *)pin.p;
@@ -662,7 +675,13 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   return MSF_OK;
 }
 
-}  // namespace
+SmallRun::~SmallRun() {
+  if (queued) {  // (an error after the start: what is queued ends before its memory goes back)
+    if (side) cudaStreamSynchronize(side);
+    cudaStreamSynchronize(stream);
+  }
+  pool_free(list);
+}
 
 // Forests of one graph (which = NULL), or of K graphs that fit (small_fits),
 // `which` of the graphs with the host offsets voff, eoff.  Synchronizes `s`;
@@ -670,14 +689,18 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
 int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
                 unsigned *status, cudaStream_t s) {
-  return solve(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, status, nullptr, s);
+  SmallRun run;
+  const int rc = run.start(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, false, false, s);
+  return rc ? rc : run.finish(status, nullptr);
 }
 
 int solve_small_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask,
                       int32_t *labels, double *totals, LoopCounts *counts, cudaStream_t s) {
   const int64_t voff[2] = {0, n}, eoff[2] = {0, m};
   unsigned status = 0;
-  return solve(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, &status, counts, s);
+  SmallRun run;
+  const int rc = run.start(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, true, false, s);
+  return rc ? rc : run.finish(&status, counts);
 }
 
 }  // namespace msf

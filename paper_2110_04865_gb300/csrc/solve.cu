@@ -1235,7 +1235,7 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 // `counts` (one graph, pairs) the rounds of the loop without classes too.
 int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
           const int32_t *dst, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
-          double *totals, unsigned *status, LoopCounts *counts, cudaStream_t s) {
+          double *totals, unsigned *status, LoopCounts *counts, int32_t spare, cudaStream_t s) {
   int64_t n = 0, m = 0;
   if (!which) {
     n = voff[1];
@@ -1259,7 +1259,7 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   // blocks: one per BLOCK_SHARE edges or vertices, at most one per SM
   int64_t want = ((m > n ? m : n) + BLOCK_SHARE - 1) / BLOCK_SHARE;
   if (want < 1) want = 1;
-  const int64_t cap = (int64_t)sm_count();
+  const int64_t cap = (int64_t)sm_count() - spare;  // (other blocks run on `spare` SMs meanwhile)
   const int blocks = (int)(want < cap ? want : cap);
   const int64_t warps = (int64_t)blocks * EW;
   A.es = page_shift(m, warps);
@@ -1409,15 +1409,15 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
 // 2 = NaN weight.
 int solve_edges(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,
                 const int32_t *dst, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels, double *totals,
-                unsigned *status, cudaStream_t s) {
-  return solve(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, status, nullptr, s);
+                unsigned *status, int32_t spare, cudaStream_t s) {
+  return solve(K, which, voff, eoff, src, dst, nullptr, w, wtype, mask, labels, totals, status, nullptr, spare, s);
 }
 
 int solve_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,
                 double *totals, LoopCounts *counts, cudaStream_t s) {
   const int64_t voff[2] = {0, n}, eoff[2] = {0, m};
   unsigned status = 0;
-  return solve(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, &status, counts, s);
+  return solve(1, nullptr, voff, eoff, nullptr, nullptr, ends, w, wtype, mask, labels, totals, &status, counts, 0, s);
 }
 
 }  // namespace msf
