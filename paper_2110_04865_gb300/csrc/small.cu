@@ -530,9 +530,11 @@ bool small_fits(int64_t n, int64_t m) {
 
 // One block against solve.cu's grid: the block's passes and rounds grow with the
 // edges and vertices, the grid's are a dozen barrier-bound phases.  Whole calls
-// in us at (n, m), block / grid: (18000, 131072) 253 / 237, (14000, 131072) 223 /
-// 235, (8000, 200000) 265 / 225, (4000, 200000) 176 / 230, (4000, 65536) 147 / 300.
-bool small_single(int64_t n, int64_t m) { return small_fits(n, m) && m + 8 * n <= ((int64_t)1 << 18); }
+// in us at (n, m), block / grid: (20000, 40000) 245 / 175, (14000, 131072) 229 / 186,
+// (14000, 28000) 180 / 168, (10000, 40000) 134 / 170, (8000, 100000) 165 / 174, (8000,
+// 200000) 219 / 178, (4000, 130000) 143 / 163, (4000, 400000) 276 / 162, (1000, 100000)
+// 114 / 153.
+bool small_single(int64_t n, int64_t m) { return small_fits(n, m) && m + 12 * n <= ((int64_t)11 << 14); }
 
 // The same with the loop's rounds counted, which needs every edge in every round:
 // (8000, 16000) 115 / 166, (1500, 15000) 109 / 147, (1500, 40000) 207 / 153,
