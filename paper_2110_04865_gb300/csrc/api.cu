@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <new>
 #include <vector>
 
 #include "internal.cuh"
@@ -522,6 +523,13 @@ int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t 
   } else {
     // a block each for the graphs that fit one, the others together
     std::vector<int32_t> small, large;
+    try {  // (no exception leaves a C entry)
+      small.reserve((size_t)G);
+      large.reserve((size_t)G);
+    } catch (const std::bad_alloc &) {
+      cudaStreamSynchronize(s);
+      return fail(MSF_ERR_OOM, "out of host memory");
+    }
     for (int32_t g = 0; g < G; ++g)
       (small_fits(voff[g + 1] - voff[g], eoff[g + 1] - eoff[g]) ? small : large).push_back(g);
     // Few small ones run beside the large ones, on SMs of their own: the grid of

@@ -165,6 +165,10 @@ constexpr size_t PIN_KEEP = 32;             // blocks kept at most
 int PinnedWords::take(size_t want) {
   {
     std::lock_guard<std::mutex> lk(g_pin_mu);
+    try {
+      g_pin_free.reserve(PIN_KEEP);  // (giving back must not throw)
+    } catch (const std::bad_alloc &) {
+    }
     for (size_t i = g_pin_free.size(); i-- > 0 && !p;)
       if (g_pin_free[i].second >= want) {
         p = g_pin_free[i].first;
@@ -186,7 +190,7 @@ PinnedWords::~PinnedWords() {
   if (!p) return;
   {
     std::lock_guard<std::mutex> lk(g_pin_mu);
-    if (bytes <= PIN_KEEP_BYTES && g_pin_free.size() < PIN_KEEP) {
+    if (bytes <= PIN_KEEP_BYTES && g_pin_free.size() < PIN_KEEP && g_pin_free.size() < g_pin_free.capacity()) {
       g_pin_free.emplace_back(p, bytes);
       return;
     }
