@@ -7,12 +7,12 @@
 // the CSR twice a round, about 240 us each for 2^24 edges.  Here an edge offers
 // to both ends at once, and most edges are read without a gathered parent:
 //
-//   round 1, conditional    parents are the vertices themselves: an edge offers
+//   first conditional       parents are the vertices themselves: an edge offers
 //                           its smaller end to its larger one;
-//   round 1, unconditional  only an edge between a star and another tree has
+//   first unconditional     only an edge between a star and another tree has
 //                           something to offer: two bits of the star bitmap
 //                           tell, from shared memory when it fits there;
-//   round 2, conditional    an edge inside the giant tree has nothing to offer
+//   second conditional      an edge inside the giant tree has nothing to offer
 //                           any more: two bits of its bitmap tell.  The edges
 //                           between trees go to the warps' lists, and all later
 //                           steps read and compact those.

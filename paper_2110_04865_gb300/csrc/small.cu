@@ -19,9 +19,9 @@
 // minima by compare-and-swap (ER 4096 112 us against 85), 512 threads with 128
 // registers (125), chains followed inside the minimum pass (115).
 //
-// Whole calls (CSR path before, this after): 100 vertices 331 -> 45 us, ER 4096
-// 417 -> 103, a batch of 64 graphs 650 -> 93, forward and backward of 256
-// graphs 1190 -> 390 (the rest of it is the autograd engine).
+// Whole calls (CSR path before, this after): 100 vertices 293 -> 35 us, ER 4096
+// 391 -> 97, a batch of 64 graphs 590 -> 90, forward and backward of 256 graphs
+// 1120 -> 351 (the rest of it is the autograd engine).
 #include <cstring>
 #include <mutex>
 

@@ -29,7 +29,7 @@
 // same pages: it fills, reads, relabels and compacts its own list in place, so
 // the lists need no global counters and cannot overflow.
 // The rounds kernel is cooperative, one block of 1024 threads per SM; its
-// phases meet at a grid barrier (about 2 us, bounded wait), which costs less
+// phases meet at a grid barrier (1 to 2 us, bounded wait), which costs less
 // than the kernel boundaries and conditional nodes of a graph loop (about 60
 // launches in the CSR path's small calls).  What bounds the steps: select and
 // filter the instruction issue and DRAM (R-MAT 20: 45 and 52 us for 201 and
@@ -37,11 +37,12 @@
 // gathered per edge), late rounds the barriers.
 //
 // Measured on the whole call (build and round loop over the CSR before, this
-// after): R-MAT 26 112 -> 21.9 ms, the 256^3 grid 9.9 -> 2.4 ms, R-MAT 20 1.75
-// -> 0.52 ms, uniform n = 10^6, m = 16 n 2.7 -> 0.55 ms, R-MAT 16 0.49 -> 0.20
-// ms.  Fractions around these (CLASS1 0.25 to 1, CLASS2 1.2 to 3): R-MAT 26
-// 20.7 to 22.9 ms, the grid 2.3 to 4.4, uniform 0.52 to 0.70, R-MAT 20 0.48 to
-// 0.54; a single light class of 1.5 n: 28.4, 3.2, 0.68 and 0.57 ms.
+// after): R-MAT 26 112 -> 21.9 ms, the 256^3 grid 9.9 -> 2.27 ms, R-MAT 20 1.75
+// -> 0.455 ms, uniform n = 10^6, m = 16 n 2.6 -> 0.51 ms, R-MAT 16 0.47 -> 0.174
+// ms, 4096 graphs of 38 M vertices 26.3 -> 5.84 ms.  Fractions around these when
+// they were chosen (CLASS1 0.25 to 1, CLASS2 1.2 to 3): R-MAT 26 20.7 to 22.9 ms,
+// the grid 2.3 to 4.4, uniform 0.52 to 0.70, R-MAT 20 0.48 to 0.54; a single light
+// class of 1.5 n: 28.4, 3.2, 0.68 and 0.57 ms.
 #include <cstring>
 
 #include "exact.cuh"
@@ -67,14 +68,22 @@ constexpr uint32_t CAND = 0x80000000u;  // list entry may be a minimum of one of
 constexpr uint32_t LONG = 0x80000000u;  // listed root whose chain goes on
 // Edges of the first class, and of both light classes, per vertex.
 constexpr double CLASS1 = 0.75, CLASS2 = 1.5;
-// Below this the light edges form one class: a second one saves less than its
-// rounds' barriers cost (R-MAT 16, m = 2^20: 197 us with one, 212 with two).
-constexpr int64_t TWO_CLASSES = 1 << 22;
-// With the loop's rounds counted one class up to here (its rounds are the
-// loop's), classes and a replay of the rounds on the forest from here on: in us,
-// one class / classes, R-MAT 2^20 edges 202 / 260, 2^21 266 / 297, 2^22 381 / 354;
-// uniform 2^20 282 / 325, 2^22 635 / 484; lattice 10^6 298 / 424.
-constexpr int64_t COUNT_CLASSES = 3 << 20;
+// The light edges form one class where a second one saves less than its rounds'
+// barriers cost.  Calls in us, one class / two, uniform unless said: (300 000, 9 M)
+// 329 / 339, R-MAT 18 of 8 M edges 261 / 273, an 80^3 lattice 293 / 312, 96^3 352 /
+// 372, (500 000, 4 M) 347 / 331, (500 000, 16 M) 446 / 397, (700 000, 16 M) 502 / 431,
+// (10^6, 2 M) 437 / 381, (2 * 10^6, 4 M) 632 / 522, a 140^3 lattice 632 / 595.
+inline bool two_classes(int64_t n, int64_t m) {
+  return n >= (int64_t)14 << 16 || (m >= (int64_t)1 << 22 && n >= (int64_t)3 << 17);
+}
+// With the loop's rounds counted: all edges in one class, whose rounds are the
+// loop's, or classes and a replay of the rounds on the forest.  In us, one class /
+// classes: R-MAT 16 of 2^20 edges 178 / 225, (200 000, 2^20) 297 / 349, a 96^3
+// lattice 416 / 515, R-MAT 18 of 2^21 257 / 288, of 2^22 355 / 306; (100 000, 2^21)
+// 395 / 336, (300 000, 3 M) 490 / 389, (10^6, 4 M) 677 / 577.
+inline bool count_by_replay(int64_t n, int64_t m) {
+  return m >= (int64_t)3 << 20 || (m >= (int64_t)3 << 19 && m >= 10 * n);
+}
 // Edges left from which a round's roots are settled in a step of their own:
 // below, all of them are in flight at once (155 648 threads) and the minimum
 // pass follows the chains itself, one barrier and about 5 us less per round
@@ -846,7 +855,6 @@ __device__ void batch_results(const Args &A, const Pages P) {
 // start; returns the entries.
 __device__ __noinline__ unsigned list_forest(const Args &A, const Pages P, const Pages Q) {
   const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
   for (uint32_t i = lane; i < Q.cap; i += 32) {
     const int64_t v = Q.at(i);
     if (v >= A.n) continue;
@@ -854,25 +862,27 @@ __device__ __noinline__ unsigned list_forest(const Args &A, const Pages P, const
     A.r[v] = KEY_INF;
     A.roots[v] = (int32_t)v;
   }
+  // a word of the bitmap per lane, whose bits it takes one after the other: all
+  // lanes' gathers are in flight (edge by edge, R-MAT 20: 86 of the call's
+  // 646 us; so the call takes 593)
   unsigned out = 0;
-  constexpr int U = 4;
-  for (uint32_t i = 0; i < P.cap; i += 32 * U) {
+  for (uint32_t i0 = 0; i0 < P.cap; i0 += 1024) {
+    const uint32_t i = i0 + 32 * lane;
     const int64_t e0 = P.at(i);
-    if (e0 >= A.m) continue;
-    uint4 x[U];
-    bool on[U];
+    uint32_t word = i < P.cap && e0 < A.m ? __ldcg(A.mbits + (e0 >> 5)) : 0u;
+    const unsigned mine = (unsigned)__popc(word);
+    unsigned incl = mine;
 #pragma unroll
-    for (int j = 0; j < U; ++j) {  // (the bitmap's words end at most 128 edges behind the last)
-      const int64_t e = e0 + j * 32 + lane;
-      on[j] = e < A.m && (__ldcg(A.mbits + (e0 >> 5) + j) >> lane & 1u);
-      const int2 uv = on[j] ? A.ends[e] : make_int2(0, 0);
-      x[j] = make_uint4((uint32_t)uv.x, (uint32_t)uv.y, (uint32_t)e, on[j] ? ord_weight_dev(A.w[e], A.wtype) : 0u);
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned o = __shfl_up_sync(FULL, incl, d);
+      if (lane >= d) incl += o;
     }
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const unsigned bal = __ballot_sync(FULL, on[j]);
-      if (on[j]) A.list[P.at(out + __popc(bal & below))] = x[j];
-      out += __popc(bal);
+    unsigned at = out + incl - mine;
+    out += __shfl_sync(FULL, incl, 31);
+    for (; word; word &= word - 1u) {
+      const int64_t e = e0 + __ffs((int)word) - 1;
+      const int2 uv = A.ends[e];
+      A.list[P.at(at++)] = make_uint4((uint32_t)uv.x, (uint32_t)uv.y, (uint32_t)e, ord_weight_dev(A.w[e], A.wtype));
     }
   }
   __syncwarp();
@@ -1266,9 +1276,9 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   A.vs = page_shift(n, warps);
   const int64_t epages = page_count(m, A.es), vpages = page_count(n, A.vs);
   A.classes = 1;
-  if (m >= (counts ? COUNT_CLASSES : 64 * SAMPLES)) {
+  if (m >= 64 * SAMPLES && (!counts || count_by_replay(n, m))) {
     double la = CLASS1, lb = CLASS2;
-    if (m < TWO_CLASSES) la = lb;
+    if (!two_classes(n, m)) la = lb;
     if ((double)m > 1.25 * la * (double)n && la < lb) A.classes = 2;
     if ((double)m > 1.25 * lb * (double)n) A.classes = 3;
     A.second = A.classes > 1 && la < lb;

@@ -45,7 +45,8 @@ def check(n, s, d, w, csr=True):
 @pytest.mark.parametrize("wtype", [0, 1])
 @pytest.mark.parametrize("n,m", [(1, 0), (1, 5), (2, 1), (127, 128), (129, 127), (8193, 4097), (100, 65535),
                                  (40000, 65536), (65536, 65537), (9000, 262147), (1700000, 300001),
-                                 (1900000, 3000001), (500001, 4194304), (2600000, 4300009)])
+                                 (1900000, 3000001), (500001, 4194304), (2600000, 4300009),
+                                 (393215, 4194305), (393216, 4194304), (917503, 1300000), (917504, 1300000)])
 def test_sizes(n, m, wtype):
     rng = np.random.default_rng(n + m)
     s = rng.integers(0, n, m).astype(np.int32)

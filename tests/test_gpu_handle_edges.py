@@ -49,7 +49,7 @@ def check(n, src, dst, w, row_ptr=None):
 
 @pytest.mark.parametrize("n,m", [(1, 0), (1, 4), (2, 1), (50, 7), (300, 900), (4096, 8192), (4096, 8195), (900, 60000),
                                  (12000, 30000), (20000, 131072), (9000, 262147), (300001, 200000),
-                                 (4000, 24576), (4000, 24577), (90000, 3145727), (90000, 3145728), (300000, 4194309), (1900000, 3000001), (2600000, 6300009)])
+                                 (4000, 24576), (4000, 24577), (300000, 3145727), (400000, 3145728), (157286, 1572860), (157287, 1572864), (300000, 4194309), (1900000, 3000001), (2600000, 6300009)])
 def test_sizes(n, m):
     rng = np.random.default_rng(n + m)
     s, d = (rng.integers(0, n, m).astype(np.int32) for _ in range(2))
