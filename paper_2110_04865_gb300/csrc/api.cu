@@ -275,8 +275,8 @@ bool one_shot_allowed() {
 // One graph's forest from the edges the build kept instead of the loop over the
 // CSR, with the loop's statistics (see k_rounds): every sweep of the loop reads
 // 12 bytes a slot and gathers a parent for each.  msf_compute, loop / this: R-MAT
-// 20 (2^24 edges) 1385 / 710 us, uniform 2^24 edges 1587 / 826, R-MAT 16 341 /
-// 202, 96^3 lattice 831 / 480, 1296 vertices 329 / 53.  MSF_ERR_OOM or
+// 20 (2^24 edges) 1385 / 594 us, uniform 2^24 edges 1587 / 698, R-MAT 16 259 /
+// 198, 96^3 lattice 831 / 424, 1296 vertices 329 / 49.  MSF_ERR_OOM or
 // SOLVE_NOT_RUN: no room or no place for it, the loop runs.
 int edges_compute(msf_graph *g, uint8_t *mask, int32_t *labels, double *totals, cudaStream_t s) {
   LoopCounts c;

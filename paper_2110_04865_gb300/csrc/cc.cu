@@ -20,9 +20,9 @@
 // R-MAT 20 with 2^24 edges, us: the first pass 91 (one gather an edge), the two
 // that read bitmaps 69 (instruction issue) and 145 (the parents of the edges
 // between trees, and their list), the lists 43 and 31, the passes over the
-// vertices 3 to 10 each, barriers about 2 each.  The call (loop over the CSR
-// before, this after): R-MAT 20 1466 -> 497 us, uniform 2^24 edges 1429 -> 556,
-// 96^3 lattice 278 -> 116, R-MAT 16 157 -> 101, 1296 vertices 142 -> 60.
+// vertices 3 to 10 each, barriers 1 to 2 each.  The call (loop over the CSR
+// before, this after): R-MAT 20 1466 -> 466 us, uniform 2^24 edges 1429 -> 520,
+// 96^3 lattice 278 -> 98, R-MAT 16 157 -> 86, 1296 vertices 142 -> 39.
 // Variants that measured slower: a block's recent offers kept in a table (first
 // pass 104, second bitmap pass 199), byte flags for the starcheck (72 against 9).
 #include <cstring>
