@@ -134,7 +134,7 @@ __global__ void k_slots_from_edges(long long *small) { small[4] = 2 * small[5]; 
 // per-vertex atomic cursors write within a window of the slot arrays that
 // stays in L2.
 constexpr int64_t LOCALITY_SAMPLES = 1 << 13;
-constexpr int64_t BUCKET_EDGES = 1 << 21, BUCKET_SLOTS = 12 << 20;  // see build_csr_device
+constexpr int64_t BUCKET_EDGES = 1 << 20, BUCKET_SLOTS = 12 << 20;  // see build_csr_device
 __global__ void __launch_bounds__(BT) k_count_scattered(const int32_t *src, const int32_t *dst, int64_t m,
                                                         int64_t win, unsigned long long *out) {
   if (m < 2) return;
@@ -646,10 +646,12 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
   // batch of small graphs: per-vertex atomic cursors then write within an
   // L2-sized window); per-vertex atomics for fewer, whose slots stay in L2; radix
   // on request.  Whole builds in us, atomic / bucketed (with the sample's 22): COO
-  // of 2^21 edges 172-217 / 221-253, 3 * 2^20 241-306 / 259-294, 2^22 324-393 /
-  // 279-338; CSR of 2^23 slots 381-460 / 393-448, 3 * 2^22 529-737 / 514-562, 2^25
-  // 1362-1707 / 1053-1145 (a CSR's rows come in order, so half of its slots are
-  // written in order; beyond 2^22 vertices the buckets would be split twice).
+  // of 2^20 edges 123-152 / 186-210, but 275 / 191 with hubs at adjacent ids (R-MAT
+  // 16, not permuted: the cursors of a few lines are written by most edges), 2^21
+  // 172-217 / 221-253, with hubs 349-469 / 233, 2^22 324-393 / 279-338; CSR of 3 *
+  // 2^22 slots 529-737 / 514-562, 2^25 1362-1707 / 1053-1145 (a CSR's rows come in
+  // order, so half of its slots are written in order; beyond 2^22 vertices the
+  // buckets would be split twice).
   const int mode = options().build_mode;
   const bool radix = mode == 2;
   bool bucket = !radix && bucket_build_fits(n) && mode == 3;
