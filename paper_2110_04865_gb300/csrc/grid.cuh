@@ -112,7 +112,8 @@ struct GridBarrier {  // in shared memory
 // Edges e to e + 4 (or hi) of pairs of ends, 16-byte aligned.
 __device__ __forceinline__ void load_pairs(const int2 *ends, int64_t e, int64_t hi, int4 &s, int4 &d) {
   if (e + 4 <= hi) {
-    const int4 a = __ldcs(reinterpret_cast<const int4 *>(ends + e)), b = __ldcs(reinterpret_cast<const int4 *>(ends + e) + 1);
+    const int4 *q = reinterpret_cast<const int4 *>(ends + e);
+    const int4 a = __ldcs(q), b = __ldcs(q + 1);
     s = make_int4(a.x, a.z, b.x, b.z);
     d = make_int4(a.y, a.w, b.y, b.w);
     return;

@@ -351,7 +351,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     L = A.list + (A.loff ? A.loff[blockIdx.x] : 0) + lo;
     int cnt = 0;
     {
-      auto load = [&](int b) { return A.ends ? pair_quad(A.ends, W, b + 4 * lane, hi) : edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi); };
+      auto load = [&](int b) {
+        return A.ends ? pair_quad(A.ends, W, b + 4 * lane, hi)
+                      : edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi);
+      };
       auto body = [&](const EdgeQuad &q, int b) {
         const int i = b + 4 * lane;
         limit.batch(a0 + b);

@@ -298,7 +298,8 @@ __device__ __noinline__ unsigned min_pass(const Args &A, Table &tab, const Pages
     for (int j = 0; j < U; ++j) {
       const unsigned bal = __ballot_sync(FULL, on[j]);
       const unsigned at = out + __popc(bal & below);
-      if (on[j]) A.list[P.at(at)] = make_uint4((uint32_t)u[j] | (cand >> j & 1u ? CAND : 0u), (uint32_t)v[j], x[j].z, x[j].w);
+      if (on[j])
+        A.list[P.at(at)] = make_uint4((uint32_t)u[j] | (cand >> j & 1u ? CAND : 0u), (uint32_t)v[j], x[j].z, x[j].w);
       out += __popc(bal);
     }
   }
@@ -310,8 +311,8 @@ __device__ __noinline__ unsigned min_pass(const Args &A, Table &tab, const Pages
 // breaking: of two roots that chose the same edge the smaller stays a root).
 // Returns the hooks of the thread in the low half and those of two roots that
 // chose each other, one for every tree formed, in the high half.
-__device__ __noinline__ unsigned hook_pass(const Args &A, const Pages P, unsigned cnt, bool small, bool mark, bool sum, BlockSums &sums,
-                                          unsigned long long &usum) {
+__device__ __noinline__ unsigned hook_pass(const Args &A, const Pages P, unsigned cnt, bool small, bool mark, bool sum,
+                                           BlockSums &sums, unsigned long long &usum) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 4;
   unsigned hooks = 0;
@@ -1076,7 +1077,8 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
     unsigned long long live = total_live(cnt);
     for (int k = 0; k < ROUND_CAP && live; ++k) {
       const bool small = live <= SMALL;
-      const unsigned h = hook_pass(A, P, cnt, small, A.mbits && !(COUNT && phase == 2), !BATCH && A.totals && !(COUNT && phase == 2), sums, usum);
+      const bool found = COUNT && phase == 2;  // (marked and summed before)
+      const unsigned h = hook_pass(A, P, cnt, small, A.mbits && !found, !BATCH && A.totals && !found, sums, usum);
       if (counting) {  // (added up with the edges left; the round's slot was cleared two rounds before)
         const unsigned t = __reduce_add_sync(FULL, h & 0xffffu), q = __reduce_add_sync(FULL, h >> 16);
         if (lane == 0 && q) atomicAdd(&s_pairs, q);
