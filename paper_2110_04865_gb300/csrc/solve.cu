@@ -1320,7 +1320,8 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   A.r = (unsigned long long *)(base + o_r);
   A.roots = (int32_t *)(base + o_roots);
   A.gbits = (uint32_t *)(base + o_gbits);
-  A.mbits = mask || (counts && A.classes > 1) ? (uint32_t *)(base + o_bits) : nullptr;
+  // the mask comes from the bitmap, and so do a batch's totals and the replay's list
+  A.mbits = mask || (which && totals) || (counts && A.classes > 1) ? (uint32_t *)(base + o_bits) : nullptr;
   A.bins = (unsigned long long *)(base + o_ctl + 256);
   A.front = (unsigned *)(base + o_front);
   A.back = (unsigned *)(base + o_back);
