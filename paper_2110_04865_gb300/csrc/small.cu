@@ -419,14 +419,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
   }
   // Results (parents are roots, the minima clear).  The last warp rounds the
   // total while the others write labels and mask.
-  if (A.totals) {
-    if (!F32) {
+  if (A.totals && !F32) {
 #pragma unroll
-      for (int d = 16; d >= 1; d >>= 1) usum += __shfl_xor_sync(FULL, usum, d);
-      if (lane == 0 && usum) atomicAdd(&s_usum, usum);
-    }
-    __syncthreads();
+    for (int d = 16; d >= 1; d >>= 1) usum += __shfl_xor_sync(FULL, usum, d);
+    if (lane == 0 && usum) atomicAdd(&s_usum, usum);
   }
+  __syncthreads();  // every warp's marks and weights are in (rounds_kept makes them last)
   if (wid == NW - 1) {
     if (!A.totals) return;
     if (F32) {

@@ -56,3 +56,34 @@ def test_batch_with_large_graphs(nv, ne, wtype):
     for want in COMBINATIONS:
         for got, r in zip(call(voff, eoff, arrays, wtype, want), ref):
             assert got is None or np.array_equal(got, r), want
+
+
+@pytest.mark.parametrize("wtype", [0, 1])
+@pytest.mark.parametrize("nv,ne", [([40], [512]), ([1500], [8192]), ([700], [30000]),
+                                   ([1500] * 40, [8192] * 40), ([60] * 400, [2048] * 400)])
+def test_small_graphs(nv, ne, wtype):
+    """Blocks of 256, 512 and 1024 threads, the last warp of each holding
+    edges (the sizes are those at which every register place is used)."""
+    voff, eoff, s, d, w = make(nv, ne, wtype)
+    ref = oracle.kruskal_batched(voff, eoff, s, d, w, wtype)
+    arrays = [to_dev(a) for a in (s, d, w)]
+    for want in COMBINATIONS * 4:
+        for got, r in zip(call(voff, eoff, arrays, wtype, want), ref):
+            assert got is None or np.array_equal(got, r), want
+
+
+@pytest.mark.parametrize("n,m", [(50, 200), (1500, 8192), (1500, 24576), (30000, 120000), (300000, 3500000)])
+def test_kept_graph(n, m):
+    import torch
+    from paper_2110_04865_gb300 import _abi, api
+    voff, eoff, s, d, w = make([n], [m], 0)
+    ref = oracle.kruskal(n, s, d, w, 0)
+    g = api.Graph(n, *(to_dev(a) for a in (s, d, w)))
+    for want in COMBINATIONS:
+        outs = [torch.full((k,), 77, dtype=t, device="cuda") if on else None
+                for on, k, t in zip(want, (m, n, 1), (torch.uint8, torch.int32, torch.float64))]
+        _abi.msf_compute(g.handle, *(o.data_ptr() if o is not None else 0 for o in outs),
+                         int(torch.cuda.current_stream().cuda_stream))
+        for o, r in zip(outs, ref):
+            assert o is None or np.array_equal(o.cpu().numpy(), np.atleast_1d(r)), want
+    g.free()
