@@ -33,10 +33,18 @@ int grid_for(int64_t work, int per_sm = 8) {
 
 // Rows of CSR slots.  A search per slot costs 20 dependent loads of row_ptr (R-MAT
 // 20, 2^25 slots: 475 us); here a warp looks for the rows of its first and last
-// slot, a lane for that of the first of its 16 between them, and walks on from
-// there (about 60 us).  Rows that are not non-decreasing are reported (err 4); the
-// searches end on them too.
-constexpr int COO_PER = 16;
+// slot, a lane for that of the first of its PER between them, and walks on from
+// there (PER = 16: about 60 us); after WALK rows without a slot it searches again
+// (a walk over a long run of empty rows: 2.7 s for 60 000 edges between the two
+// ends of 2^25 vertices).  Where many rows are empty a lane searches for one slot
+// (PER = 1), as a lane's searches follow one another: with fewer slots than
+// vertices, or than twice the vertices while the latency counts.  Whole builds in
+// us at (vertices, slots), PER 16 / 1: (2^20, 40 000) 184 / 122, (10^5, 10^5) 130 /
+// 112, (10^5, 2 * 10^5) 123 / 112, (2^24, 2^22) 717 / 631, (2^21, 2^21) 225 / 220,
+// (2^21, 2^22) 294 / 336, (2^24, 2^24) 1560 / 1750.  Rows that are not
+// non-decreasing are reported (err 4); the searches end on them too.
+constexpr int WALK = 4;
+template <int PER>
 __global__ void __launch_bounds__(BT) k_csr_to_coo(const int64_t *row_ptr, const int32_t *col,
                                                    int64_t n, int64_t m, int32_t *src_out, int *err) {
   const int64_t tid = (int64_t)blockIdx.x * BT + threadIdx.x, stride = (int64_t)gridDim.x * BT;
@@ -50,20 +58,31 @@ __global__ void __launch_bounds__(BT) k_csr_to_coo(const int64_t *row_ptr, const
     }
     return lo;
   };
-  for (int64_t s0 = (tid - lane) * COO_PER; s0 < m; s0 += stride * COO_PER) {
-    const int64_t s1 = s0 + 32 * COO_PER < m ? s0 + 32 * COO_PER : m;
-    const int64_t r0 = row_of(0, n, s0), r1 = row_of(r0, n, s1 - 1);
-    const int64_t a = s0 + (int64_t)lane * COO_PER, b = a + COO_PER < s1 ? a + COO_PER : s1;
-    if (a >= s1) continue;
-    int64_t r = row_of(r0, r1 + 1, a);
-    int64_t end = row_ptr[r + 1];
-    for (int64_t s = a; s < b; ++s) {
-      while (s >= end && r + 1 < n) end = row_ptr[++r + 1];
-      const int32_t c = col[s];
-      int32_t u = 0;
-      if (c < 0 || c >= n) atomicOr(err, 1);
-      else u = r < c ? (int32_t)r : c;  // slots with row >= column are not edges: make them self-loops
-      src_out[s] = u;
+  auto put = [&](int64_t s, int64_t r) {
+    const int32_t c = col[s];
+    int32_t u = 0;
+    if (c < 0 || c >= n) atomicOr(err, 1);
+    else u = r < c ? (int32_t)r : c;  // slots with row >= column are not edges: make them self-loops
+    src_out[s] = u;
+  };
+  if (PER == 1) {
+    for (int64_t s = tid; s < m; s += stride) put(s, row_of(0, n, s));
+  } else {
+    for (int64_t s0 = (tid - lane) * PER; s0 < m; s0 += stride * PER) {
+      const int64_t s1 = s0 + 32 * PER < m ? s0 + 32 * PER : m;
+      const int64_t r0 = row_of(0, n, s0), r1 = row_of(r0, n, s1 - 1);
+      const int64_t a = s0 + (int64_t)lane * PER, b = a + PER < s1 ? a + PER : s1;
+      if (a >= s1) continue;
+      int64_t r = row_of(r0, r1 + 1, a);
+      int64_t end = row_ptr[r + 1];
+      for (int64_t s = a; s < b; ++s) {
+        for (int k = 0; s >= end && r + 1 < n; ++k) {
+          r = k < WALK ? r + 1 : row_of(r + 1, r1 + 1, s);
+          end = row_ptr[r + 1];
+          if (k == WALK) break;
+        }
+        put(s, r);
+      }
     }
   }
   for (int64_t i = tid; i < n; i += stride)
@@ -680,7 +699,9 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
   MSF_CK(cudaMemsetAsync(small, 0, 64, s));
   int *errw = (int *)(small + 3);
   if (row_ptr) {
-    k_csr_to_coo<<<grid_for(m), BT, 0, s>>>(row_ptr, dst, n, m, coo_src, errw);
+    const bool gaps = m < n || (m < 2 * n && m <= ((int64_t)1 << 21));  // see k_csr_to_coo
+    if (gaps) k_csr_to_coo<1><<<grid_for(m > n ? m : n), BT, 0, s>>>(row_ptr, dst, n, m, coo_src, errw);
+    else k_csr_to_coo<16><<<grid_for(m), BT, 0, s>>>(row_ptr, dst, n, m, coo_src, errw);
     src = coo_src;
   }
   int rc = MSF_OK;
