@@ -432,7 +432,8 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
       g->w = nullptr;
       set_error("");
     } else if (m > 0) {
-      const cudaError_t e = cudaMemcpyAsync(g->w, sw.dev, (size_t)m * 4, cudaMemcpyDeviceToDevice, s);
+      // (page-locked weights may be read in place: MSF_OPT_HOST_INPUT)
+      const cudaError_t e = cudaMemcpyAsync(g->w, sw.dev, (size_t)m * 4, cudaMemcpyDefault, s);
       if (e != cudaSuccess) {
         free_graph(g);
         return cuda_fail(e, "copying weights");
