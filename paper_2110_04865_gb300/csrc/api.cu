@@ -298,6 +298,7 @@ int graph_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *tot
   int rc;
   if (g->G == 1 && g->w && one_shot_allowed() && options().tau == Options().tau) {
     Staged sm, sl, st;
+    Settle settle(s);
     if ((rc = sm.output(edge_mask, (size_t)g->m)) || (rc = sl.output(labels, (size_t)g->n * 4)) ||
         (rc = st.output(totals, 8)))
       return rc;
@@ -305,6 +306,7 @@ int graph_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *tot
     if (rc != MSF_ERR_OOM && rc != SOLVE_NOT_RUN) {
       if (rc || (rc = sm.copy_back(s)) || (rc = sl.copy_back(s)) || (rc = st.copy_back(s))) return rc;
       if (sm.owned || sl.owned || st.owned) MSF_CK(cudaStreamSynchronize(s));
+      settle.done = true;
       g->stats.n = g->n;
       g->stats.m = g->m;
       g->stats.nnz = g->nnz0;
@@ -317,6 +319,7 @@ int graph_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *tot
   if (rc) return rc;
   if ((rc = ensure_pairwise(g))) return rc;
   Staged sm, sl, st;
+  Settle settle(s);
   if ((rc = sm.output(edge_mask, (size_t)g->m))) return rc;
   if ((rc = sl.output(labels, (size_t)g->n * 4))) return rc;
   if ((rc = st.output(totals, (size_t)ntot * 8))) return rc;
@@ -335,6 +338,7 @@ int graph_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *tot
   if ((rc = sl.copy_back(s))) return rc;
   if ((rc = st.copy_back(s))) return rc;
   MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   g->stats.n = g->n;
   g->stats.m = g->m;
   g->stats.nnz = g->nnz0;
@@ -381,36 +385,31 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
   g->G = G;
   g->wtype = wtype;
   Staged ss, sd, sw, sr;
+  // (what is queued ends before its buffers return to the pool)
+  auto refuse = [&](int code) -> int {
+    cudaStreamSynchronize(s);
+    free_graph(g);
+    return code;
+  };
   if ((rc = sd.input(dst, (size_t)m * 4, s)) || (rc = sw.input(w, (size_t)m * 4, s)) ||
       (!row_ptr && (rc = ss.input(src, (size_t)m * 4, s))) ||
-      (row_ptr && (rc = sr.input(row_ptr, (size_t)(n + 1) * 8, s)))) {
-    cudaStreamSynchronize(s);  // copies already queued finish before their buffers return to the pool
-    free_graph(g);
-    return rc;
-  }
+      (row_ptr && (rc = sr.input(row_ptr, (size_t)(n + 1) * 8, s))))
+    return refuse(rc);
   if (row_ptr) {
     int64_t ends2[2] = {0, 0};
     cudaError_t e = cudaMemcpyAsync(&ends2[0], sr.dev, 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&ends2[1], (const int64_t *)sr.dev + n, 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-      free_graph(g);
-      return cuda_fail(e, "reading row_ptr");
-    }
-    if (ends2[0] != 0 || ends2[1] != m) {
-      free_graph(g);
-      return fail(MSF_ERR_INVALID_ARG, "row_ptr[0] must be 0 and row_ptr[n] must equal m");
-    }
+    if (e != cudaSuccess) return refuse(cuda_fail(e, "reading row_ptr"));
+    if (ends2[0] != 0 || ends2[1] != m)
+      return refuse(fail(MSF_ERR_INVALID_ARG, "row_ptr[0] must be 0 and row_ptr[n] must equal m"));
   }
   if (G > 1) {
     // the offsets, each followed by its block table (internal.cuh)
     int err = MSF_OK;
     g->voff_d = (int64_t *)pool_alloc((size_t)(G + 1) * 8 + (size_t)(off_table_len(n) + 1) * 4, &err);
     if (!err) g->eoff_d = (int64_t *)pool_alloc((size_t)(G + 1) * 8 + (size_t)(off_table_len(m) + 1) * 4, &err);
-    if (err) {
-      free_graph(g);
-      return err;
-    }
+    if (err) return refuse(err);
     cudaError_t e = cudaMemcpyAsync(g->voff_d, voff_h, (size_t)(G + 1) * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(g->eoff_d, eoff_h, (size_t)(G + 1) * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
@@ -418,10 +417,7 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
       launch_off_table(g->eoff_d, G, m, s);
       e = cudaGetLastError();
     }
-    if (e != cudaSuccess) {
-      free_graph(g);
-      return cuda_fail(e, "copying offsets");
-    }
+    if (e != cudaSuccess) return refuse(cuda_fail(e, "copying offsets"));
   }
   if (G == 1) {
     // msf_compute reads the edges (4 bytes an edge more, 25 us of 770 us at 2^24
@@ -434,18 +430,12 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
     } else if (m > 0) {
       // (page-locked weights may be read in place: MSF_OPT_HOST_INPUT)
       const cudaError_t e = cudaMemcpyAsync(g->w, sw.dev, (size_t)m * 4, cudaMemcpyDefault, s);
-      if (e != cudaSuccess) {
-        free_graph(g);
-        return cuda_fail(e, "copying weights");
-      }
+      if (e != cudaSuccess) return refuse(cuda_fail(e, "copying weights"));
     }
   }
   rc = build_csr_device(n, m, (const int32_t *)ss.dev, (const int32_t *)sd.dev, (const int64_t *)sr.dev, sw.dev,
                         wtype, G, g->eoff_d, g->voff_d, s, g);
-  if (rc) {
-    free_graph(g);
-    return rc;
-  }
+  if (rc) return refuse(rc);
   *out = g;
   return MSF_OK;
 }
@@ -506,12 +496,11 @@ int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t 
   const int64_t n = voff[G], m = eoff[G];
   int rc;
   Staged ss, sd, sw, om, ol, ot;
+  Settle settle(s);
   if ((rc = ss.input(src, (size_t)m * 4, s)) || (rc = sd.input(dst, (size_t)m * 4, s)) ||
       (rc = sw.input(w, (size_t)m * 4, s)) || (rc = om.output(edge_mask, (size_t)m)) ||
-      (rc = ol.output(labels, (size_t)n * 4)) || (rc = ot.output(totals, (size_t)G * 8))) {
-    cudaStreamSynchronize(s);  // copies already queued finish before their buffers return to the pool
+      (rc = ol.output(labels, (size_t)n * 4)) || (rc = ot.output(totals, (size_t)G * 8)))
     return rc;
-  }
   const int32_t *u = (const int32_t *)ss.dev, *v = (const int32_t *)sd.dev;
   const uint32_t *wd = (const uint32_t *)sw.dev;
   uint8_t *mk = (uint8_t *)om.dev;
@@ -528,7 +517,6 @@ int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t 
       small.reserve((size_t)G);
       large.reserve((size_t)G);
     } catch (const std::bad_alloc &) {
-      cudaStreamSynchronize(s);
       return fail(MSF_ERR_OOM, "out of host memory");
     }
     for (int32_t g = 0; g < G; ++g)
@@ -555,6 +543,7 @@ int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t 
   if (status & 2u) return fail(MSF_ERR_INVALID_ARG, "NaN weight");
   if ((rc = om.copy_back(s)) || (rc = ol.copy_back(s)) || (rc = ot.copy_back(s))) return rc;
   if (om.owned || ol.owned || ot.owned) MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   return MSF_OK;
 }
 
@@ -627,12 +616,14 @@ int msf_min_edge(msf_graph *g, const int32_t *parent, uint64_t *r, void *stream)
   cudaStream_t s = (cudaStream_t)stream;
   int rc;
   Staged sp, sr;
+  Settle settle(s);
   if ((rc = sp.input(parent, (size_t)g->n * 4, s))) return rc;
   if ((rc = sr.output(r, (size_t)g->n * 8))) return rc;
   if (plain_sweep()) {
     if ((rc = min_edge_slots(g, (const int32_t *)sp.dev, 0, g->nnz0, (uint64_t *)sr.dev, s))) return rc;
     if ((rc = sr.copy_back(s))) return rc;
     if (sr.owned) MSF_CK(cudaStreamSynchronize(s));
+    settle.done = true;
     return MSF_OK;
   }
   int err = MSF_OK;
@@ -645,7 +636,8 @@ int msf_min_edge(msf_graph *g, const int32_t *parent, uint64_t *r, void *stream)
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
   pool_free(flag);
   if (e != cudaSuccess) return cuda_fail(e, "checking parent");
   if (hflag) return fail(MSF_ERR_INVALID_ARG, "parent value outside [0, n)");
@@ -672,6 +664,7 @@ int msf_min_edge(msf_graph *g, const int32_t *parent, uint64_t *r, void *stream)
   g->stats.min_edge_ms = ms;
   if ((rc = sr.copy_back(s))) return rc;
   MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   return MSF_OK;
 }
 
@@ -684,6 +677,7 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
   cudaStream_t s = (cudaStream_t)stream;
   int rc;
   Staged sp, sr;
+  Settle settle(s);
   if ((rc = sp.input(parent, (size_t)g->n * 4, s))) return rc;
   if ((rc = sr.output(r, (size_t)g->n * 8))) return rc;
   // the part's slots [s0, s1): cuts at multiples of SLOT_PAD, so that every
@@ -699,6 +693,7 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
     if ((rc = min_edge_slots(g, (const int32_t *)sp.dev, s0, s1, (uint64_t *)sr.dev, s))) return rc;
     if ((rc = sr.copy_back(s))) return rc;
     if (sr.owned) MSF_CK(cudaStreamSynchronize(s));
+    settle.done = true;
     return MSF_OK;
   }
   int err = MSF_OK;
@@ -711,7 +706,8 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
   pool_free(flag);
   if (e != cudaSuccess) return cuda_fail(e, "checking parent");
   if (hflag) return fail(MSF_ERR_INVALID_ARG, "parent value outside [0, n)");
@@ -748,6 +744,7 @@ int msf_min_edge_part(msf_graph *g, const int32_t *parent, int32_t part, int32_t
   }
   if ((rc = sr.copy_back(s))) return rc;
   MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   return MSF_OK;
 }
 
@@ -794,6 +791,7 @@ int msf_connected_components(msf_graph *g, int32_t *labels, void *stream) {
   cudaStream_t s = (cudaStream_t)stream;
   int rc;
   Staged sl;
+  Settle settle(s);
   if ((rc = sl.output(labels, (size_t)g->n * 4))) return rc;
   if (options().round_limit >= 64 && options().jump_limit >= 64) {
     // the kernel over the edges stops at no round of the caller's and counts no
@@ -805,6 +803,7 @@ int msf_connected_components(msf_graph *g, int32_t *labels, void *stream) {
       g->stats.cc_rounds = rounds;
       if ((rc = sl.copy_back(s))) return rc;
       if (sl.owned) MSF_CK(cudaStreamSynchronize(s));
+      settle.done = true;
       return MSF_OK;
     }
     set_error("");
@@ -822,6 +821,7 @@ int msf_connected_components(msf_graph *g, int32_t *labels, void *stream) {
   if ((rc = enqueue_cc_graph(hs, s, &back))) return rc;
   if ((rc = sl.copy_back(s))) return rc;
   MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   g->stats.cc_rounds = back->round;
   if (back->status == MSF_ERR_ROUND_LIMIT) return fail(MSF_ERR_ROUND_LIMIT, "round limit reached");
   if (back->status == MSF_ERR_SHORTCUT_LIMIT) return fail(MSF_ERR_SHORTCUT_LIMIT, "shortcutting did not settle");
@@ -839,6 +839,7 @@ int msf_weight_backward(int64_t m, int32_t G, const int64_t *eoff, const uint8_t
   cudaStream_t s = (cudaStream_t)stream;
   int rc;
   Staged se, sm, sg, sw;
+  Settle settle(s);
   // few graphs: their offsets go with the launch (eoff is read here)
   const bool few = G <= BACKWARD_GRAPHS && m <= MAX_M && !(G > 1 && is_device_ptr(eoff));
   if (!few && G > 1 && (rc = se.input(eoff, (size_t)(G + 1) * 8, s))) return rc;
@@ -860,6 +861,7 @@ int msf_weight_backward(int64_t m, int32_t G, const int64_t *eoff, const uint8_t
   MSF_CK(cudaGetLastError());
   if ((rc = sw.copy_back(s))) return rc;
   if (se.owned || sm.owned || sg.owned || sw.owned) MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   return MSF_OK;
 }
 

@@ -487,6 +487,7 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
   PoolBlock back{base};
   PinnedWords pin;
   if (int rc = pin.take(64)) return rc;
+  Settle settle(s);
   pin.p[0] = 1u;
   A.ctl = (CcCtrl *)(base + o_ctl);
   A.p = (int32_t *)(base + o_p);
@@ -507,6 +508,7 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
     return SOLVE_NOT_RUN;
   }
   const cudaError_t e2 = cudaStreamSynchronize(s);
+  settle.done = true;
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "connected components");
   const volatile unsigned *st = pin.p;

@@ -614,6 +614,7 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
                      msf_graph *g) {
   int err = MSF_OK;
   Tmp tmp;
+  Settle settle(s);
   const int64_t cap_slots = 2 * m;
   const int64_t padded = (cap_slots + SLOT_PAD - 1) / SLOT_PAD * SLOT_PAD + SLOT_PAD;
   g->ends = (int2 *)pool_alloc((size_t)(m > 0 ? m : 1) * sizeof(int2), &err);
@@ -644,6 +645,7 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
                                     pin.p);
     MSF_CK(cudaGetLastError());
     MSF_CK(cudaStreamSynchronize(s));
+    settle.done = true;
     const volatile unsigned *h = pin.p;
     if (int rc = refused((int)h[3])) return rc;
     g->nnz0 = h[1];
@@ -753,6 +755,7 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
   long long hsmall[4] = {0, 0, 0, 0};
   MSF_CK(cudaMemcpyAsync(hsmall, small, sizeof(hsmall), cudaMemcpyDeviceToHost, s));
   MSF_CK(cudaStreamSynchronize(s));
+  settle.done = true;
   if ((rc = refused((int)(hsmall[3] & 0xffffffff)))) return rc;
   g->nnz0 = hsmall[1];
   g->nrows0 = hsmall[2];

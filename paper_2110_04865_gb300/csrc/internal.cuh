@@ -191,6 +191,17 @@ struct PoolBlock {
   void *p;
   ~PoolBlock() { pool_free(p); }
 };
+// Waits for a stream at the end of a scope unless the call got past its own wait:
+// declared behind what holds the call's memory, it makes a call that fails midway
+// give its blocks back with nothing queued on them any more.
+struct Settle {
+  cudaStream_t s;
+  bool done = false;
+  explicit Settle(cudaStream_t st) : s(st) {}
+  ~Settle() {
+    if (!done) cudaStreamSynchronize(s);
+  }
+};
 // Pinned host memory of one call (its first 64 bytes zeroed), for a status that
 // a kernel writes and small tables that it reads in place.
 struct PinnedWords {

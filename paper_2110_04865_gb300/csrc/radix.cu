@@ -357,8 +357,9 @@ int radix_build_csr(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, i
                    reinterpret_cast<int64_t *>(nrows_dev), s);
   k_rb_write<<<NB, RT, 0, s>>>(rowtmp, nslots_dev, hist, nrows_dev, csr.rows, csr.rp);
   cudaError_t e = cudaGetLastError();
-  // the scratch returns to the pool after the caller's synchronisation
-  e = (e == cudaSuccess) ? cudaStreamSynchronize(s) : e;
+  // (waited for whatever was queued: the scratch returns to the pool)
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
   for (int i = 0; i < nk; ++i) pool_free(keep[i]);
   if (e != cudaSuccess) return cuda_fail(e, "radix CSR build");
   return MSF_OK;

@@ -1313,6 +1313,7 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   PoolBlock back{base};
   PinnedWords pin;
   if (int rc = pin.take(64 + tab_bytes)) return rc;
+  Settle settle(s);
   pin.p[0] = 0x80000000u;  // not finished
   pin.p[1] = counts ? 0x80000000u : 0u;
   A.ctl = (Ctrl *)(base + o_ctl);
@@ -1399,6 +1400,7 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   const cudaError_t e2 = cudaStreamSynchronize(s);
+  settle.done = true;
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "forest of an edge list");
   const unsigned st = *(volatile unsigned *)pin.p;

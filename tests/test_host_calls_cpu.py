@@ -44,3 +44,14 @@ def test_copies_name_their_memory(program, scenario):
     """Page-locked arrays that are read in place are host memory: no copy of
     them is one between device buffers."""
     assert not [x for x in run(program, scenario + " locked") if x.startswith("plain") and "a copy" in x]
+
+
+@pytest.mark.parametrize("where", ["", " host", " locked"])
+@pytest.mark.parametrize("scenario", SCENARIOS)
+def test_failed_calls_give_back_idle_blocks(program, scenario, where):
+    """Every allocation and every queued call of the scenario fails in turn:
+    no block goes back to the pool while queued work may use it, and none is
+    lost."""
+    out = run(program, scenario + where)
+    assert out[-1].startswith("done")
+    assert not out[:-1], out[:20]
