@@ -115,6 +115,33 @@ void free_buf(CsrBuf &b) {
   b = CsrBuf{};
 }
 
+// The loop's buffers (all of them, or those that an allocation that failed left).
+void free_workspace(msf_graph *g) {
+  free_buf(g->w1);
+  free_buf(g->w2);
+  auto drop = [](auto *&p) {
+    pool_free(p);
+    p = nullptr;
+  };
+  drop(g->p);
+  drop(g->tgt);
+  drop(g->changed);
+  drop(g->star);
+  drop(g->prow);
+  drop(g->colr);
+  drop(g->r);
+  drop(g->rl_a);
+  drop(g->rl_b);
+  drop(g->msf_keys);
+  drop(g->mbits);
+  drop(g->rowcnt);
+  drop(g->rowflag);
+  drop(g->tilecnt);
+  drop(g->scan_tmp);
+  drop(g->bins);
+  g->ws_ready = false;
+}
+
 void free_graph(msf_graph *g) {
   if (!g) return;
   pool_free(g->ends);
@@ -122,25 +149,8 @@ void free_graph(msf_graph *g) {
   pool_free(g->voff_d);
   pool_free(g->eoff_d);
   free_buf(g->csr0);
-  free_buf(g->w1);
-  free_buf(g->w2);
-  pool_free(g->p);
-  pool_free(g->tgt);
-  pool_free(g->changed);
-  pool_free(g->star);
   pool_free(g->pjs);
-  pool_free(g->prow);
-  pool_free(g->colr);
-  pool_free(g->r);
-  pool_free(g->rl_a);
-  pool_free(g->rl_b);
-  pool_free(g->msf_keys);
-  pool_free(g->mbits);
-  pool_free(g->rowcnt);
-  pool_free(g->rowflag);
-  pool_free(g->tilecnt);
-  pool_free(g->scan_tmp);
-  pool_free(g->bins);
+  free_workspace(g);
   delete g;
 }
 
@@ -169,8 +179,7 @@ int alloc_n(T **p, int64_t count) {
   return err;
 }
 
-int ensure_workspace(msf_graph *g) {
-  if (g->ws_ready) return MSF_OK;
+int take_workspace(msf_graph *g) {
   const int64_t n = g->n;
   int rc;
   if ((rc = alloc_n(&g->p, n + 1))) return rc;
@@ -199,12 +208,33 @@ int ensure_workspace(msf_graph *g) {
   return MSF_OK;
 }
 
+// The kept weights make room for the loop's buffers, which need the CSR alone.
+int ensure_workspace(msf_graph *g) {
+  if (g->ws_ready) return MSF_OK;
+  int rc = take_workspace(g);
+  if (rc) free_workspace(g);
+  if (rc == MSF_ERR_OOM && g->w) {
+    pool_free(g->w);
+    g->w = nullptr;
+    set_error("");
+    if ((rc = take_workspace(g))) free_workspace(g);
+  }
+  return rc;
+}
+
 // The pairwise formulation's slot array (nnz0 + padding int32), allocated on
 // first use.
 int ensure_pairwise(msf_graph *g) {
   if (g->pjs || !options().pairwise) return MSF_OK;
   const int64_t padded = (g->nnz0 + SLOT_PAD - 1) / SLOT_PAD * SLOT_PAD + SLOT_PAD;
-  return alloc_n(&g->pjs, padded);
+  int rc = alloc_n(&g->pjs, padded);
+  if (rc == MSF_ERR_OOM && g->w) {  // (as above)
+    pool_free(g->w);
+    g->w = nullptr;
+    set_error("");
+    rc = alloc_n(&g->pjs, padded);
+  }
+  return rc;
 }
 
 DevState make_state(msf_graph *g) {
@@ -418,20 +448,6 @@ int build_graph_common(int64_t n, int64_t m, const int32_t *src, const int32_t *
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return refuse(cuda_fail(e, "copying offsets"));
-  }
-  if (G == 1) {
-    // msf_compute reads the edges (4 bytes an edge more, 25 us of 770 us at 2^24
-    // edges); without room for them it runs the loop over the CSR
-    int err = MSF_OK;
-    g->w = (uint32_t *)pool_alloc((size_t)(m > 0 ? m : 1) * 4, &err);
-    if (err) {
-      g->w = nullptr;
-      set_error("");
-    } else if (m > 0) {
-      // (page-locked weights may be read in place: MSF_OPT_HOST_INPUT)
-      const cudaError_t e = cudaMemcpyAsync(g->w, sw.dev, (size_t)m * 4, cudaMemcpyDefault, s);
-      if (e != cudaSuccess) return refuse(cuda_fail(e, "copying weights"));
-    }
   }
   rc = build_csr_device(n, m, (const int32_t *)ss.dev, (const int32_t *)sd.dev, (const int64_t *)sr.dev, sw.dev,
                         wtype, G, g->eoff_d, g->voff_d, s, g);

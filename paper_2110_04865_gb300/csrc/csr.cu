@@ -606,6 +606,23 @@ void launch_tile_rows(DevState *st, int which, cudaStream_t s) {
   k_tile_rows_state<<<(int)sm_count() * 4, BT, 0, s>>>(st, which);
 }
 
+// One graph's weights, which msf_compute reads with the ends (4 bytes an edge more,
+// 25 us of 770 us at 2^24 edges).  The build's last allocation: without room for
+// them msf_compute runs the loop over the CSR.
+static int keep_weights(msf_graph *g, const void *w, cudaStream_t s) {
+  if (g->G != 1) return MSF_OK;
+  int err = MSF_OK;
+  g->w = (uint32_t *)pool_alloc((size_t)(g->m > 0 ? g->m : 1) * 4, &err);
+  if (err) {
+    g->w = nullptr;
+    set_error("");
+    return MSF_OK;
+  }
+  // (page-locked weights may be read in place: MSF_OPT_HOST_INPUT)
+  if (g->m > 0) MSF_CK(cudaMemcpyAsync(g->w, w, (size_t)g->m * 4, cudaMemcpyDefault, s));
+  return MSF_OK;
+}
+
 // Builds g->csr0 and g->ends on the device from device-resident inputs.
 // `src` is ignored when row_ptr != NULL.  Synchronizes `s`.
 int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *dst,
@@ -641,11 +658,13 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
   if (options().build_mode == 0 && G == 1 && n <= ONE_N && m <= ONE_M && (row_ptr || n + m <= ONE_SUM)) {
     PinnedWords pin;
     if (int rc = pin.take(64)) return rc;
+    Settle pinned(s);
     k_build_one<<<1, ONE_T, 0, s>>>(src, dst, row_ptr, (const uint32_t *)w, wtype, (int)n, (int)m, g->ends, g->csr0,
                                     pin.p);
     MSF_CK(cudaGetLastError());
+    if (int rc = keep_weights(g, w, s)) return rc;
     MSF_CK(cudaStreamSynchronize(s));
-    settle.done = true;
+    settle.done = pinned.done = true;
     const volatile unsigned *h = pin.p;
     if (int rc = refused((int)h[3])) return rc;
     g->nnz0 = h[1];
@@ -752,6 +771,7 @@ int build_csr_device(int64_t n, int64_t m, const int32_t *src, const int32_t *ds
                                                          (const int64_t *)(small + 1), g->csr0.tile_row,
                                                          g->csr0.col, g->csr0.key, marked);
   MSF_CK(cudaGetLastError());
+  if ((rc = keep_weights(g, w, s))) return rc;
   long long hsmall[4] = {0, 0, 0, 0};
   MSF_CK(cudaMemcpyAsync(hsmall, small, sizeof(hsmall), cudaMemcpyDeviceToHost, s));
   MSF_CK(cudaStreamSynchronize(s));

@@ -6,7 +6,8 @@
 // does not fit their source.  Runs without a GPU; no kernel is executed.
 //
 //   program SCENARIO         every allocation, then every call, fails in turn
-//   program SCENARIO budget  the smallest device memory in which it succeeds
+//   program SCENARIO SIZE    the smallest pool in which it does not run out of
+//                            memory, as it is and with no blocks of SIZE bytes
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -32,7 +33,7 @@ std::map<char *, Block> blocks;
 std::map<cudaStream_t, Streams> waits;  // streams whose work a stream waits for
 std::vector<std::string> found;
 long allocs, calls, fail_alloc = -1, fail_call = -1;
-size_t budget = ~(size_t)0, used;
+size_t budget = ~(size_t)0, used, refused = ~(size_t)0;
 cudaError_t last = cudaSuccess;
 cudaStream_t launch_stream;
 
@@ -231,7 +232,7 @@ cudaError_t cudaStreamUpdateCaptureDependencies(cudaStream_t, cudaGraphNode_t *,
 
 namespace msf {
 void *pool_alloc(size_t bytes, int *err) {
-  if (allocs++ == fail_alloc || used + bytes > budget) {
+  if (allocs++ == fail_alloc || used + bytes > budget || bytes == refused) {
     *err = MSF_ERR_OOM;
     return nullptr;
   }
@@ -384,13 +385,17 @@ int main(int argc, char **argv) {
     return rc;
   };
   if (argc > 2) {
-    // smallest budget in which the call does not run out of memory
-    size_t lo = 0, hi = (size_t)1 << 32;
-    while (hi - lo > 1) {
-      budget = (lo + hi) / 2;
-      (once("budget", (long)budget) == MSF_ERR_OOM ? lo : hi) = budget;
-    }
-    std::printf("budget %zu\n", hi);
+    auto least = [&]() {
+      size_t lo = 0, hi = (size_t)1 << 32;
+      while (hi - lo > 1) {
+        budget = (lo + hi) / 2;
+        (once("budget", (long)budget) == MSF_ERR_OOM ? lo : hi) = budget;
+      }
+      return hi;
+    };
+    const size_t a = least();
+    refused = (size_t)std::atol(argv[2]);
+    std::printf("%zu %zu\n", a, least());
     return 0;
   }
   const int rc = once("plain", 0);

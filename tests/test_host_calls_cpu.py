@@ -55,3 +55,12 @@ def test_failed_calls_give_back_idle_blocks(program, scenario, where):
     out = run(program, scenario + where)
     assert out[-1].startswith("done")
     assert not out[:-1], out[:20]
+
+
+@pytest.mark.parametrize("scenario,edges", [("build_one", 300), ("build", 60000), ("build_bucket", 60000),
+                                            ("compute_loop", 60000)])
+def test_kept_weights_need_no_room(program, scenario, edges):
+    """A build and the loop over the CSR take no more memory than where the
+    weights kept for msf_compute are refused theirs."""
+    with_weights, without = map(int, run(program, scenario, str(4 * edges))[-1].split())
+    assert with_weights == without
