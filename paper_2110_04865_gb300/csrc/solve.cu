@@ -87,8 +87,11 @@ inline bool count_by_replay(int64_t n, int64_t m) {
 // Edges left from which a round's roots are settled in a step of their own:
 // below, all of them are in flight at once (155 648 threads) and the minimum
 // pass follows the chains itself, one barrier and about 5 us less per round
-// (R-MAT 16: 257 -> 199 us).
-constexpr unsigned long long SMALL = 1 << 17;
+// (R-MAT 16: 257 -> 199 us).  A graph with few more edges than vertices may be one
+// long chain, whose edges all wait at the same parents: there from 2^15 on (a path
+// with rising weights and permuted ids, 40 000 vertices 177 -> 140 us, 131 000
+// 224 -> 155; for all graphs that line took R-MAT 16 from 174 to 184).
+constexpr unsigned long long SMALL = 1 << 17, SMALL_CHAINS = 1 << 15;
 // Edges or vertices per block: a call that does not fill the device.
 constexpr int64_t BLOCK_SHARE = 1024;
 
@@ -1076,7 +1079,7 @@ __global__ void __launch_bounds__(ET, 1) k_rounds(const __grid_constant__ Args A
   auto rounds = [&](unsigned cnt) -> bool {
     unsigned long long live = total_live(cnt);
     for (int k = 0; k < ROUND_CAP && live; ++k) {
-      const bool small = live <= SMALL;
+      const bool small = live <= (A.m > A.n + A.n / 4 ? SMALL : SMALL_CHAINS);
       const bool found = COUNT && phase == 2;  // (marked and summed before)
       const unsigned h = hook_pass(A, P, cnt, small, A.mbits && !found, !BATCH && A.totals && !found, sums, usum);
       if (counting) {  // (added up with the edges left; the round's slot was cleared two rounds before)

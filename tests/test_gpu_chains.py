@@ -84,3 +84,20 @@ def test_chains_take_no_longer_than_random_graphs(kind):
     assert median(g.compute) < 2 * median(tree.compute)
     g.free()
     tree.free()
+
+
+@pytest.mark.parametrize("kind", ["rising", "falling", "permuted"])
+@pytest.mark.parametrize("n", [40000, 100000])
+def test_chains_take_no_longer_than_the_round_loop(kind, n):
+    """(A threshold of its own selects the loop over the CSR.)"""
+    from paper_2110_04865_gb300 import _abi, api
+    g = api.Graph(n, *(to_dev(a) for a in chain(kind, n)))
+    edges = median(g.compute)
+    old = _abi.msf_get_option(_abi.OPT_COMPACT_TAU)
+    try:
+        _abi.msf_set_option(_abi.OPT_COMPACT_TAU, 0.25)
+        loop = median(g.compute)
+    finally:
+        _abi.msf_set_option(_abi.OPT_COMPACT_TAU, old)
+    g.free()
+    assert edges < loop
