@@ -507,6 +507,18 @@ int min_edge_slots(msf_graph *g, const int32_t *p, int64_t s0, int64_t s1, uint6
   return MSF_OK;
 }
 
+// Very many tiny graphs go through the union's CSR: a block each costs about 32 ns a
+// graph whatever its size, and the table that the blocks read in place 300 us more
+// once it is too large to be kept between calls; the union's loop costs its edges.
+// Whole calls in us at (graphs, vertices and edges of each), blocks / union: (23 000,
+// 10, 20) 739 / 844, (24 000, 10, 20) 1037 / 896, (24 000, 32, 100) 1158 / 1179,
+// (50 000, 32, 100) 2223 / 1908, (50 000, 48, 150) 2155 / 2237, (50 000, 100, 100)
+// 2321 / 2489, (100 000, 10, 20) 3487 / 2341, (100 000, 48, 150) 4079 / 4031, (100
+// 000, 64, 256) 4379 / 5155, (10^6, 4, 6) 29 590 / 17 011.
+bool many_tiny(int32_t G, int64_t n, int64_t m) {
+  return (size_t)G * SMALL_TABLE > PIN_KEEP_BYTES && n + m < (int64_t)(G < 65536 ? 160 : 200) * G;
+}
+
 int one_shot(int32_t G, const int64_t *voff, const int64_t *eoff, const int32_t *src, const int32_t *dst,
              const void *w, int wtype, uint8_t *edge_mask, int32_t *labels, double *totals, cudaStream_t s) {
   const int64_t n = voff[G], m = eoff[G];
@@ -607,7 +619,7 @@ int msf_compute_batched(int32_t G, const int64_t *voff, const int64_t *eoff, con
   if (m > 0 && (!src || !dst || !w)) return fail(MSF_ERR_INVALID_ARG, "NULL edge array");
   if (m > 0 && n == 0) return fail(MSF_ERR_INVALID_ARG, "edges given for an empty vertex set");
   cudaStream_t s = (cudaStream_t)stream;
-  if (one_shot_allowed()) {
+  if (one_shot_allowed() && !many_tiny(G, n, m)) {
     const int rc = one_shot(G, voff, eoff, src, dst, w, wtype, edge_mask, labels, totals, s);
     if (rc != SOLVE_NOT_RUN) return rc;
   }

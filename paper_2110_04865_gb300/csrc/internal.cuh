@@ -204,6 +204,7 @@ struct Settle {
 };
 // Pinned host memory of one call (its first 64 bytes zeroed), for a status that
 // a kernel writes and small tables that it reads in place.
+constexpr size_t PIN_KEEP_BYTES = 1 << 20;  // larger blocks are not kept between calls
 struct PinnedWords {
   unsigned *p = nullptr;
   size_t bytes = 0;
@@ -350,6 +351,7 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
 // small.cu
 // The same for graphs that each fit in one SM's shared memory (small_fits),
 // one block per graph.
+constexpr size_t SMALL_TABLE = 44;  // bytes a graph of a batch takes in the pinned table
 bool small_fits(int64_t n, int64_t m);
 bool small_single(int64_t n, int64_t m);  // one graph: faster so than by solve_edges
 int solve_small(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *eoff, const int32_t *src,

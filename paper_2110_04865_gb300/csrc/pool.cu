@@ -158,7 +158,6 @@ void pool_free_after(void *p, cudaStream_t s) {
 namespace {
 std::mutex g_pin_mu;
 std::vector<std::pair<unsigned *, size_t>> g_pin_free;
-constexpr size_t PIN_KEEP_BYTES = 1 << 20;  // larger blocks are not kept
 constexpr size_t PIN_KEEP = 32;             // blocks kept at most
 }  // namespace
 

@@ -579,7 +579,7 @@ int SmallRun::start(int32_t K, const int32_t *which, const int64_t *voff, const 
   int err = MSF_OK;
   // pinned: status words, then the offsets and the blocks' graphs, which the
   // blocks read in place (a copy would cost a call more than their one read)
-  if (int rc = pin.take(64 + (which ? (size_t)K * 44 : 0))) return rc;
+  if (int rc = pin.take(64 + (which ? (size_t)K * SMALL_TABLE : 0))) return rc;
   A.host = pin.p;
   int64_t entries = m + 256;
   for (int32_t k = 0; which && k < K; ++k) entries += eoff[which[k] + 1] - eoff[which[k]] + 128;
