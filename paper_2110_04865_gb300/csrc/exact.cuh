@@ -290,7 +290,8 @@ struct Limit {
     }
   }
   __device__ static uint32_t from_ord(uint32_t o) {
-    const uint32_t b = (o & 0x80000000u) ? o & 0x7fffffffu : ~o;
+    uint32_t b = (o & 0x80000000u) ? o & 0x7fffffffu : ~o;
+    if (b == 0x80000000u) b = 0x80000001u;  // (-0 is ordered as +0: below +0 are the negative weights)
     return (b << 1) > 0xff000000u ? ((b >> 31) ? 0x7fffffffu : 0x7f800000u) : b;
   }
   __device__ __forceinline__ void batch(int64_t e) {  // the batch of edges from e on
