@@ -80,8 +80,12 @@ inline bool two_classes(int64_t n, int64_t m) {
 // loop's, or classes and a replay of the rounds on the forest.  In us, one class /
 // classes: R-MAT 16 of 2^20 edges 178 / 225, (200 000, 2^20) 297 / 349, a 96^3
 // lattice 416 / 515, R-MAT 18 of 2^21 257 / 288, of 2^22 355 / 306; (100 000, 2^21)
-// 395 / 336, (300 000, 3 M) 490 / 389, (10^6, 4 M) 677 / 577.
+// 395 / 336, (300 000, 3 M) 490 / 389, (10^6, 4 M) 677 / 577.  Trees and little more
+// are counted directly whatever their size, as the replay's list is then nearly
+// all of their edges: a path of 8 M vertices 1159 / 2443, (8 M, 8 M) 1212 / 1974,
+// (8 M, 12 M) 1826 / 2222, (8 M, 16 M) 2499 / 2470, (8 M, 24 M) 3667 / 2564.
 inline bool count_by_replay(int64_t n, int64_t m) {
+  if (5 * m < 8 * n) return false;
   return m >= (int64_t)3 << 20 || (m >= (int64_t)3 << 19 && m >= 10 * n);
 }
 // Edges left from which a round's roots are settled in a step of their own:
