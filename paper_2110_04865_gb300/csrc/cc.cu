@@ -46,6 +46,12 @@ constexpr size_t CC_BITS = 224 << 10;  // largest bitmap kept in shared memory
 // bitmap before the parents (its making costs about 7 us at 2^20 vertices).
 constexpr unsigned LONG_LIST = 1u << 12;  // (in units of 256)
 constexpr uint32_t NONE = 0xffffffffu;
+// Up to FEW vertices of many edges each the first offers are collected per block.
+// Calls in us at (vertices, edges), loop over the CSR / edge by edge / collected:
+// (30, 10^6) 150 / 175 / 62, (300, 500 000) 131 / 161 / 63, (300, 2 M) 163 / 191 / 66,
+// (2000, 500 000) 192 / 117 / 88; (2000, 60 000) 182 / 81 / 84, (1296, 5000) 180 / 62
+// / 70.
+constexpr int64_t FEW = 2048;
 // Edges or vertices per block of a call that does not fill the device; one block
 // up to ONE_BLOCK of them, whose barriers are its own (whole calls in us, several
 // blocks / one, uniform: 2000 edges 60 / 45, 5000 65 / 55, 10 000 65 / 61).
@@ -61,6 +67,7 @@ struct CcArgs {
   const int2 *ends;
   int32_t es, vs;      // pages of 2^es edges and 2^vs vertices
   int32_t smem_bits;   // a bitmap of the vertices fits in shared memory
+  int32_t few;         // the first offers are collected per block
   int32_t *p;          // parents
   uint32_t *q;         // smallest offered parent of each root
   uint32_t *deep;      // bitmap: roots of trees that are not stars (and some of their vertices)
@@ -227,7 +234,24 @@ __global__ void __launch_bounds__(CT, 1) k_components(const __grid_constant__ Cc
       return;
     }
     // conditional hooking: every tree is a star
-    if (round == 0) {
+    if (round == 0 && A.few) {
+      // few vertices: their offers meet in the block first (an edge would find
+      // q as it was when its line came to L1, and most edges would offer)
+      for (int i = threadIdx.x; i < (int)n; i += CT) dyn[i] = NONE;
+      __syncthreads();
+      auto body = [&](const PairQuad &x, int) {
+        const int32_t u[4] = {x.s.x, x.s.y, x.s.z, x.s.w}, v[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int32_t lo = min(u[j], v[j]), hi = max(u[j], v[j]);
+          if (lo != hi && (uint32_t)lo < *(volatile uint32_t *)(dyn + hi)) atomicMin(dyn + hi, (uint32_t)lo);
+        }
+      };
+      stream2<PairQuad>(0, (int)P.cap, load, body);
+      __syncthreads();
+      for (int i = threadIdx.x; i < (int)n; i += CT)
+        if (dyn[i] != NONE) offer(q, i, (int32_t)dyn[i]);
+    } else if (round == 0) {
       auto body = [&](const PairQuad &x, int) {
         const int32_t u[4] = {x.s.x, x.s.y, x.s.z, x.s.w}, v[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
         uint32_t old[4];
@@ -472,6 +496,7 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
   A.vs = page_shift(n, warps);
   const size_t bit_bytes = (size_t)((n + 127) / 128) * 16;
   A.smem_bits = bit_bytes <= CC_BITS;
+  A.few = n <= FEW && m >= 32 * n;
   size_t off = 0;
   auto place = [&](size_t bytes) {
     const size_t at = off;
@@ -497,7 +522,8 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
   A.list = (int2 *)(base + o_list);
   A.host = pin.p;
   MSF_CK(cudaMemsetAsync(A.ctl, 0, sizeof(CcCtrl), s));
-  const size_t dyn = A.smem_bits ? bit_bytes : 0;
+  size_t dyn = A.smem_bits ? bit_bytes : 0;
+  if (A.few && dyn < FEW * 4) dyn = FEW * 4;
   cudaError_t e = cudaFuncSetAttribute(k_components, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_BITS);
   void *args[] = {&A};
   if (e == cudaSuccess)
