@@ -133,9 +133,11 @@ def _one(n: int, src, dst, w, labels: bool = True):
     _check_i32(src, "src")
     m = int(dst.shape[0])
     wtype = _wtype(w)
+    if not 0 <= n < 1 << 31:  # refused by the library, before anything of that size is allocated
+        n = -1 if n < 0 else 1 << 31
     off = _I64x4(0, n, 0, m)  # voff, then eoff
     voff = ctypes.addressof(off)
-    return _solve(1, voff, voff + 16, n, m, src, dst, w, wtype, labels)
+    return _solve(1, voff, voff + 16, n if 0 <= n < 1 << 31 else 0, m, src, dst, w, wtype, labels)
 
 
 def _solve(G: int, voff: int, eoff: int, n: int, m: int, src, dst, w, wtype: int, labels: bool):
