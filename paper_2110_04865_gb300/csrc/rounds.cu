@@ -793,18 +793,53 @@ __global__ void __launch_bounds__(BT) k_backward(int64_t m, int32_t G, const int
 // copied or waited for (the copy, its block and the wait took 23 us a call of 256
 // graphs and 1.7 M edges, this 5).  A thread takes 16 edges of one 16-byte mask
 // load and looks for the first one's graph, among offsets in shared memory, when
-// one of them is in the forest.
+// one of them is in the forest.  Off a 16-byte boundary a warp takes 256 edges, its
+// lanes neighbouring ones (900 graphs of 2^26 edges in all: 126 to 129 us; by
+// sixteens, whose single loads and stores lie apart, 275 to 318; one search an
+// edge 390 to 406, or 159 where no edge is in the forest).
 __global__ void __launch_bounds__(BT) k_backward_few(const __grid_constant__ BackwardOffsets off, int64_t m, int32_t G,
                                                      const uint8_t *mask, const double *gt, float *gw, int vec) {
   __shared__ uint32_t end[BACKWARD_GRAPHS];  // first edge behind each graph
   for (int i = threadIdx.x; i < G; i += BT) end[i] = off.end[i];
   __syncthreads();
+  auto graph_of_edge = [&](int64_t e) {  // the first graph whose end lies behind e
+    int lo = 0, hi = G - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((int64_t)end[mid] > e) hi = mid;
+      else lo = mid + 1;
+    }
+    return lo;
+  };
+  if (!vec) {  // a warp's lanes take neighbouring edges, EDGES in all, from one search
+    constexpr int EDGES = 256;
+    const int lane = threadIdx.x & 31;
+    for (int64_t c = tid64() >> 5; c * EDGES < m; c += stride64() >> 5) {
+      const int64_t e0 = c * EDGES + lane;
+      bool on[EDGES / 32];
+#pragma unroll
+      for (int j = 0; j < EDGES / 32; ++j) on[j] = e0 + 32 * j < m && mask[e0 + 32 * j];
+      int lo = graph_of_edge(c * EDGES);
+      float x = (float)gt[lo];
+#pragma unroll
+      for (int j = 0; j < EDGES / 32; ++j) {
+        const int64_t e = e0 + 32 * j;
+        if (e >= m) break;
+        if ((int64_t)end[lo] <= e) {
+          while ((int64_t)end[lo] <= e) ++lo;
+          x = (float)gt[lo];
+        }
+        gw[e] = on[j] ? x : 0.f;
+      }
+    }
+    return;
+  }
   const int64_t chunks = (m + 15) >> 4;
   for (int64_t i = tid64(); i < chunks; i += stride64()) {
     const int64_t e0 = i << 4;
     const int k = (int)(m - e0 < 16 ? m - e0 : 16);
     uint32_t b[4] = {0u, 0u, 0u, 0u};
-    if (k == 16 && vec) {
+    if (k == 16) {
       const uint4 x = __ldcs(reinterpret_cast<const uint4 *>(mask + e0));
       b[0] = x.x, b[1] = x.y, b[2] = x.z, b[3] = x.w;
     } else {
@@ -816,12 +851,7 @@ __global__ void __launch_bounds__(BT) k_backward_few(const __grid_constant__ Bac
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = 0.f;
     if (b[0] | b[1] | b[2] | b[3]) {
-      int lo = 0, hi = G - 1;  // the first graph whose end lies behind e0
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if ((int64_t)end[mid] > e0) hi = mid;
-        else lo = mid + 1;
-      }
+      int lo = graph_of_edge(e0);
       float x = (float)gt[lo];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
@@ -833,7 +863,7 @@ __global__ void __launch_bounds__(BT) k_backward_few(const __grid_constant__ Bac
         v[j] = x;
       }
     }
-    if (k == 16 && vec) {
+    if (k == 16) {
       float4 *o = reinterpret_cast<float4 *>(gw + e0);
 #pragma unroll
       for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -925,10 +955,10 @@ void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cuda
 }
 void launch_backward_few(const BackwardOffsets &off, int64_t m, int32_t G, const uint8_t *mask, const double *gt,
                          float *gw, cudaStream_t s) {
-  int64_t b = ((m + 15) / 16 + BT - 1) / BT;
+  const int vec = ((reinterpret_cast<uintptr_t>(mask) | reinterpret_cast<uintptr_t>(gw)) & 15) == 0;
+  int64_t b = ((vec ? (m + 15) / 16 : (m + 7) / 8) + BT - 1) / BT;
   if (b > vgrid(8)) b = vgrid(8);
   if (b < 1) b = 1;
-  const int vec = ((reinterpret_cast<uintptr_t>(mask) | reinterpret_cast<uintptr_t>(gw)) & 15) == 0;
   k_backward_few<<<(int)b, BT, 0, s>>>(off, m, G, mask, gt, gw, vec);
 }
 void launch_backward(int64_t m, int32_t G, const int64_t *eoff_d, const uint8_t *mask, const double *gt,
