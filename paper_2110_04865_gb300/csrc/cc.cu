@@ -55,7 +55,7 @@ constexpr int64_t FEW = 2048;
 // Edges or vertices per block of a call that does not fill the device; one block
 // up to ONE_BLOCK of them, whose barriers are its own (whole calls in us, several
 // blocks / one, uniform: 2000 edges 60 / 45, 5000 65 / 55, 10 000 65 / 61).
-constexpr int64_t BLOCK_SHARE = 1024, ONE_BLOCK = 8192;
+constexpr int64_t BLOCK_SHARE = 4096, ONE_BLOCK = 8192;
 
 struct CcCtrl {
   unsigned long long arrive[2];
@@ -489,7 +489,8 @@ int components_pairs(int64_t n, int64_t m, const int2 *ends, int32_t *labels, in
   A.labels = labels;
   int64_t want = ((m > n ? m : n) + BLOCK_SHARE - 1) / BLOCK_SHARE;
   if (want < 1 || (m <= ONE_BLOCK && n <= ONE_BLOCK)) want = 1;
-  const int64_t cap = (int64_t)sm_count();
+  DeviceShare share(n, m);
+  const int64_t cap = (int64_t)share.sms;
   const int blocks = (int)(want < cap ? want : cap);
   const int64_t warps = (int64_t)blocks * CW;
   A.es = page_shift(m, warps);

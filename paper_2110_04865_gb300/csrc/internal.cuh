@@ -214,6 +214,22 @@ struct PinnedWords {
 
 // ---- device properties ---------------------------------------------------------
 int sm_count();
+// A solver that fills the device with one cooperative kernel, as long as the object
+// lives: `sms` are the SMs it takes.  One at a time takes them all; calls of several
+// threads at once take a half to a quarter, so that they run side by side instead
+// of one after the other (its results do not depend on the number of blocks).
+// Us a call in a row of calls, one thread / eight, all SMs each / eight, shared:
+// msf_compute on 2^16 vertices and 2^18 edges 240 / 185 / 75, 2^20 edges 310 / 252 /
+// 134, 2^18 vertices and 2^20 edges 330 / 278 / 151, 2^20 and 2^24 880 / 700 / 478
+// (in the round loop, whose launches interleave: 127, 181, 221, 1480 by eight).
+struct DeviceShare {
+  int sms;
+  DeviceShare(int64_t n, int64_t m);
+  ~DeviceShare();
+
+ private:
+  int dev = 0;
+};
 
 // ---- options ---------------------------------------------------------------------
 struct Options {

@@ -8,6 +8,7 @@
 // cached block of the device is released and the request retried once.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -218,6 +219,21 @@ int sm_count() {
   }
   return cached[dev];
 }
+
+namespace {
+std::atomic<int> g_solvers[64];           // at work on each device
+constexpr int64_t SHARED_WORK = 1 << 26;  // edges and vertices up to which a call shares
+}  // namespace
+
+DeviceShare::DeviceShare(int64_t n, int64_t m) : sms(sm_count()) {
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) dev = 0;
+  const int others = g_solvers[dev].fetch_add(1, std::memory_order_relaxed);
+  if (others > 0 && n <= SHARED_WORK && m <= SHARED_WORK) sms /= others < 3 ? others + 1 : 4;
+  if (sms < 1) sms = 1;
+}
+
+DeviceShare::~DeviceShare() { g_solvers[dev].fetch_sub(1, std::memory_order_relaxed); }
 
 Options &options() {
   static Options o;

@@ -96,8 +96,10 @@ inline bool count_by_replay(int64_t n, int64_t m) {
 // with rising weights and permuted ids, 40 000 vertices 177 -> 140 us, 131 000
 // 224 -> 155; for all graphs that line took R-MAT 16 from 174 to 184).
 constexpr unsigned long long SMALL = 1 << 17, SMALL_CHAINS = 1 << 15;
-// Edges or vertices per block: a call that does not fill the device.
-constexpr int64_t BLOCK_SHARE = 1024;
+// Edges or vertices per block of a call that does not fill the device.  (1024 a
+// block take all SMs from 152 000 on and are no faster: 209 us against 205 at
+// 30 000 vertices and 200 000 edges; 8192 251.)
+constexpr int64_t BLOCK_SHARE = 4096;
 
 constexpr size_t SMEM_BITS = 224 << 10;  // largest bitmap kept in shared memory
 
@@ -1278,7 +1280,9 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
   // blocks: one per BLOCK_SHARE edges or vertices, at most one per SM
   int64_t want = ((m > n ? m : n) + BLOCK_SHARE - 1) / BLOCK_SHARE;
   if (want < 1) want = 1;
-  const int64_t cap = (int64_t)sm_count() - spare;  // (other blocks run on `spare` SMs meanwhile)
+  DeviceShare share(n, m);
+  int64_t cap = (int64_t)sm_count() - spare;  // (other blocks run on `spare` SMs meanwhile)
+  if (cap > share.sms) cap = share.sms;
   const int blocks = (int)(want < cap ? want : cap);
   const int64_t warps = (int64_t)blocks * EW;
   A.es = page_shift(m, warps);

@@ -263,6 +263,8 @@ int fail(int code, const std::string &m) {
 int cuda_fail(cudaError_t e, const char *) { return e == cudaErrorMemoryAllocation ? MSF_ERR_OOM : MSF_ERR_CUDA; }
 const char *last_error_cstr() { return message.c_str(); }
 int sm_count() { return 152; }
+DeviceShare::DeviceShare(int64_t, int64_t) : sms(152) {}
+DeviceShare::~DeviceShare() {}
 Options &options() {
   static Options o;
   return o;
