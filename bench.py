@@ -22,7 +22,8 @@ Also reported on the same JSON line:
   batched       one msf_compute_batched call on 4096 uneven graphs vs a loop
                 of per-graph build + compute + free calls on the same GPU;
   pairwise_vs_multilinear  the Sec. 4.1 ablation on R-MAT 17, edge factor 8:
-                round loop and full sweep, fused kernel vs two-pass form.
+                the round loop (selected for both) with the fused kernel vs the
+                two-pass form, and msf_min_edge in both.
 With --impl reference the CPU oracle is timed as the reference arm.
 Under torchrun (N > 1) every rank solves its own replica of the workload
 (the forest of one graph is not sharded); value = all ranks' edges / max time.
@@ -655,9 +656,12 @@ def bench_pairwise(dev, sh, flush):
     """Sec. 4.1 / Sec. 7.4 ablation on R-MAT scale 17, edge factor 8: the fused
     multilinear min-edge kernel against the pairwise formulation (a first pass
     writes p_j next to every slot, a second reduces the (a_ij, p_j) pairs).
-    Per formulation: the whole round loop (msf_compute) and one full sweep
-    (msf_min_edge, every slot live), best of 5 each with L2 flushed; the two
-    forests must be identical."""
+    Per formulation: the whole round loop (msf_compute with the builder named,
+    which selects the loop; by default the forest is solved from the edges
+    without either formulation) and one msf_min_edge with every slot live
+    (pairwise against the kernel made for it, which gathers the parent of a
+    row's smallest slots only), best of 5 each with L2 flushed; the two forests
+    must be identical."""
     import numpy as np
     import torch
 
@@ -667,12 +671,13 @@ def bench_pairwise(dev, sh, flush):
     n, m = d["n"], len(d["src"])
     src, dst, w = (torch.from_numpy(d[k]).to(dev) for k in ("src", "dst", "w"))
     stream = torch.cuda.current_stream(dev)
-    old = _abi.msf_get_option(_abi.OPT_KERNEL)
+    old = {o: _abi.msf_get_option(o) for o in (_abi.OPT_KERNEL, _abi.OPT_BUILD)}
     g = _abi.msf_build_csr(n, m, src.data_ptr(), dst.data_ptr(), 0, w.data_ptr(), 0, 0, sh)
     parent = torch.arange(n, dtype=torch.int32, device=dev)
     r = torch.empty(n, dtype=torch.int64, device=dev)
     out, masks = {}, []
     try:
+        _abi.msf_set_option(_abi.OPT_BUILD, max(1, int(old[_abi.OPT_BUILD])))
         for name, k in (("multilinear", 0), ("pairwise", 1)):
             _abi.msf_set_option(_abi.OPT_KERNEL, k)
             mask = torch.empty(m, dtype=torch.uint8, device=dev)
@@ -695,7 +700,8 @@ def bench_pairwise(dev, sh, flush):
             out[name] = {"compute_ms": min(ct), "sweep_ms": min(st)}
             masks.append(mask.cpu().numpy())
     finally:
-        _abi.msf_set_option(_abi.OPT_KERNEL, old)
+        for o, v in old.items():
+            _abi.msf_set_option(o, v)
         _abi.msf_free(g)
     assert np.array_equal(masks[0], masks[1])
     out.update({"workload": workload_desc("rmat17e8"), "n": n, "m": m, "same_forest": True,
