@@ -262,6 +262,19 @@ def env_shape():
             "blocks_per_sm": int(os.environ.get("MSF_BPS", "4")), "sweep": int(os.environ.get("MSF_SWEEP", "0"))}
 
 
+def sweep_and_path():
+    """Bytes a slot that msf_min_edge's sweep cannot do without, and what
+    msf_compute runs under the options of the moment: the round loop, or the
+    solvers from the edges.  Every form streams a slot's column and key; the
+    loop's forms and the pairwise one gather a parent for each slot besides,
+    msf_min_edge's own one for a row's smallest slots only."""
+    from paper_2110_04865_gb300 import _abi, autotune
+    g = _abi.msf_get_option
+    own = g(_abi.OPT_SWEEP) == 0 and g(_abi.OPT_KERNEL) == 0
+    loop = autotune.round_loop_selected() or g(_abi.OPT_SWEEP) != 0 or g(_abi.OPT_COMPACT_TAU) != 0.5
+    return 12 if own else 16, "loop" if loop else "edges"
+
+
 def ingest_traffic(args):
     """profiles/min_edge_traffic.json from the ncu CSV of
     `bench.py --profile-min-edge --workload W` run with the sweep shape in
@@ -569,7 +582,8 @@ def main():
     compute_ms = statistics.median(c for _, c in bparts)
 
     k_ms = statistics.median(k_times)
-    alg_bytes = 16 * gst.nnz + 24 * gst.rows
+    slot_bytes, path = sweep_and_path()
+    alg_bytes = slot_bytes * gst.nnz + 24 * gst.rows
     peak, peak_kind = peaks()
     achieved = alg_bytes / (k_ms / 1e3) / 1e9
     traffic = None
@@ -624,7 +638,8 @@ def main():
                        "edges_without_self_loops": int(gst.nnz) // 2,
                        "min_edge_tile": ({k: tuned[k] for k in autotune.CONFIG_KEYS}
                                          if tuned else None),
-                       "exec": args.exec, "builder": args.build, "kernel": args.kernel,
+                       "exec": args.exec if path == "loop" else "cooperative kernels", "builder": args.build,
+                       "kernel": args.kernel if path == "loop" else "solved from the edges, no sweep",
                        "shortcut": args.shortcut,
                        "parallelism": "replicas" if ws > 1 else "single GPU"},
             "e2e": {"value": ws * m / t_e2e, "unit": "edges/s", "h2d_bytes_per_step": m * 12,
@@ -635,7 +650,7 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                          "kernel": "min-edge sweep (multilinear + projection)", "alg_bytes": alg_bytes,
-                         "ms": k_ms, "alg_bytes_rule": "16 B/slot + 24 B/row",
+                         "ms": k_ms, "alg_bytes_rule": f"{slot_bytes} B/slot + 24 B/row",
                          "samples_ms": [round(x, 4) for x in k_times]},
             "cpu_baseline": cpu,
             "cpu_baseline_all_cores": cpu_all,
