@@ -113,9 +113,10 @@ int msf_compute(msf_graph *g, uint8_t *edge_mask, int32_t *labels, double *total
  * Graphs that each fit in one SM's shared memory (about 10 bytes a vertex and
  * a bit an edge: some 20 000 vertices) are solved side by side, one thread
  * block each; the larger ones (with G = 1 the one-shot form of build, compute
- * and free) are solved together from their edge lists without a CSR.  The
- * forest, labels and total are those of the round loop over the disjoint union,
- * since they are unique.  An option
+ * and free) are solved together from their edge lists without a CSR.  Very many
+ * tiny graphs (from some 24 000 on, of fewer than 160 to 200 vertices and edges
+ * each) take the round loop over the CSR of their disjoint union.  The forest,
+ * labels and totals are the same either way, since they are unique.  An option
  * that asks for a schedule, a builder, a kernel form, the host-driven loop, or
  * a round or jump limit below its default always selects the round loop.
  *   voff, eoff  HOST int64[G+1] vertex and edge offsets, voff[0] = eoff[0] = 0,
@@ -272,17 +273,22 @@ typedef struct msf_stats {
   int64_t n, m;          /* vertices and edges */
   int64_t nnz;           /* directed CSR slots of the original graph */
   int64_t rows;          /* CSR rows (vertices of nonzero degree) */
-  int32_t rounds;        /* rounds of the loop, the final one without hooks included */
-  int32_t compactions;   /* rounds that compacted the edge list */
+  int32_t rounds;        /* rounds of the loop, the final one without hooks included (counted
+                            also when the forest is solved from the edges) */
+  int32_t compactions;   /* rounds that compacted the edge list; 0 when the forest is solved from
+                            the edges, which has no such step */
   int64_t forest_edges;  /* edges in the forest */
-  int32_t jump_steps;    /* pointer-jumping steps over all rounds */
+  int32_t jump_steps;    /* pointer-jumping steps over all rounds; solved from the edges, the passes
+                            in which that solver lets the hooked roots find their new ones (it
+                            may follow a round's chains in one, so the two differ) */
   float min_edge_ms;     /* duration of the sweep kernel in the last msf_min_edge call
                             (CUDA events on the caller's stream around that launch only) */
   int32_t cc_rounds;     /* rounds of the last msf_connected_components call */
   int32_t kernels;       /* kernels the library ran for msf_build_csr plus the last msf_compute
                             (host launches and the executed nodes of the round-loop graph) */
-  int32_t builder;       /* the CSR builder msf_build_csr ran: 1 per-vertex atomic, 2 radix,
-                            3 bucketed (MSF_OPT_BUILD's numbering) */
+  int32_t builder;       /* the CSR builder msf_build_csr ran: 1 per-vertex atomic (a small
+                            graph's in one kernel), 2 radix, 3 bucketed (MSF_OPT_BUILD's
+                            numbering) */
 } msf_stats;
 
 int msf_get_stats(const msf_graph *g, msf_stats *out);
@@ -292,8 +298,8 @@ enum msf_option {
   MSF_OPT_COMPACT_TAU = 0,   /* compact when live slots < tau * slots (0 < tau < 1; default 0.5; 0 = never) */
   MSF_OPT_ROUND_LIMIT = 1,   /* maximum rounds (default 64) */
   MSF_OPT_JUMP_LIMIT = 2,    /* maximum shortcut passes per round (default 64) */
-  MSF_OPT_SLOTS_PER_LANE = 3,/* min-edge tile: slots per lane, 4, 8 or 16 (default 4;
-                                msf_min_edge then takes 8 where rows are long enough) */
+  MSF_OPT_SLOTS_PER_LANE = 3,/* min-edge tile: slots per lane, 4, 8 or 16 (default 4; for 4
+                                msf_min_edge takes 8 where rows have four slots or more) */
   MSF_OPT_BLOCKS_PER_SM = 4, /* min-edge grid: resident blocks per SM (1..8, default 4) */
   MSF_OPT_PREFETCH = 5,      /* the round loop's sweep loads the next tile early: 0 or 1
                                 (default 0) */
@@ -306,11 +312,13 @@ enum msf_option {
   MSF_OPT_KERNEL = 9,        /* 0 = fused multilinear min-edge kernel (default); 1 = pairwise
                                 formulation of Sec. 4.1: one pass writes p_j next to every slot
                                 (nnz extra writes and an nnz-word buffer), a second reduces */
-  MSF_OPT_BUILD = 10,        /* CSR builder: 0 = automatic (default: bucketed from 2^20 edges
+  MSF_OPT_BUILD = 10,        /* CSR builder: 0 = automatic (default: bucketed from 2^20 edges, or
+                                from 12 * 2^20 slots of CSR input on at most 2^22 vertices,
                                 unless a sample shows locality -- consecutive sampled edges with
                                 endpoints close together, as in a lattice listed vertex by vertex
                                 or a batch listed graph by graph -- then per-vertex atomic
-                                counters, as for small graphs), 1 = atomic,
+                                counters, as for smaller graphs; the smallest in one kernel of
+                                one block), 1 = atomic,
                                 2 = radix grouping, 3 = bucketed (rows grouped in at most 1024
                                 buckets of consecutive vertices, counted in shared memory).  All
                                 give the same CSR up to the order of slots inside a row. */

@@ -56,12 +56,12 @@ struct Pages {
 // above the block's addend, so the word that says that all have come also holds the
 // sum (two words in turn: a block arrives at the next barrier but one only after all
 // have read this one's).  An arrival takes the block's addend of the word's last
-// barrier out again, so a sum is that of one barrier; until all have come it may be
-// negative, which makes the count above too small, never too large.  The wait is
-// bounded.  One block's barrier is about 2 us of
-// latency; what the words save is measured on whole calls, fences around the
-// arrival, a counter and its read beside it before, this after: R-MAT 16
-// 203 -> 173 us, R-MAT 20 500 -> 455, uniform m = 16 n 553 -> 505.
+// barrier out again, so a sum is that of one barrier; until all have come it holds
+// one addend of every block, this barrier's or the last one's: it neither borrows
+// from the count above nor carries into it.  The wait is bounded.  One
+// barrier is about 2 us of latency; what the words save is measured on whole calls,
+// fences around the arrival, a counter and its read beside it before, this after:
+// R-MAT 16 203 -> 173 us, R-MAT 20 500 -> 455, uniform m = 16 n 553 -> 505.
 struct GridBarrier {  // in shared memory
   static constexpr int SHIFT = 46;  // arrivals above (1700 barriers of 152 blocks), sums below
   unsigned long long *word;         // [2], zero at the start

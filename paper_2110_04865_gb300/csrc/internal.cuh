@@ -353,7 +353,7 @@ struct LoopCounts {
   int32_t hooked;  // rounds in which roots hooked
   uint32_t left;   // trees with edges after the last of them
   uint32_t edges;  // forest edges
-  int32_t passes;  // passes that settle the hooked roots
+  int32_t passes;  // passes that settle the hooked roots, as the solver makes them
   int32_t kernels;
 };
 int solve_pairs(int64_t n, int64_t m, const int2 *ends, const uint32_t *w, int wtype, uint8_t *mask, int32_t *labels,

@@ -1,10 +1,10 @@
-// One-shot forest of one edge list, without a CSR.
+// Forests from edge lists, without a CSR: of one list, of the larger graphs of a
+// batch, and of a kept graph from the ends and weights that its handle holds.
 //
-// A caller that hands over an edge list and keeps no handle needs no adjacency
-// structure: the strict order on (weight, edge index) makes the forest unique,
-// so any exact method returns the round loop's mask, labels and total.  The
-// CSR costs several passes over two records per edge and every round of the
-// loop sweeps all of them; here the edges are read once or twice:
+// The strict order on (weight, edge index) makes the forest unique, so any exact
+// method returns the round loop's mask, labels and total.  A CSR costs several
+// passes over two records per edge and every round of the loop sweeps all of
+// them; here the edges are read once or twice:
 //
 //   select   one pass validates the edges and keeps the light ones, in two
 //            classes: about CLASS1 * n edges below a first threshold key, those
