@@ -797,8 +797,9 @@ __global__ void __launch_bounds__(BT) k_backward(int64_t m, int32_t G, const int
 // lanes neighbouring ones (900 graphs of 2^26 edges in all: 126 to 129 us; by
 // sixteens, whose single loads and stores lie apart, 275 to 318; one search an
 // edge 390 to 406, or 159 where no edge is in the forest).
+template <bool VEC>
 __global__ void __launch_bounds__(BT) k_backward_few(const __grid_constant__ BackwardOffsets off, int64_t m, int32_t G,
-                                                     const uint8_t *mask, const double *gt, float *gw, int vec) {
+                                                     const uint8_t *mask, const double *gt, float *gw) {
   __shared__ uint32_t end[BACKWARD_GRAPHS];  // first edge behind each graph
   for (int i = threadIdx.x; i < G; i += BT) end[i] = off.end[i];
   __syncthreads();
@@ -811,7 +812,7 @@ __global__ void __launch_bounds__(BT) k_backward_few(const __grid_constant__ Bac
     }
     return lo;
   };
-  if (!vec) {  // a warp's lanes take neighbouring edges, EDGES in all, from one search
+  if (!VEC) {  // a warp's lanes take neighbouring edges, EDGES in all, from one search
     constexpr int EDGES = 256;
     const int lane = threadIdx.x & 31;
     for (int64_t c = tid64() >> 5; c * EDGES < m; c += stride64() >> 5) {
@@ -955,11 +956,12 @@ void launch_check_range(const int32_t *a, int64_t n, int32_t hi, int *flag, cuda
 }
 void launch_backward_few(const BackwardOffsets &off, int64_t m, int32_t G, const uint8_t *mask, const double *gt,
                          float *gw, cudaStream_t s) {
-  const int vec = ((reinterpret_cast<uintptr_t>(mask) | reinterpret_cast<uintptr_t>(gw)) & 15) == 0;
+  const bool vec = ((reinterpret_cast<uintptr_t>(mask) | reinterpret_cast<uintptr_t>(gw)) & 15) == 0;
   int64_t b = ((vec ? (m + 15) / 16 : (m + 7) / 8) + BT - 1) / BT;
   if (b > vgrid(8)) b = vgrid(8);
   if (b < 1) b = 1;
-  k_backward_few<<<(int)b, BT, 0, s>>>(off, m, G, mask, gt, gw, vec);
+  if (vec) k_backward_few<true><<<(int)b, BT, 0, s>>>(off, m, G, mask, gt, gw);
+  else k_backward_few<false><<<(int)b, BT, 0, s>>>(off, m, G, mask, gt, gw);
 }
 void launch_backward(int64_t m, int32_t G, const int64_t *eoff_d, const uint8_t *mask, const double *gt,
                      float *gw, cudaStream_t s) {
