@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       }
       lo = __reduce_min_sync(FULL, lo);
       up = __reduce_max_sync(FULL, up);
-      const int rank = (int)(LIGHT * (double)n / (double)m * (32.0 * PER));
+      const int rank = light_rank(LIGHT, n, m, 32 * PER, 8);
       auto below_key = [&](uint32_t tw, uint32_t te) {
         int c = 0;
 #pragma unroll

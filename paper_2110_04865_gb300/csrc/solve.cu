@@ -1295,8 +1295,8 @@ int solve(int32_t K, const int32_t *which, const int64_t *voff, const int64_t *e
     if ((double)m > 1.25 * la * (double)n && la < lb) A.classes = 2;
     if ((double)m > 1.25 * lb * (double)n) A.classes = 3;
     A.second = A.classes > 1 && la < lb;
-    A.rank[0] = (unsigned)(la * (double)n / (double)m * SAMPLES);
-    A.rank[1] = (unsigned)(lb * (double)n / (double)m * SAMPLES);
+    A.rank[0] = (unsigned)light_rank(la, n, m, SAMPLES, la < lb ? 8 : 16);
+    A.rank[1] = (unsigned)light_rank(lb, n, m, SAMPLES, 16);
   }
   const size_t bit_bytes = (size_t)((n + 127) / 128) * 16;
   A.smem_bits = A.classes > 2 && bit_bytes <= SMEM_BITS;
