@@ -220,6 +220,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     for (int j = 0; j < KEEP; ++j)
       if (in >> j & 1u) mark(ke[j], kw[j]);
   };
+  // The warp's list lies in the places of its batches of 128 edges, batch k of warp
+  // w the one w + k * NW of the graph: an input sorted by weight, or with one
+  // weight for all, has its light edges side by side, and one run of edges per
+  // warp gave nearly all of them to one (2 graphs of 4000 vertices and 400 000
+  // sorted edges 850 us, now 257; with weights in any order 2 % more than runs).
+  auto place = [&](int i) { return (((i >> 7) * NW + wid) << 7) | (i & 127); };
   // Rounds on the warp's list; one of at most KEEP entries a lane goes to
   // registers first.
   uint4 *L = nullptr;
@@ -230,7 +236,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
 #pragma unroll
         for (int j = 0; j < KEEP; ++j) {
           const int i = j * 32 + lane;
-          const uint4 x = i < cnt ? L[i] : make_uint4(0u, 0u, 0u, 0u);
+          const uint4 x = i < cnt ? L[place(i)] : make_uint4(0u, 0u, 0u, 0u);
           kuv[j] = x.x;
           ke[j] = x.z;
           kw[j] = x.w;
@@ -240,17 +246,18 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       }
       int out = 0;
       if (threadIdx.x == 0) s_pairs[hooked & 1] = 0;
-      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {
+      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {  // (a batch)
+        const uint4 *Lb = L + place(b0);
         uint4 x[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? L[b0 + j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
+        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? Lb[j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int j = 0; j < U; ++j) {
           if (x[j].x) x[j].x = relabel(x[j].x);
           const unsigned bal = __ballot_sync(FULL, x[j].x != 0);
           if (x[j].x) {
             min_weight(x[j].x, x[j].w);
-            L[out + __popc(bal & below)] = x[j];
+            L[place(out + __popc(bal & below))] = x[j];
           }
           out += __popc(bal);
         }
@@ -258,19 +265,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       __syncwarp();
       cnt = out;
       if (!__syncthreads_or(cnt > 0)) return;
-      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {
+      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {  // (a batch)
+        const uint4 *Lb = L + place(b0);
         uint4 x[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? L[b0 + j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
+        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? Lb[j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int j = 0; j < U; ++j)
           if (x[j].x) min_edge(x[j].x, x[j].z, x[j].w);
       }
       __syncthreads();
-      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {
+      for (int b0 = 0; b0 < cnt; b0 += 32 * U) {  // (a batch)
+        const uint4 *Lb = L + place(b0);
         uint4 x[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? L[b0 + j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
+        for (int j = 0; j < U; ++j) x[j] = b0 + j * 32 + lane < cnt ? Lb[j * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int j = 0; j < U; ++j)
           if (x[j].x && hook(x[j].x, x[j].z, x[j].w)) mark(x[j].z, x[j].w);
@@ -352,24 +361,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     __syncthreads();
     Limit<F32> limit(filter ? s_thresh : KEY_INF);
 
-    // every warp: a run of whole batches of 128 edges (indices from the first
-    // batch on), and the list region that starts at its first edge
+    // the warp's batches of 128 edges (indices from the first batch on)
     const int64_t a0 = e0 & ~(int64_t)127;
     const int first = (int)(e0 - a0), end = (int)(e1 - a0);
-    const int per = ((end + NW - 1) / NW + 127) / 128 * 128;
-    const int lo = wid * per, hi = lo + per < end ? lo + per : end;
+    const int batches = (end + 127) >> 7, mine = wid < batches ? ((batches - wid + NW - 1) / NW) << 7 : 0;
     const int32_t *S = A.src + a0, *D = A.dst + a0;
     const uint32_t *W = A.w + a0;
     const bool vec = A.vec != 0;
-    L = A.list + (A.loff ? A.loff[blockIdx.x] : 0) + lo;
+    L = A.list + (A.loff ? A.loff[blockIdx.x] : 0);
     int cnt = 0;
     {
-      auto load = [&](int b) {
-        return A.ends ? pair_quad(A.ends, W, b + 4 * lane, hi)
-                      : edge_quad<true>(S, D, W, vec, b + 4 * lane, first, hi);
+      auto load = [&](int k) {
+        const int i = place(k) + 4 * lane, hi = k < mine ? end : 0;
+        return A.ends ? pair_quad(A.ends, W, i, hi) : edge_quad<true>(S, D, W, vec, i, first, hi);
       };
-      auto body = [&](const EdgeQuad &q, int b) {
-        const int i = b + 4 * lane;
+      auto body = [&](const EdgeQuad &q, int k) {
+        const int b = place(k), i = b + 4 * lane;
         limit.batch(a0 + b);
         const uint32_t u[4] = {(uint32_t)q.s.x, (uint32_t)q.s.y, (uint32_t)q.s.z, (uint32_t)q.s.w};
         const uint32_t v[4] = {(uint32_t)q.d.x, (uint32_t)q.d.y, (uint32_t)q.d.z, (uint32_t)q.d.w};
@@ -381,12 +388,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
           const bool sel = limit.below(w[j]) && u[j] != v[j];
           const unsigned bal = __ballot_sync(FULL, sel);
           if (sel)
-            L[cnt + __popc(bal & below)] = make_uint4(u[j] | (v[j] << 16), 0u, (uint32_t)a0 + (uint32_t)(i + j),
+            L[place(cnt + __popc(bal & below))] = make_uint4(u[j] | (v[j] << 16), 0u, (uint32_t)a0 + (uint32_t)(i + j),
                                                       ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
           cnt += __popc(bal);
         }
       };
-      stream2<EdgeQuad>(lo, hi, load, body);
+      stream2<EdgeQuad>(0, mine, load, body);
       __syncwarp();
     }
     if (invalid()) return;
@@ -394,9 +401,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     if (filter) {
       // the edges between components (the heavy ones: a light edge lies inside)
       cnt = 0;
-      auto load = [&](int b) { return edge_quad<false>(S, D, W, vec, b + 4 * lane, first, hi); };
-      auto body = [&](const EdgeQuad &q, int b) {
-        const int i = b + 4 * lane;
+      auto load = [&](int k) {
+        return edge_quad<false>(S, D, W, vec, place(k) + 4 * lane, first, k < mine ? end : 0);
+      };
+      auto body = [&](const EdgeQuad &q, int k) {
+        const int i = place(k) + 4 * lane;
         const uint32_t u[4] = {p[q.s.x], p[q.s.y], p[q.s.z], p[q.s.w]};
         const uint32_t v[4] = {p[q.d.x], p[q.d.y], p[q.d.z], p[q.d.w]};
         uint32_t w[4];
@@ -407,12 +416,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
           const bool sel = u[j] != v[j];
           const unsigned bal = __ballot_sync(FULL, sel);
           if (sel)
-            L[cnt + __popc(bal & below)] = make_uint4(u[j] | (v[j] << 16), 0u, (uint32_t)a0 + (uint32_t)(i + j),
+            L[place(cnt + __popc(bal & below))] = make_uint4(u[j] | (v[j] << 16), 0u, (uint32_t)a0 + (uint32_t)(i + j),
                                                       ord_weight_dev(w[j], F32 ? MSF_F32 : MSF_U32));
           cnt += __popc(bal);
         }
       };
-      stream2<EdgeQuad>(lo, hi, load, body);
+      stream2<EdgeQuad>(0, mine, load, body);
       __syncwarp();
       rounds(cnt);
     }
@@ -582,7 +591,7 @@ int SmallRun::start(int32_t K, const int32_t *which, const int64_t *voff, const 
   if (int rc = pin.take(64 + (which ? (size_t)K * SMALL_TABLE : 0))) return rc;
   A.host = pin.p;
   int64_t entries = m + 256;
-  for (int32_t k = 0; which && k < K; ++k) entries += eoff[which[k] + 1] - eoff[which[k]] + 128;
+  for (int32_t k = 0; which && k < K; ++k) entries += eoff[which[k] + 1] - eoff[which[k]] + 256;
   char *base = (char *)pool_alloc((size_t)entries * 16, &err);
   if (err) return err;
   list = base;
@@ -625,7 +634,7 @@ int SmallRun::start(int32_t K, const int32_t *which, const int64_t *voff, const 
       he[2 * k] = eoff[g];
       he[2 * k + 1] = eoff[g + 1];
       hl[k] = entry;
-      entry += eoff[g + 1] - eoff[g] + 128;
+      entry += eoff[g + 1] - eoff[g] + 256;
     }
     // one launch per block size, side by side: 1024 threads (one block per SM)
     // for graphs from 2^13 vertices and edges on (for all while every graph
