@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     rounds_kept();
   } else {
     // The threshold: about the key of the wanted rank in a sample of warp 0,
-    // found bit by bit with ballots -- twelve bits below the samples' common
-    // prefix; any threshold is a valid one.
+    // found bit by bit with ballots -- as a rule twelve bits below the samples'
+    // common prefix; any threshold is a valid one.
     const bool filter = !A.count && (double)m > 1.5 * LIGHT * (double)n;
     if (wid == 0 && filter) {
       constexpr int PER = 8;
@@ -344,9 +344,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
       };
       const int high = 31 - __clz((int)((lo ^ up) | 1u));  // the highest bit in which samples differ
       uint32_t tw = high >= 31 ? 0u : lo >> (high + 1) << (high + 1), te = NONE;
-      for (int b = high; b >= 0 && b > high - 12; --b) {
-        const uint32_t c = tw | (1u << b);
-        if (below_key(c, 0u) <= rank) tw = c;
+      auto refine = [&](int from, int to) {
+        for (int b = from; b >= 0 && b > to; --b) {
+          const uint32_t c = tw | (1u << b);
+          if (below_key(c, 0u) <= rank) tw = c;
+        }
+      };
+      refine(high, high - 12);
+      if (high >= 12) {
+        // all weights with these bits, unless many samples share them (a few
+        // weights of which the others are exact multiples, negative ones): by the
+        // other bits too.  None of them, where -1 and 1 are the only weights, left
+        // no edge light (40 graphs of 4000 vertices and 400 000 edges 2.6 ms, now 0.36)
+        const uint32_t up = tw | ((2u << (high - 12)) - 1u);
+        if (below_key(up, NONE) <= rank + rank / 4 + 1) tw = up;
+        else refine(high - 12, -1);
       }
       if (below_key(tw, NONE) > rank + rank / 4 + 1) {  // many ties: by edge index
         te = 0;
