@@ -297,8 +297,10 @@ int enqueue_msf_graph(const DevState &hs, cudaStream_t s, const DevState **host_
   Executor *ex = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_exec_mu);
+    // every option that decides what is captured, each with a place of its own
+    // (three sweep forms: the pairwise kernel's number is none of theirs)
     auto key = std::make_tuple(dev, (uintptr_t)s, o.spl, o.blocks_per_sm * 2 + o.prefetch, o.shortcut_mode,
-                               o.pairwise * 2 + o.sweep);
+                               o.pairwise * 3 + o.sweep);
     auto it = g_execs.find(key);
     if (it != g_execs.end()) {
       ex = it->second;
