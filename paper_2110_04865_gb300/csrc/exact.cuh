@@ -275,13 +275,15 @@ __device__ inline double combine_bins_warp(const long long *b, int wtype) {
 // low unless that makes 32 a vertex.  Mean of 8 to 24 seeds in us, without / with:
 // 40 graphs of 2000 vertices and 2^19 edges 2258 / 443, 152 of 1000 and 60 000 278 /
 // 133, 100 of 2000 and 10^5 399 / 165; one of 10^5 and 16 M 396 / 307.
+// (In float: a block's warp 0 waits for it, and double operations were 2 us of the
+// 95 of 4096 vertices and 32 768 edges.)
 __host__ __device__ inline int light_rank(double light, int64_t n, int64_t m, int samples, int low) {
-  const double per = (double)n / (double)m * samples;  // samples to an edge a vertex
-  double least = 32.0 * per < low ? 32.0 * per : low;
-  if (least < 2.0) least = 2.0;
-  double want = 3.0 * per < 2.0 * low ? 3.0 * per : 2.0 * low;
+  const float per = (float)n / (float)m * (float)samples;  // samples to an edge a vertex
+  float least = 32.f * per < (float)low ? 32.f * per : (float)low;
+  if (least < 2.f) least = 2.f;
+  float want = 3.f * per < 2.f * (float)low ? 3.f * per : 2.f * (float)low;
   if (want < least) want = least;
-  const double rank = light * per;
+  const float rank = (float)light * per;
   return (int)(rank > want ? rank : want);
 }
 

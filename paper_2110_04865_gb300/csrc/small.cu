@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small(SmallArgs A) {
     // The threshold: about the key of the wanted rank in a sample of warp 0,
     // found bit by bit with ballots -- as a rule twelve bits below the samples'
     // common prefix; any threshold is a valid one.
-    const bool filter = !A.count && (double)m > 1.5 * LIGHT * (double)n;
+    const bool filter = !A.count && (float)m > (float)(1.5 * LIGHT) * (float)n;
     if (wid == 0 && filter) {
       constexpr int PER = 8;
       uint32_t w[PER], e[PER], lo = NONE, up = 0u;
