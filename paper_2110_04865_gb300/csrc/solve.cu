@@ -32,12 +32,12 @@
 // phases meet at a grid barrier (1 to 2 us, bounded wait), which costs less
 // than the kernel boundaries and conditional nodes of a graph loop (about 60
 // launches in the CSR path's small calls).  What bounds the steps: select and
-// filter the instruction issue and DRAM (R-MAT 20: 45 and 52 us for 201 and
-// 150 MB), the minimum passes L1 wavefronts (two parents and two minima
+// filter the instruction issue and DRAM (R-MAT 20: 43 and 58 us for 201 MB
+// each, from pairs of ends 42 and 52), the minimum passes L1 wavefronts (two parents and two minima
 // gathered per edge), late rounds the barriers.
 //
 // Measured on the whole call (build and round loop over the CSR before, this
-// after): R-MAT 26 112 -> 21.9 ms, the 256^3 grid 9.9 -> 2.27 ms, R-MAT 20 1.75
+// after): R-MAT 26 112 -> 21.9 ms, the 256^3 grid 9.9 -> 2.31 ms, R-MAT 20 1.75
 // -> 0.455 ms, uniform n = 10^6, m = 16 n 2.6 -> 0.51 ms, R-MAT 16 0.47 -> 0.174
 // ms, 4096 graphs of 38 M vertices 26.3 -> 5.84 ms.  Fractions around these when
 // they were chosen (CLASS1 0.25 to 1, CLASS2 1.2 to 3): R-MAT 26 20.7 to 22.9 ms,
